@@ -207,8 +207,10 @@ CompositeArgs composite_args(const Layout& L, void* ws, int feat_bf16, const voi
 }
 
 // ---------------------------------------------------------------------------
-// Batched views: a 256-byte batch header (the two work-item counters of the
-// persistent compositing launches), then one single-view workspace per view.
+// Batched views: a 256-byte batch header (the work-item counters of the
+// persistent compositing launches: one per channel part, the forward's from
+// word 0, the reverse's four from word kRevQueue), then one single-view
+// workspace per view.
 // ---------------------------------------------------------------------------
 static_assert(FE_MAX_VIEWS == kMaxViews, "view limit of the ABI and the kernels");
 
@@ -217,6 +219,7 @@ static_assert(FE_MAX_VIEWS == kMaxViews, "view limit of the ABI and the kernels"
 // stream, views dealt round-robin; the reverse's gradient sums of each
 // helper stream go to a buffer of its own in the workspace.
 constexpr int kBatchStreams = 4;
+constexpr int kRevQueue = 4;
 constexpr int kGradArrays = 6;  // means, log_scales, quats, opacity logits, sh, feat
 
 struct BatchLayout {
@@ -633,8 +636,8 @@ fe_status fe_render_batch_backward(const fe_gaussians* g, const fe_deform* defor
   std::unique_ptr<BatchCompositeArgs> ba(new (std::nothrow) BatchCompositeArgs());
   std::unique_ptr<CompositeArgs[]> cv(new (std::nothrow) CompositeArgs[kMaxViews]);
   if (!ba || !cv) return FE_ERR_WORKSPACE;
-  FE_TRY_CUDA(cudaMemsetAsync(static_cast<uint32_t*>(workspace) + 1, 0, 4, st));      // reverse counters
-  FE_TRY_CUDA(cudaMemsetAsync(static_cast<uint32_t*>(workspace) + 3, 0, 4, st));      // (second channel half)
+  // The reverse's work counters, one per channel part.
+  FE_TRY_CUDA(cudaMemsetAsync(static_cast<uint32_t*>(workspace) + kRevQueue, 0, 16, st));
   for (int v = 0; v < b->V; ++v) {
     const Layout& L = BL->L[v];
     void* ws = static_cast<char*>(workspace) + BL->off[v];
@@ -646,7 +649,7 @@ fe_status fe_render_batch_backward(const fe_gaussians* g, const fe_deform* defor
     c.g_feat = grad_out[v].feat;
     cv[v] = c;
   }
-  batch_items(*BL, cv.get(), workspace, 1, *ba);
+  batch_items(*BL, cv.get(), workspace, kRevQueue, *ba);
   FE_TRY_CUDA(mark(o0, 4, st));
   FE_TRY_CUDA(launch_composite_bwd_batch(*ba, g->D, g->feat_bf16, st));
   FE_TRY_CUDA(mark(o0, 5, st));

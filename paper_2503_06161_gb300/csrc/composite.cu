@@ -9,10 +9,11 @@
 //
 // Reverse: the same block walks the list backwards from the largest
 // n_contrib of the tile, replaying T_i = T_{i+1} / (1 - alpha_i) from
-// T_final (no per-pixel lists are stored).  Per batch, the per-(pixel,
-// Gaussian) terms go to shared memory and are summed over the tile's pixels
-// in a fixed order, one partial row per (tile, Gaussian) entry: no
-// floating-point atomics, bitwise deterministic.
+// T_final (no per-pixel lists are stored).  Per batch, the terms of each
+// warp's (pixel, Gaussian) pairs are summed over its pixels by tensor-core
+// products and then over the tile's warps in a fixed order, one partial row
+// per (tile, Gaussian) entry: no floating-point atomics, bitwise
+// deterministic.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -384,67 +385,139 @@ __global__ void __launch_bounds__(kThreads, D <= 32 ? 3 : (D <= 64 ? 2 : 1))
 }
 
 // ---------------------------------------------------------------------------
-// Reverse pass.  Per batch of B list entries (walked backwards), each pixel
-// thread replays its recurrence and forms, per (pixel, entry): the blend
-// weight w and six geometric terms (du, dv, dA, dB, dCc, dopacity).  Then:
-//  * geometric terms: a shuffle reduce-scatter over the warp's 32 pixels,
-//    only for entries where some lane of the warp contributed;
-//  * linear terms sum_p w_p G_p with G_p = (g_rgb, g_depth, g_feat): a
-//    register-blocked (entries x channels) product over the warp's pixels;
-//  * a fixed-order sum of the 8 warp partials per entry.
+// Reverse pass.  Per batch of 32 list entries (walked backwards), each warp
+// takes the entries some pixel of its 8 x 4 block blended (the forward's
+// masks), up to 16 at a time (a chunk), and forms three matrix products over
+// them on the tensor cores (mma.sync, warp-local: no block barrier and no
+// operand shared between warps but the staged entries):
+//   S[entry][pixel]  = feature . feature gradient      (K = D channels)
+//   P[entry][channel] = sum over pixels of w G           (K = 32 pixels)
+//   M[entry][6]       = sum over pixels of e (1 x y xx xy yy)
+// with w the blend weight, G the pixel's upstream gradient and e =
+// dL/dalpha alpha.  Between S and the other two, each lane replays its
+// pixel's recurrence over the chunk's entries (T_i = T_{i+1} / (1 - alpha_i)).
+// The geometric sums of an entry (du .. dopacity) follow from its six
+// moments M, taken about the centre of the warp's block, where the
+// pixel coordinates and their products are exact in BF16.
+//
+// Every FP32 operand is carried as three BF16 terms x = hi + mid + lo (24
+// significant bits) and a product as the six term products down to 2^-16 of
+// |x||y|, smallest first, accumulated in FP32; a BF16-stored feature and the
+// moments' coordinates are exact in one term (three products).
+//
+// The pass is bound by instruction issue and the latency of the few warps
+// that its shared memory leaves room for.  With FP32 FMAs for the products
+// and shuffles for the geometric sums an entry cost a warp 256 instructions
+// at D = 32 (75 the product with G, 46 the geometric terms, 30 the feature
+// dot), now about 180; at D = 128 the gradient rows had to be re-read from
+// shared memory for every entry.  Measured, before and now: 200k Gaussians at
+// 640 x 512, D = 32: 365 -> 330 us; 90k, D = 128: 1520 -> 1345 us; 1M at
+// 1280 x 1024, D = 64 BF16: 2135 -> 1811 us; eight views of 100k, D = 32
+// BF16, in one launch: 1960 -> 1528 us.  (tcgen05 products over the whole
+// tile were costed: they take every entry of a batch for every pixel where a
+// warp needs half of them, and their operands in three terms leave one block
+// per SM at D = 32 too.)
 template <int D>
 struct BwdCfg {
-  static constexpr int NC = 4 + D;                  // linear channels
-  static constexpr int B = D <= 64 ? 32 : 16;       // entries per batch
-  static constexpr int JG = 16, CG = 2;             // lane grid of the per-warp product
-  static constexpr int JPL = B / JG;                // entries per lane
-  static constexpr int CPL = NC / CG;               // channels per lane (even: packed FMA)
-  static constexpr bool GREG = D <= 64;             // upstream gradients kept in registers
-  static constexpr int GS = NC + 2;                 // per-pixel gradient row stride (8-byte rows)
-  static constexpr int WS = B + 2;                  // w row stride (8-byte rows; 2-way bank conflicts on the w writes)
-  static constexpr int SLICE = (32 * WS > B * NC) ? 32 * WS : B * NC;
-  // Scalar row of a warp's entry: du dv dA dB dCc dopacity | r g b | depth | 0 0
-  // (the layout of the partial row's scalar columns); B + 1 rows per warp,
-  // the last one a sink for the sums of no entry.
-  static constexpr int GR = 12;
-  static_assert(B % JG == 0 && CPL % 2 == 0 && JPL <= 2, "lane grid of the per-warp product");
-  // Byte offsets in dynamic shared memory: per-pixel gradient rows, warp
-  // slices, geometric warp partials, two staging buffers, the fp32 copy of
-  // bf16 feature rows, list entries of the two staged batches.
+  static_assert(D == 16 || D == 32 || D == 64, "channels of one reverse pass");
+  static constexpr int B = 32;          // entries per batch
+  static constexpr int CH = 16;         // entries per chunk (MMA rows)
+  static constexpr int KS = D / 16;     // K steps of S
+  static constexpr int NT = D / 8;      // channel tiles of P (one more for colour and depth)
+  static constexpr int SS = 36;         // row stride of the [entry][pixel] slices (floats)
+  static constexpr int PR = D + 12;     // a warp's partial row: features | du dv dA dB dCc dopacity r g b depth 0 0
+  // A warp's area (floats): its partial rows of the batch from the start,
+  // and the two slices of the chunk in flight (S, overwritten by w; e) at
+  // the end, which end up under the chunk's own rows.  A later chunk of the
+  // batch takes at most as many entries as the place behind the rows so far
+  // has slices for: 16 at D = 16 and 64; at D = 32, where two blocks per SM
+  // leave less, 26 entries are two chunks and 32 are four (of the synthetic
+  // scenes' warps and batches under 5% have more than 26).
+  static constexpr int AREA = D == 16 ? CH * PR + 2 * CH * SS : D == 32 ? 1472 : B * PR;
+  static_assert(AREA >= B * PR && AREA >= 2 * CH * SS && AREA % 4 == 0, "partial rows and slices of a warp");
+  // Upstream gradients of a warp's pixels, per term [channel][32 pixels]
+  // BF16 (64-byte rows, 16-byte chunk t of row c at t ^ ((c >> 2) & 3): the
+  // fragment loads below touch every bank once).
+  static constexpr int GTERM = (D + 4) * 64;
+  static constexpr int GWARP = 3 * GTERM;
   static constexpr size_t off_G = 0;
-  static constexpr size_t off_slice = off_G + (size_t)kThreads * GS * 4;
-  static constexpr size_t off_geo = off_slice + (size_t)8 * SLICE * 4;
-  static constexpr size_t off_stage = (off_geo + (size_t)8 * (B + 1) * GR * 4 + 127) / 128 * 128;
-  __host__ __device__ static constexpr size_t off_wide(int bf16) { return off_stage + 2 * (size_t)stage_bytes(B, D, bf16); }
-  __host__ __device__ static constexpr size_t off_e(int bf16) {
-    return off_wide(bf16) + (bf16 ? (size_t)B * D * 4 : 0);
-  }
-  __host__ __device__ static constexpr size_t smem_bytes(int bf16) { return off_e(bf16) + (size_t)(2 * B + 8 + 4) * 4; }
+  static constexpr size_t off_area = off_G + (size_t)8 * GWARP;
+  static constexpr size_t off_stage = (off_area + (size_t)8 * AREA * 4 + 127) / 128 * 128;
+  __host__ __device__ static constexpr size_t off_e(int bf16) { return off_stage + 2 * (size_t)stage_bytes(B, D, bf16); }
+  // List entries of the two staged batches, the warps' entry masks, the
+  // warps' entry lists.
+  __host__ __device__ static constexpr size_t smem_bytes(int bf16) { return off_e(bf16) + (size_t)(2 * B + 8 + 8 * B) * 4; }
 };
 
-static_assert(BwdCfg<16>::smem_bytes(1) <= 232448 && BwdCfg<32>::smem_bytes(1) <= 232448 &&
-                  BwdCfg<64>::smem_bytes(1) <= 232448 && BwdCfg<128>::smem_bytes(1) <= 232448 &&
-                  BwdCfg<128>::smem_bytes(0) <= 232448,
-              "reverse compositing shared memory per block");
-static_assert(2 * (BwdCfg<32>::smem_bytes(1) + 1024) <= 233472, "two reverse blocks per SM at D <= 32");
+static_assert(BwdCfg<64>::smem_bytes(0) <= 232448, "reverse compositing shared memory per block");
+static_assert(2 * (BwdCfg<32>::smem_bytes(0) + 128 + 1024) <= 233472, "two reverse blocks per SM at D <= 32");
+
+// 1 / x by the hardware approximation (about 1 ulp).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float x, float y) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// Three-term BF16 split of a pair (low half = first value).
+__device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  hi = pack_bf16(x, y);
+  x -= __uint_as_float(hi << 16);
+  y -= __uint_as_float(hi & 0xFFFF0000u);
+  mid = pack_bf16(x, y);
+  x -= __uint_as_float(mid << 16);
+  y -= __uint_as_float(mid & 0xFFFF0000u);
+  lo = pack_bf16(x, y);
+}
+
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// The same with a zero accumulator in.
+__device__ __forceinline__ void mma_bf16_16816_first(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+}
+
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&v)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr));
+}
+
+// Terms (of the first operand, of the second) of the six products, smallest first.
+__device__ constexpr int kTermA[6] = {2, 1, 0, 1, 0, 0};
+__device__ constexpr int kTermB[6] = {0, 1, 2, 0, 1, 0};
+
+// Byte offset of 16-byte chunk t (pixels 8 t .. 8 t + 7) of row c of a term.
+__device__ __forceinline__ uint32_t g_chunk(int c, int t) { return (uint32_t)(c * 64 + ((t ^ ((c >> 2) & 3)) << 4)); }
 
 // Reverse compositing of one tile by the whole block.
 template <int D>
 __device__ __forceinline__ void bwd_tile(const CompositeArgs& a, const int tile, unsigned char* smem, uint64_t* s_bar,
                                          int* s_abort, StageState& stg) {
   using K = BwdCfg<D>;
-  constexpr int B = K::B, NC = K::NC, GS = K::GS, WS = K::WS;
+  constexpr int B = K::B, CH = K::CH, SS = K::SS, PR = K::PR, KS = K::KS, NT = K::NT;
   const bool bf16 = a.feat_bf16 != 0;
   const uint32_t sbytes = stage_bytes(B, D, a.feat_bf16);
-  float* s_G = reinterpret_cast<float*>(smem + K::off_G);          // [256][GS]
-  float* s_slice = reinterpret_cast<float*>(smem + K::off_slice);  // [8][SLICE]: w[p][j], then P[j][c]
-  float* s_geo = reinterpret_cast<float*>(smem + K::off_geo);      // [8][B + 1][GR]
-  unsigned char* s_stage = smem + K::off_stage;                     // [2][sbytes]
-  float* s_wide = reinterpret_cast<float*>(smem + K::off_wide(a.feat_bf16));
+  float* s_area = reinterpret_cast<float*>(smem + K::off_area);  // [8][AREA]
+  unsigned char* s_stage = smem + K::off_stage;                   // [2][sbytes]
   uint32_t* s_e = reinterpret_cast<uint32_t*>(smem + K::off_e(a.feat_bf16));  // [2][B]
   uint32_t* s_jact = s_e + 2 * B;
-  uint32_t* s_maxn = s_jact + 8;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t* s_list = s_jact + 8 + warp * B;  // this warp's entries of the batch, latest first
+  unsigned char* s_G = smem + K::off_G + warp * K::GWARP;
+  float* area = s_area + warp * K::AREA;
   const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
   int lx, ly;
   tile_pixel(tid, a.tw, lx, ly);
@@ -453,58 +526,35 @@ __device__ __forceinline__ void bwd_tile(const CompositeArgs& a, const int tile,
   const float pxc = (float)px + 0.5f, pyc = (float)py + 0.5f;
   const size_t HW = (size_t)a.W * a.H, pix = inside ? (size_t)py * a.W + px : 0;
   const uint2 rg = a.ranges[tile];
-  float* grow = s_G + tid * GS;
-  float ga = 0.f;
-  {
-    float g0 = 0.f, g1 = 0.f, g2 = 0.f, gz = 0.f;
-    if (inside) {
-      if (a.g_rgb) { g0 = a.g_rgb[pix]; g1 = a.g_rgb[HW + pix]; g2 = a.g_rgb[2 * HW + pix]; }
-      if (a.g_depth) gz = a.g_depth[pix];
-      if (a.g_alpha) ga = a.g_alpha[pix];
-    }
-    grow[0] = g0; grow[1] = g1; grow[2] = g2; grow[3] = gz;
-    if (inside && a.g_feat) {
-      const float4* src = reinterpret_cast<const float4*>(a.g_feat + pix * a.out_ld);
-#pragma unroll
-      for (int d4 = 0; d4 < D / 4; ++d4) {
-        const float4 v = __ldg(src + d4);
-        grow[4 + 4 * d4] = v.x; grow[5 + 4 * d4] = v.y; grow[6 + 4 * d4] = v.z; grow[7 + 4 * d4] = v.w;
-      }
-    } else {
-#pragma unroll
-      for (int d = 0; d < D; ++d) grow[4 + d] = 0.0f;
-    }
-  }
-  for (int i = tid; i < 8 * (B + 1); i += kThreads) {
-    s_geo[i * K::GR + 10] = 0.0f;
-    s_geo[i * K::GR + 11] = 0.0f;
-  }
-  float2 G[K::GREG ? NC / 2 : 1];
-  if (K::GREG) {
-#pragma unroll
-    for (int c = 0; c < NC / 2; ++c) G[c] = make_float2(grow[2 * c], grow[2 * c + 1]);
-  }
   const float Tf = inside ? a.t_final[pix] : 1.0f;
   const uint32_t nc = inside ? a.n_contrib[pix] : 0u;
-  float T = Tf;
-  float Q = (grow[0] * a.bg[0] + grow[1] * a.bg[1] + grow[2] * a.bg[2]) * Tf;
+  // Upstream gradients of this pixel: every load is issued before the first
+  // is used, and the first batches are on their way before the split below.
+  float g0 = 0.f, g1 = 0.f, g2 = 0.f, gz = 0.f, ga = 0.f;
+  if (inside) {
+    if (a.g_rgb) { g0 = a.g_rgb[pix]; g1 = a.g_rgb[HW + pix]; g2 = a.g_rgb[2 * HW + pix]; }
+    if (a.g_depth) gz = a.g_depth[pix];
+    if (a.g_alpha) ga = a.g_alpha[pix];
+  }
+  float4 gf[D / 4];
+  {
+    const bool has = inside && a.g_feat != nullptr;
+    const float4* src = reinterpret_cast<const float4*>(a.g_feat + (has ? pix * a.out_ld : 0));
+#pragma unroll
+    for (int d4 = 0; d4 < D / 4; ++d4) gf[d4] = has ? __ldg(src + d4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, nc);
-  if (tid == 0) *s_maxn = 0u;
+  if (lane == 0) s_jact[warp] = wmax;
   __syncthreads();
-  if (lane == 0 && wmax) atomicMax(s_maxn, wmax);
-  __syncthreads();
-  // Batches walk [rg.x, rg.x + maxn) backwards: batch k covers
-  // [max(rg.x, hi_k - B), hi_k) with hi_k = rg.x + maxn - k B.
-  const uint32_t n = *s_maxn;
+  // Batches aligned to multiples of B from the tile start, walked backwards
+  // from the largest n_contrib (the first one processed, the last in list
+  // order, may be short).
+  uint32_t n = 0;
+#pragma unroll
+  for (int w8 = 0; w8 < 8; ++w8) n = max(n, s_jact[w8]);
   const uint32_t nbatch = (n + B - 1) / B;
-  // Batches aligned to multiples of B from the tile start (the first one
-  // processed, the last in list order, may be short).
   auto batch_lo = [&](uint32_t k) -> uint32_t { return (nbatch - 1 - k) * (uint32_t)B; };
   auto batch_len = [&](uint32_t k) -> int { return (int)min((uint32_t)B, n - batch_lo(k)); };
-  // The forward's masks say which entries of each 32-entry group blended in
-  // some pixel of this warp; the others are skipped (a 16-entry batch takes
-  // its half of the group's word).
-  const bool masked = a.cmask != nullptr;
   const size_t cslot0 = (size_t)(rg.x >> 5) + (size_t)tile;
   // List entry and Gaussian of this thread's slot in batch k.
   auto slot = [&](uint32_t k, uint32_t& e, uint32_t& g) {
@@ -517,12 +567,11 @@ __device__ __forceinline__ void bwd_tile(const CompositeArgs& a, const int tile,
       g = eg.y;
     }
   };
-  // The forward's blend-mask word of this warp for batch k (read a batch
-  // ahead, so its global latency overlaps the previous batch).
+  // The forward's blend mask of this warp for batch k: the entries some
+  // pixel of its block blended (read a batch ahead, so its global latency
+  // overlaps the previous batch).
   auto mask_word = [&](uint32_t k) -> uint32_t {
-    return (masked && k < nbatch && batch_lo(k) < wmax)
-               ? __ldg(a.cmask + (cslot0 + batch_lo(k) / 32) * 8 + warp) >> (batch_lo(k) & 31u)
-               : 0xFFFFFFFFu;
+    return (k < nbatch && batch_lo(k) < wmax) ? __ldg(a.cmask + (cslot0 + batch_lo(k) / 32) * 8 + warp) : 0u;
   };
   uint32_t mask_next = mask_word(0);
   uint32_t e_next, g_next;
@@ -534,7 +583,52 @@ __device__ __forceinline__ void bwd_tile(const CompositeArgs& a, const int tile,
     issued = 1;
   }
   slot(1, e_next, g_next);
-  float* slice = s_slice + warp * K::SLICE;
+  // The gradients as the warp's operand rows (features, then r g b depth).
+  auto put_pair = [&](int c, float x, float y) {  // rows c and c + 1, this lane's pixel
+    uint32_t t3[3];
+    split3(x, y, t3[0], t3[1], t3[2]);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      unsigned char* p = s_G + t * K::GTERM + 2 * (lane & 7);
+      *reinterpret_cast<uint16_t*>(p + g_chunk(c, lane >> 3)) = (uint16_t)(t3[t] & 0xFFFFu);
+      *reinterpret_cast<uint16_t*>(p + g_chunk(c + 1, lane >> 3)) = (uint16_t)(t3[t] >> 16);
+    }
+  };
+#pragma unroll
+  for (int d4 = 0; d4 < D / 4; ++d4) {
+    put_pair(4 * d4, gf[d4].x, gf[d4].y);
+    put_pair(4 * d4 + 2, gf[d4].z, gf[d4].w);
+  }
+  put_pair(D, g0, g1);
+  put_pair(D + 2, g2, gz);
+  __syncwarp();
+  float T = Tf;
+  float Q = (g0 * a.bg[0] + g1 * a.bg[1] + g2 * a.bg[2]) * Tf;
+  const float gaTf = ga * Tf;
+  // Fragment coordinates of this lane: rows fr and fr + 8, columns 2 ft and
+  // 2 ft + 1 of an accumulator.
+  const int fr = lane >> 2, ft = lane & 3;
+  // S: the second operand G[channel][pixel], read transposed.  K index
+  // 2 t + e (+ 8 h) of a step is channel 4 t + 2 h + e, so that a lane's four
+  // first-operand values of a row are one 16-byte load.
+  const uint32_t g_addr = smem_addr(s_G);
+  const int lm_c = 4 * ((lane & 7) >> 1) + 2 * ((lane >> 3) & 1) + (lane & 1), lm_t = lane >> 4;
+  // Moments: the second operand, moment fr of pixels 8 ft + i (row ft of the
+  // block, column i), about the block's centre.  K index 2 t + e (+ 8 h) of
+  // step s is pixel 8 t + 4 s + 2 h + e, for P and M alike.
+  uint32_t mom[4];
+  {
+    const float y = (float)ft - 1.5f;
+    auto moment = [&](int i) -> float {
+      const float x = (float)i - 3.5f;
+      return fr == 0 ? 1.0f : fr == 1 ? x : fr == 2 ? y : fr == 3 ? x * x : fr == 4 ? x * y : fr == 5 ? y * y : 0.0f;
+    };
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mom[i] = pack_bf16(moment(2 * i), moment(2 * i + 1));
+  }
+  // Centre of this warp's block.
+  const float cxw = (float)(tx * a.tw + ((warp % (a.tw >> 3)) << 3)) + 4.0f;
+  const float cyw = (float)(ty * a.th + ((warp / (a.tw >> 3)) << 2)) + 2.0f;
   for (uint32_t k = 0; k < nbatch; ++k) {
     // Every thread is past batch k-1 (and its combine) here.  A wait on
     // batch k-1 that gave up ends the tile for the whole block (the flag
@@ -555,253 +649,223 @@ __device__ __forceinline__ void bwd_tile(const CompositeArgs& a, const int tile,
     }
     const unsigned char* buf = s_stage + (k & 1) * (size_t)sbytes;
     const float* s_rec = reinterpret_cast<const float*>(buf);
-    const float* s_feat = reinterpret_cast<const float*>(buf + (size_t)B * kRec * 4);
+    const unsigned char* s_feat = buf + (size_t)B * kRec * 4;  // rows as stored (fp32 or bf16)
     const int nb = batch_len(k);
-    if (bf16) {
-      if (live) widen_bf16<D>(buf + (size_t)B * kRec * 4, s_wide, nb);
-      __syncthreads();
-      s_feat = s_wide;
-    }
     const uint32_t rel0 = batch_lo(k);
-    const uint32_t mask_k = mask_next;
+    const uint32_t jact = mask_next & (nb >= 32 ? 0xFFFFFFFFu : ((1u << nb) - 1u));
     mask_next = mask_word(k + 1);
-    uint32_t jact = 0;
-    if (rel0 < wmax) {
-      const uint32_t lenmask = nb >= 32 ? 0xFFFFFFFFu : ((1u << nb) - 1u);
-      uint32_t todo = mask_k & lenmask;
-      // Every lane writes w (0 where it did not blend) for every entry the
-      // warp visits; rows of entries it does not visit may hold stale values:
-      // the products of those columns are never combined.
-      // Entry j given its evaluation (hit: the pixel includes it): the T
-      // replay and the gradient terms v (six geometric values, then two
-      // zeros), and the blend weight written to the warp's w slice.
-      auto entry = [&](int j, bool hit, const PairEval& pe, float (&v)[8]) {
-        // Without branches, so that the two entries of a pair interleave:
-        // a lane that did not blend takes alpha = 0, which leaves T and Q
-        // exactly as they were (1 / (1 - 0) = 1, w = 0), and zero terms.
-        const float* rec = s_rec + j * kRec;
-        const float al = hit ? pe.alpha : 0.0f;
-        const float one_m = 1.0f - al;
-        const float inv = __fdividef(1.0f, one_m);  // one_m >= 0.01
-        T = T * inv;  // transmittance before this Gaussian
-        const float w = al * T;
-        // s = g . (rgb, depth, feature) of this Gaussian, in four
-        // independent chains of channel pairs (pair i in chain i mod 4).
-        const float4 r0 = *reinterpret_cast<const float4*>(rec);      // ., ., A, B
-        const float4 r4 = *reinterpret_cast<const float4*>(rec + 4);  // Cc, ., depth, r
-        const float4 r8 = *reinterpret_cast<const float4*>(rec + 8);  // g, b, ., .
-        const float4* f4 = reinterpret_cast<const float4*>(s_feat + j * D);
-        const float2* g2 = reinterpret_cast<const float2*>(grow);
-        float2 sc[4];
-        sc[0] = __fmul2_rn(K::GREG ? G[0] : g2[0], make_float2(r4.w, r8.x));
-        sc[1] = __fmul2_rn(K::GREG ? G[1] : g2[1], make_float2(r8.y, r4.z));
-        sc[2] = make_float2(0.0f, 0.0f);
-        sc[3] = make_float2(0.0f, 0.0f);
+    const int cnt = __popc(jact);
+    if (cnt > 0) {
+      // Entry list, latest first: slot = number of later entries.
+      if ((jact >> lane) & 1u) s_list[__popc((jact >> lane) >> 1)] = (uint32_t)lane;
+      __syncwarp();
+    }
+    uint32_t todo = jact;
+    for (int c0 = 0, m; c0 < cnt; c0 += m) {
+      m = min(min(CH, cnt - c0), (K::AREA - c0 * PR) / (2 * SS));  // entries of this chunk
+      float* sl_w = area + (K::AREA - 2 * SS * m);  // [m][SS]: S, then w
+      float* sl_e = sl_w + SS * m;                  // [m][SS]: e
+      // ---- S[entry][pixel] ----
+      {
+        // First operand: the feature rows of entries fr and fr + 8 (slots past
+        // the chunk repeat its last entry; their results are not used).
+        const int ra = (int)s_list[c0 + min(fr, m - 1)], rb = (int)s_list[c0 + min(fr + 8, m - 1)];
+        uint32_t xa[3][KS][4];
+        if (bf16) {
 #pragma unroll
-        for (int d4 = 0; d4 < D / 4; ++d4) {
-          const float4 xv = f4[d4];
-          const int c0 = 2 + 2 * d4;  // channel pair of xv.x, xv.y
-          sc[c0 & 3] = __ffma2_rn(K::GREG ? G[c0] : g2[c0], make_float2(xv.x, xv.y), sc[c0 & 3]);
-          sc[(c0 + 1) & 3] = __ffma2_rn(K::GREG ? G[c0 + 1] : g2[c0 + 1], make_float2(xv.z, xv.w), sc[(c0 + 1) & 3]);
+          for (int ks = 0; ks < KS; ++ks) {
+            const uint2 va = *reinterpret_cast<const uint2*>(s_feat + ra * (2 * D) + 32 * ks + 8 * ft);
+            const uint2 vb = *reinterpret_cast<const uint2*>(s_feat + rb * (2 * D) + 32 * ks + 8 * ft);
+            xa[0][ks][0] = va.x; xa[0][ks][2] = va.y; xa[0][ks][1] = vb.x; xa[0][ks][3] = vb.y;
+          }
+        } else {
+#pragma unroll
+          for (int ks = 0; ks < KS; ++ks) {
+            const float4 va = *reinterpret_cast<const float4*>(s_feat + ra * (4 * D) + 64 * ks + 16 * ft);
+            const float4 vb = *reinterpret_cast<const float4*>(s_feat + rb * (4 * D) + 64 * ks + 16 * ft);
+            split3(va.x, va.y, xa[0][ks][0], xa[1][ks][0], xa[2][ks][0]);
+            split3(va.z, va.w, xa[0][ks][2], xa[1][ks][2], xa[2][ks][2]);
+            split3(vb.x, vb.y, xa[0][ks][1], xa[1][ks][1], xa[2][ks][1]);
+            split3(vb.z, vb.w, xa[0][ks][3], xa[1][ks][3], xa[2][ks][3]);
+          }
         }
-        const float2 s01 = __fadd2_rn(sc[0], sc[1]), s23 = __fadd2_rn(sc[2], sc[3]);
-        const float2 s2 = __fadd2_rn(s01, s23);
-        const float s = s2.x + s2.y;
-        const float dalpha = T * s - (Q - ga * Tf) * inv;
-        Q = fmaf(w, s, Q);
-        // Geometric terms: zero where the pixel did not blend, and all but
-        // the opacity term zero where alpha was clamped.
-        const bool geo = hit && !pe.clamped;
-        const float dp2 = geo ? dalpha * pe.alpha * kLn2 : 0.0f;
-        v[0] = -dp2 * (2.0f * r0.z * pe.dx + r0.w * pe.dy);
-        v[1] = -dp2 * (2.0f * r4.x * pe.dy + r0.w * pe.dx);
-        v[2] = dp2 * pe.dx * pe.dx;
-        v[3] = dp2 * pe.dx * pe.dy;
-        v[4] = dp2 * pe.dy * pe.dy;
-        v[5] = hit ? dalpha * pe.G : 0.0f;
-        v[6] = 0.0f;
-        v[7] = 0.0f;
-        slice[lane * WS + j] = w;
-      };
-      const int b16 = (lane >> 4) & 1, b8 = (lane >> 3) & 1, b4 = (lane >> 2) & 1, b2 = (lane >> 1) & 1;
-      // Warp sums of one entry's v[0..7] (reduce-scatter: lane 4m ends with
-      // the sum of index m).
-      auto scatter1 = [&](int j, float (&v)[8]) {
+        // The four pixel tiles' chains run side by side.
+        float sa[4][4];
+        auto step = [&](int tx, int tg, int ks, bool first) {
+          uint32_t v[2][4];
+          ldmatrix_x4_trans(g_addr + tg * K::GTERM + g_chunk(16 * ks + lm_c, lm_t), v[0]);
+          ldmatrix_x4_trans(g_addr + tg * K::GTERM + g_chunk(16 * ks + lm_c, 2 + lm_t), v[1]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float send = b16 ? v[i] : v[i + 4];
-          const float keep = b16 ? v[i + 4] : v[i];
-          v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 16);
+          for (int pt = 0; pt < 4; ++pt) {
+            const uint32_t b0 = v[pt >> 1][2 * (pt & 1)], b1 = v[pt >> 1][2 * (pt & 1) + 1];
+            if (first) mma_bf16_16816_first(sa[pt], xa[tx][ks], b0, b1);
+            else mma_bf16_16816(sa[pt], xa[tx][ks], b0, b1);
+          }
+        };
+        if (bf16) {
+#pragma unroll
+          for (int t = 2; t >= 0; --t)
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) step(0, t, ks, t == 2 && ks == 0);
+        } else {
+#pragma unroll
+          for (int p = 0; p < 6; ++p)
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) step(kTermA[p], kTermB[p], ks, p == 0 && ks == 0);
         }
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const float send = b8 ? v[i] : v[i + 2];
-          const float keep = b8 ? v[i + 2] : v[i];
-          v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 8);
-        }
-        {
-          const float send = b4 ? v[0] : v[1];
-          const float keep = b4 ? v[1] : v[0];
-          v[0] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 4);
-        }
-        v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 2);
-        v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], 1);
-        const int m = lane >> 2;
-        if ((lane & 3) == 0 && m < 6) s_geo[(warp * (B + 1) + j) * K::GR + m] = v[0];
-      };
-      // Both entries' sums at once: u = (va, vb), lane 2m ends with the sum
-      // of index m (16 shuffles instead of 18, and no warp-wide exchange
-      // between the two entries' arithmetic).
-      auto scatter2 = [&](int ja, int jb, const float (&va)[8], const float (&vb)[8]) {
-        float u[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float send = b16 ? va[i] : vb[i];
-          const float keep = b16 ? vb[i] : va[i];
-          u[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 16);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float send = b8 ? u[i] : u[i + 4];
-          const float keep = b8 ? u[i + 4] : u[i];
-          u[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 8);
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const float send = b4 ? u[i] : u[i + 2];
-          const float keep = b4 ? u[i + 2] : u[i];
-          u[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 4);
-        }
-        {
-          const float send = b2 ? u[0] : u[1];
-          const float keep = b2 ? u[1] : u[0];
-          u[0] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 2);
-        }
-        u[0] += __shfl_xor_sync(0xFFFFFFFFu, u[0], 1);
-        // lane 2m holds index m = 8 b16 + 4 b8 + 2 b4 + b2 of u = (va, vb).
-        const int m = lane >> 1, e = m & 7;
-        if ((lane & 1) == 0 && e < 6) s_geo[(warp * (B + 1) + (m < 8 ? ja : jb)) * K::GR + e] = u[0];
-      };
-      auto evaluate = [&](int j, PairEval& pe) -> bool {
-        const bool h = eval_pair_flat(s_rec + j * kRec, pxc, pyc, pe);
-        return h && live && rel0 + (uint32_t)j < nc;
-      };
-      // The entries to visit, back to front: with an odd count the first
-      // (the latest in list order) alone, then pairs -- both evaluated, then
-      // replayed in order (the T chain).  A pair's warp sums are formed
-      // after the next pair's arithmetic (the first time, zeros go to the
-      // sink row), so the shuffles overlap independent work.
-      const int cnt = __popc(todo);
-      if (cnt & 1) {
-        const int ja = 31 - __clz(todo);
-        todo &= ~(1u << ja);
-        PairEval pa;
-        float va[8];
-        const bool ha = evaluate(ja, pa);
-        entry(ja, ha, pa, va);
-        if (__any_sync(0xFFFFFFFFu, ha)) {
-          jact |= 1u << ja;
-          scatter1(ja, va);
+        for (int pt = 0; pt < 4; ++pt) {
+          float* o = sl_w + fr * SS + 8 * pt + 2 * ft;
+          if (fr < m) *reinterpret_cast<float2*>(o) = make_float2(sa[pt][0], sa[pt][1]);
+          if (fr + 8 < m) *reinterpret_cast<float2*>(o + 8 * SS) = make_float2(sa[pt][2], sa[pt][3]);
         }
       }
-      float qa[8], qb[8];
+      __syncwarp();
+      // ---- replay of the chunk's entries, two at a time ----
+      // Entries of this batch the pixel reached (none if the wait gave up).
+      const uint32_t nc_rel = live && nc > rel0 ? nc - rel0 : 0u;
+      float clamp_sum = 0.0f;  // lane q: opacity sum of slot q's clamped pixels
+      auto evaluate = [&](int j, PairEval& pe) -> bool {
+        const bool h = eval_pair_flat(s_rec + j * kRec, pxc, pyc, pe);
+        return h & ((uint32_t)j < nc_rel);
+      };
+      // Entry j (slot q of the chunk) given its evaluation (hit: the pixel
+      // includes it), without branches so that the two entries of a pair
+      // interleave: a lane that did not blend takes alpha = 0, which leaves
+      // T and Q exactly as they were (1 / (1 - 0) = 1, w = 0).
+      auto entry = [&](int j, int q, bool hit, const PairEval& pe) {
+        const float2 zr = *reinterpret_cast<const float2*>(s_rec + j * kRec + 6);  // depth, r
+        const float2 gbl = *reinterpret_cast<const float2*>(s_rec + j * kRec + 8);  // g, b
+        float s = sl_w[q * SS + lane];
+        s = fmaf(zr.x, gz, fmaf(zr.y, g0, s)) + fmaf(gbl.x, g1, gbl.y * g2);
+        const float al = hit ? pe.alpha : 0.0f;
+        const float inv = rcp_approx(1.0f - al);  // 1 - alpha >= 0.01
+        T = T * inv;  // transmittance before this Gaussian
+        const float w = al * T;
+        const float dalpha = T * s - (Q - gaTf) * inv;
+        Q = fmaf(w, s, Q);
+        sl_w[q * SS + lane] = w;
+        sl_e[q * SS + lane] = hit && !pe.clamped ? dalpha * pe.alpha : 0.0f;
+        const bool over = hit && pe.clamped;
+        if (__any_sync(0xFFFFFFFFu, over)) {
+          // Pixels whose alpha was clamped add to the opacity sum alone.
+          float v = over ? dalpha * pe.G : 0.0f;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) qa[i] = qb[i] = 0.0f;
-      int qja = B, qjb = B;
-      for (int n = 0; n < cnt / 2; ++n) {
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+          if (lane == q) clamp_sum = v;
+        }
+      };
+      int q = 0;
+      for (; q + 1 < m; q += 2) {
         const int ja = 31 - __clz(todo);
         todo &= ~(1u << ja);
         const int jb = 31 - __clz(todo);
         todo &= ~(1u << jb);
         PairEval pa, pb;
-        float va[8], vb[8];
         const bool ha = evaluate(ja, pa);
         const bool hb = evaluate(jb, pb);
-        const bool aa = __any_sync(0xFFFFFFFFu, ha), ab = __any_sync(0xFFFFFFFFu, hb);
-        // Neither entry blends in this warp (only without the forward's
-        // masks): nothing changes, nothing to sum.
-        if (!(aa || ab)) continue;
-        entry(ja, ha, pa, va);
-        entry(jb, hb, pb, vb);
-        jact |= (aa ? 1u << ja : 0u) | (ab ? 1u << jb : 0u);
-        scatter2(qja, qjb, qa, qb);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          qa[i] = va[i];
-          qb[i] = vb[i];
-        }
-        qja = ja;
-        qjb = jb;
+        entry(ja, q, ha, pa);
+        entry(jb, q + 1, hb, pb);
       }
-      if (cnt >= 2) scatter2(qja, qjb, qa, qb);
+      if (q < m) {
+        const int ja = 31 - __clz(todo);
+        todo &= ~(1u << ja);
+        PairEval pa;
+        const bool ha = evaluate(ja, pa);
+        entry(ja, q, ha, pa);
+      }
       __syncwarp();
-      if (K::JPL == 2 && jact && __popc(jact) <= 16) {
-        // At most 16 active entries: lane pair jg takes the jg-th active
-        // entry, so one pass covers them all (P rows of inactive entries
-        // are left unwritten: the combine reads only active ones).
-        constexpr int CP2 = K::CPL / 2;
-        const int jg = lane >> 1, cg = lane & 1;
-        const bool has = jg < __popc(jact);
-        const int jl = has ? (int)__fns(jact, 0, jg + 1) : 0;
-        float2 acc[CP2];
+      // ---- P[entry][channel] and M[entry][moment] ----
+      // First operands: rows fr and fr + 8 of the slices (slots past the
+      // chunk repeat its last entry or are zero; their results are not used).
+      auto load_rows = [&](const float* sl, uint32_t (&v)[3][2][4]) {
 #pragma unroll
-        for (int c = 0; c < CP2; ++c) acc[c] = make_float2(0.0f, 0.0f);
-#pragma unroll 4
-        for (int p = 0; p < 32; ++p) {
-          const float wv = has ? slice[p * WS + jl] : 0.0f;
-          const float2* gr = reinterpret_cast<const float2*>(s_G + (warp * 32 + p) * GS + cg * K::CPL);
-#pragma unroll
-          for (int c = 0; c < CP2; ++c) acc[c] = __ffma2_rn(make_float2(wv, wv), gr[c], acc[c]);
-        }
-        __syncwarp();
-        if (has) {
-#pragma unroll
-          for (int c = 0; c < CP2; ++c) {
-            // Colour and depth (the first two pairs) go to the scalar row.
-            float* dst = (cg == 0 && c < 2) ? s_geo + (warp * (B + 1) + jl) * K::GR + 6 + 2 * c
-                                            : slice + jl * NC + cg * K::CPL + 2 * c;
-            *reinterpret_cast<float2*>(dst) = acc[c];
-          }
-        }
-      } else if (jact) {
-        // P[j][c] = sum over the warp's pixels of w[p][j] * G[p][c], channel
-        // pairs in packed FMAs.
-        constexpr int CP2 = K::CPL / 2;
-        const int jg = lane >> 1, cg = lane & 1;
-        float2 acc[K::JPL][CP2];
-#pragma unroll
-        for (int jj = 0; jj < K::JPL; ++jj)
-#pragma unroll
-          for (int c = 0; c < CP2; ++c) acc[jj][c] = make_float2(0.0f, 0.0f);
-#pragma unroll 4
-        for (int p = 0; p < 32; ++p) {
-          float wv[K::JPL];
-          if (K::JPL == 2) {
-            const float2 t2 = *reinterpret_cast<const float2*>(slice + p * WS + jg * 2);
-            wv[0] = t2.x; wv[1] = t2.y;
+        for (int s = 0; s < 2; ++s) {
+          const float4 va = *reinterpret_cast<const float4*>(sl + min(fr, m - 1) * SS + 8 * ft + 4 * s);
+          split3(va.x, va.y, v[0][s][0], v[1][s][0], v[2][s][0]);
+          split3(va.z, va.w, v[0][s][2], v[1][s][2], v[2][s][2]);
+          if (m > 8) {
+            const float4 vb = *reinterpret_cast<const float4*>(sl + min(fr + 8, m - 1) * SS + 8 * ft + 4 * s);
+            split3(vb.x, vb.y, v[0][s][1], v[1][s][1], v[2][s][1]);
+            split3(vb.z, vb.w, v[0][s][3], v[1][s][3], v[2][s][3]);
           } else {
-            wv[0] = slice[p * WS + jg];
-          }
-          const float2* gr = reinterpret_cast<const float2*>(s_G + (warp * 32 + p) * GS + cg * K::CPL);
 #pragma unroll
-          for (int c = 0; c < CP2; ++c) {
-            const float2 gv = gr[c];
-#pragma unroll
-            for (int jj = 0; jj < K::JPL; ++jj) acc[jj][c] = __ffma2_rn(make_float2(wv[jj], wv[jj]), gv, acc[jj][c]);
+            for (int t = 0; t < 3; ++t) v[t][s][1] = v[t][s][3] = 0u;
           }
         }
-        __syncwarp();
+      };
+      float mo[4] = {0.f, 0.f, 0.f, 0.f};
+      {
+        uint32_t ea[3][2][4];
+        load_rows(sl_e, ea);
 #pragma unroll
-        for (int jj = 0; jj < K::JPL; ++jj)
+        for (int t = 2; t >= 0; --t)
 #pragma unroll
-          for (int c = 0; c < CP2; ++c)
-          {
-            const int jj2 = jg * K::JPL + jj;
-            float* dst = (cg == 0 && c < 2) ? s_geo + (warp * (B + 1) + jj2) * K::GR + 6 + 2 * c
-                                            : slice + jj2 * NC + cg * K::CPL + 2 * c;
-            *reinterpret_cast<float2*>(dst) = acc[jj][c];
-          }
+          for (int s = 0; s < 2; ++s) mma_bf16_16816(mo, ea[t][s], mom[2 * s], mom[2 * s + 1]);
       }
+      uint32_t wa[3][2][4];
+      load_rows(sl_w, wa);
+      __syncwarp();  // every lane has its rows: partial rows may take their place
+      // Channel tiles, then colour and depth as four more channels (columns
+      // 4-7 of their tile zero).
+      float acc[NT + 1][4];
+      // The tiles' chains run side by side.
+#pragma unroll
+      for (int p = 0; p < 6; ++p) {
+        uint4 g[NT + 1];
+#pragma unroll
+        for (int nt = 0; nt <= NT; ++nt)
+          g[nt] = nt < NT || fr < 4 ? *reinterpret_cast<const uint4*>(s_G + kTermB[p] * K::GTERM + g_chunk(8 * nt + fr, ft))
+                                    : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int nt = 0; nt <= NT; ++nt) {
+          if (p == 0) mma_bf16_16816_first(acc[nt], wa[kTermA[p]][0], g[nt].x, g[nt].y);
+          else mma_bf16_16816(acc[nt], wa[kTermA[p]][0], g[nt].x, g[nt].y);
+        }
+#pragma unroll
+        for (int nt = 0; nt <= NT; ++nt) mma_bf16_16816(acc[nt], wa[kTermA[p]][1], g[nt].z, g[nt].w);
+      }
+      // Geometric sums of rows fr and fr + 8 from their moments (spread over
+      // the quad: lane ft holds moments 2 ft and 2 ft + 1): two columns to a
+      // lane.
+      float2 geo[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float lo = mo[2 * h], hi = mo[2 * h + 1];
+        const float m0 = __shfl_sync(0xFFFFFFFFu, lo, 0, 4), mx = __shfl_sync(0xFFFFFFFFu, hi, 0, 4);
+        const float my = __shfl_sync(0xFFFFFFFFu, lo, 1, 4), mxx = __shfl_sync(0xFFFFFFFFu, hi, 1, 4);
+        const float mxy = __shfl_sync(0xFFFFFFFFu, lo, 2, 4), myy = __shfl_sync(0xFFFFFFFFu, hi, 2, 4);
+        const int r = fr + 8 * h;
+        const float cl = __shfl_sync(0xFFFFFFFFu, clamp_sum, r);
+        const float* rec = s_rec + s_list[c0 + min(r, m - 1)] * kRec;
+        const float4 r0 = *reinterpret_cast<const float4*>(rec);      // u, v, A, B
+        const float2 r4 = *reinterpret_cast<const float2*>(rec + 4);  // Cc, opacity
+        const float ox = cxw - r0.x, oy = cyw - r0.y;
+        // Sums of e dx^i dy^j, dx = x + ox, dy = y + oy.
+        const float ex = fmaf(ox, m0, mx), ey = fmaf(oy, m0, my);
+        const float exx = fmaf(ox, mx + ex, mxx);
+        const float exy = fmaf(ox, my, fmaf(oy, ex, mxy));
+        const float eyy = fmaf(oy, my + ey, myy);
+        // power2 = log2(alpha / opacity): dL/dpower2 = e ln 2.
+        if (ft == 0) geo[h] = make_float2(-kLn2 * fmaf(2.0f * r0.z, ex, r0.w * ey), -kLn2 * fmaf(2.0f * r4.x, ey, r0.w * ex));
+        else if (ft == 1) geo[h] = make_float2(kLn2 * exx, kLn2 * exy);
+        else geo[h] = make_float2(kLn2 * eyy, __fdividef(m0, r4.y) + cl);
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (fr + 8 * h < m) {
+          float* row = area + (c0 + fr + 8 * h) * PR + 2 * ft;
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt)
+            *reinterpret_cast<float2*>(row + 8 * nt) = make_float2(acc[nt][2 * h], acc[nt][2 * h + 1]);
+          if (ft < 3) {
+            // du dv | dA dB | dCc dopacity, then r g | b depth | 0 0.
+            *reinterpret_cast<float2*>(row + D) = geo[h];
+            *reinterpret_cast<float2*>(row + D + 6) = make_float2(acc[NT][2 * h], acc[NT][2 * h + 1]);
+          }
+        }
+      }
+      __syncwarp();  // the area may be written again
     }
     if (lane == 0) s_jact[warp] = jact;
     __syncthreads();
@@ -815,33 +879,29 @@ __device__ __forceinline__ void bwd_tile(const CompositeArgs& a, const int tile,
       jm[w8] = s_jact[w8];
       bm |= jm[w8];
     }
-    // One item = four consecutive columns of an active entry's partial row
-    // [features | du dv dA dB dCc dopacity | r g b | depth | 0 0]: the warp
-    // partials (feature columns from the warp slices, the rest from the
-    // warps' scalar rows, which have that layout) summed in warp order, one
-    // 16-byte store.  A channel-split pass that is not the first adds its
-    // geometric terms (du .. dopacity) to the row the first pass wrote and
-    // leaves colour and depth alone.
-    // Items over every entry slot (a compile-time count of column groups):
-    // slots no pixel blended, and the last group outside the first pass,
-    // are skipped.
-    constexpr int NQ = D / 4 + 3;
-    for (int item = tid; item < B * NQ; item += kThreads) {
-      const int j = item / NQ, q4 = item - j * NQ;
-      if (!((bm >> j) & 1u) || (!a.aux && q4 == NQ - 1)) continue;
-      const bool fcol = q4 < D / 4;
-      const float* src = fcol ? s_slice + j * NC + 4 + 4 * q4 : s_geo + j * K::GR + 4 * (q4 - D / 4);
-      const int wstride = fcol ? K::SLICE : (B + 1) * K::GR;
+    // A group of lanes takes one active entry at a time, each lane four
+    // consecutive columns of its partial row [features | du dv dA dB dCc
+    // dopacity | r g b | depth | 0 0]: the warps' rows of that entry (in warp
+    // w at the number of its later entries) summed in warp order, one 16-byte
+    // store.  A channel-split pass that is not the first adds its geometric
+    // terms (du .. dopacity) to the row the first pass wrote and leaves
+    // colour and depth (the last four columns) alone.
+    constexpr int NQ = PR / 4, GL = NQ <= 8 ? 8 : NQ <= 16 ? 16 : 32;
+    const int q4 = tid % GL;
+    const bool col = q4 < NQ && (a.aux || q4 < NQ - 1);
+    for (int j = tid / GL; j < B; j += kThreads / GL) {
+      if (!((bm >> j) & 1u) || !col) continue;
+      const float* src = s_area + 4 * q4;
       float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
       for (int w8 = 0; w8 < 8; ++w8) {
-        if ((jm[w8] >> j) & 1u) {
-          const float4 v = *reinterpret_cast<const float4*>(src + w8 * wstride);
-          acc.x += v.x;
-          acc.y += v.y;
-          acc.z += v.z;
-          acc.w += v.w;
-        }
+        const uint32_t later = jm[w8] >> j;
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (later & 1u) v = *reinterpret_cast<const float4*>(src + w8 * K::AREA + __popc(later >> 1) * PR);
+        acc.x += v.x;
+        acc.y += v.y;
+        acc.z += v.z;
+        acc.w += v.w;
       }
       if ((int64_t)se[j] < a.cap) {
         float* row = a.partials + (size_t)se[j] * a.prow;
@@ -988,28 +1048,32 @@ cudaError_t launch_bwd_batch_t(const BatchCompositeArgs& b, int bf16, cudaStream
   return cudaGetLastError();
 }
 
-// D = 256 runs as two passes over 128-channel halves (h = 0, 1): the same
-// list, the same per-pixel decisions, each pass staging and accumulating
-// its half of every feature row.  Pass 0 owns colour, depth, alpha, T_final,
-// n_contrib, the blend masks and (reverse) the colour / depth / alpha /
-// background terms; the reverse's geometric terms are linear in the dot
-// products g . x, so pass 1 adds the share of its channels to the rows pass
-// 0 wrote (same stream, pass 0 first: a fixed order).
-CompositeArgs channel_half(const CompositeArgs& a, int h) {
+// Wide features run as several passes over `width` channels each (part h of
+// them): the same list, the same per-pixel decisions, each pass staging and
+// accumulating its part of every feature row.  Part 0 owns colour, depth,
+// alpha, T_final, n_contrib, the blend masks and (reverse) the colour / depth
+// / alpha / background terms; the reverse's geometric terms are linear in the
+// dot products g . x, so a later part adds the share of its channels to the
+// rows the earlier ones wrote (same stream, in order: a fixed order).  The
+// forward takes 128 channels a pass, the reverse 64 (its operands of 128
+// channels do not fit in shared memory; two 64-channel passes repeat the
+// evaluation and the replay but not the products, which dominate).
+CompositeArgs channel_part(const CompositeArgs& a, int width, int h) {
   CompositeArgs c = a;
   const size_t elem = a.feat_bf16 ? 2 : 4;
-  c.D = 128;
-  c.feat = static_cast<const unsigned char*>(a.feat) + (size_t)h * 128 * elem;
-  if (a.out_feat) c.out_feat = a.out_feat + h * 128;
-  if (a.out_feat_bf16) c.out_feat_bf16 = a.out_feat_bf16 + h * 128;
-  if (a.g_feat) c.g_feat = a.g_feat + h * 128;
-  c.pcol0 = a.pcol0 + h * 128;
+  c.D = width;
+  c.feat = static_cast<const unsigned char*>(a.feat) + (size_t)h * width * elem;
+  if (a.out_feat) c.out_feat = a.out_feat + h * width;
+  if (a.out_feat_bf16) c.out_feat_bf16 = a.out_feat_bf16 + h * width;
+  if (a.g_feat) c.g_feat = a.g_feat + h * width;
+  c.pcol0 = a.pcol0 + h * width;
   if (h > 0) {
     c.aux = 0;
     c.g_rgb = c.g_depth = c.g_alpha = nullptr;
   }
   return c;
 }
+constexpr int kFwdPart = 128, kBwdPart = 64;
 
 }  // namespace
 
@@ -1023,9 +1087,9 @@ cudaError_t launch_composite_fwd(const CompositeArgs& a, int fwd_batch, cudaStre
     case 64: return launch_fwd_d<64>(a, fwd_batch, st);
     case 128: return launch_fwd_d<128>(a, fwd_batch, st);
     case 256: {
-      if (a.counts) return launch_fwd_d<128>(channel_half(a, 0), fwd_batch, st);
-      const cudaError_t e = launch_fwd_d<128>(channel_half(a, 0), fwd_batch, st);
-      return e != cudaSuccess ? e : launch_fwd_d<128>(channel_half(a, 1), fwd_batch, st);
+      const cudaError_t e = launch_fwd_d<128>(channel_part(a, kFwdPart, 0), fwd_batch, st);
+      if (e != cudaSuccess || a.counts) return e;
+      return launch_fwd_d<128>(channel_part(a, kFwdPart, 1), fwd_batch, st);
     }
   }
   return cudaErrorInvalidValue;
@@ -1037,20 +1101,21 @@ cudaError_t launch_composite_bwd(const CompositeArgs& a, cudaStream_t st) {
     case 16: return launch_bwd_t<16>(a, st);
     case 32: return launch_bwd_t<32>(a, st);
     case 64: return launch_bwd_t<64>(a, st);
-    case 128: return launch_bwd_t<128>(a, st);
+    case 128:
     case 256: {
-      const cudaError_t e = launch_bwd_t<128>(channel_half(a, 0), st);
-      return e != cudaSuccess ? e : launch_bwd_t<128>(channel_half(a, 1), st);
+      cudaError_t e = cudaSuccess;
+      for (int h = 0; h < a.D / kBwdPart && e == cudaSuccess; ++h) e = launch_bwd_t<64>(channel_part(a, kBwdPart, h), st);
+      return e;
     }
   }
   return cudaErrorInvalidValue;
 }
 
-// The batch's per-view arguments for channel half h, its own work counter.
-static BatchCompositeArgs batch_half(const BatchCompositeArgs& b, int h) {
+// The batch's per-view arguments for channel part h, its own work counter.
+static BatchCompositeArgs batch_part(const BatchCompositeArgs& b, int width, int h) {
   BatchCompositeArgs c = b;
-  for (int v = 0; v < b.V; ++v) c.view[v] = channel_half(b.view[v], h);
-  c.queue = b.queue + 2 * h;
+  for (int v = 0; v < b.V; ++v) c.view[v] = channel_part(b.view[v], width, h);
+  c.queue = b.queue + h;
   return c;
 }
 
@@ -1063,8 +1128,8 @@ cudaError_t launch_composite_fwd_batch(const BatchCompositeArgs& b, int D, int f
     case 64: return launch_fwd_batch_d<64>(b, feat_bf16, fwd_batch, st);
     case 128: return launch_fwd_batch_d<128>(b, feat_bf16, fwd_batch, st);
     case 256: {
-      const cudaError_t e = launch_fwd_batch_d<128>(batch_half(b, 0), feat_bf16, fwd_batch, st);
-      return e != cudaSuccess ? e : launch_fwd_batch_d<128>(batch_half(b, 1), feat_bf16, fwd_batch, st);
+      const cudaError_t e = launch_fwd_batch_d<128>(batch_part(b, kFwdPart, 0), feat_bf16, fwd_batch, st);
+      return e != cudaSuccess ? e : launch_fwd_batch_d<128>(batch_part(b, kFwdPart, 1), feat_bf16, fwd_batch, st);
     }
   }
   return cudaErrorInvalidValue;
@@ -1076,10 +1141,12 @@ cudaError_t launch_composite_bwd_batch(const BatchCompositeArgs& b, int D, int f
     case 16: return launch_bwd_batch_t<16>(b, feat_bf16, st);
     case 32: return launch_bwd_batch_t<32>(b, feat_bf16, st);
     case 64: return launch_bwd_batch_t<64>(b, feat_bf16, st);
-    case 128: return launch_bwd_batch_t<128>(b, feat_bf16, st);
+    case 128:
     case 256: {
-      const cudaError_t e = launch_bwd_batch_t<128>(batch_half(b, 0), feat_bf16, st);
-      return e != cudaSuccess ? e : launch_bwd_batch_t<128>(batch_half(b, 1), feat_bf16, st);
+      cudaError_t e = cudaSuccess;
+      for (int h = 0; h < D / kBwdPart && e == cudaSuccess; ++h)
+        e = launch_bwd_batch_t<64>(batch_part(b, kBwdPart, h), feat_bf16, st);
+      return e;
     }
   }
   return cudaErrorInvalidValue;
