@@ -142,6 +142,7 @@ BinArgs bin_args(const Layout& L, void* ws) {
   b.ntiles = L.ntiles;
   b.tiles_x = L.tiles_x;
   b.pblocks = L.pblocks;
+  b.bchunk = L.bchunk;
   b.bblocks = L.bblocks;
   b.cap = L.cap;
   b.rect = at<ushort4>(ws, L.rect);

@@ -2,12 +2,14 @@
 // builds on (Sec. 2.1), reorganised for one GPU:
 //   1. stable LSD radix sort of the P depth keys (4 x 8-bit passes);
 //   2. exclusive scan of tiles_touched in depth order (decoupled look-back)
-//      and, per block of 1024 depth-ordered Gaussians, its count of
-//      entries per tile (a tile-major (tile, block) table);
+//      and, per block of depth-ordered Gaussians, its count of entries per
+//      tile (a tile-major (tile, block) table);
 //   3. exclusive scan of that table: the start of every (tile, block)
 //      segment of the final list, and the tile ranges;
-//   4. a scatter in which each warp walks its Gaussians in depth order with
-//      per-warp tile counters, so every entry lands at its final position.
+//   4. a scatter in which a block marks, per tile, which of its Gaussians
+//      touch it (bit masks); an entry's place is its segment's start plus the
+//      number of earlier Gaussians in the tile's mask, so the entries are
+//      taken in any order.
 // The result is the order of a stable sort on (tile << 32 | depth bits) with
 // ties by index, built with one write per entry instead of radix passes over
 // 64-bit keys.  Every inter-block wait is a bounded spin that records
@@ -251,11 +253,18 @@ __device__ __forceinline__ uint64_t lookback64(uint64_t* status, uint32_t b, uin
   return lookback64_resolve(status, b, aggregate, err);
 }
 
-// Step 2: block b (ticket) owns depth ranks [512 b, 512 b + 512); thread t
-// scans ranks 2t..2t+1.  Writes offs / offs_by_gid and column b of the
-// tile-major count table.
+// Tile of item k (row-major) of a Gaussian's tile rectangle, iw = 1 / width
+// (exact for k < 2^20).
+__device__ __forceinline__ uint32_t rect_tile(const ushort4 rc, float iw, uint32_t k, int tiles_x) {
+  const uint32_t dy = (uint32_t)(((float)k + 0.5f) * iw), dx = k - dy * (rc.z - rc.x + 1u);
+  return (rc.y + dy) * (uint32_t)tiles_x + rc.x + dx;
+}
+
+// Step 2: block b (ticket) owns depth ranks [chunk b, chunk b + chunk), chunk
+// <= 512; thread t scans ranks 2t and 2t + 1.  Writes offs / offs_by_gid and
+// column b of the tile-major count table.
 struct CountArgs {
-  int P, tiles_x, ntiles, nblocks;
+  int P, tiles_x, ntiles, nblocks, chunk;
   int64_t cap;
   const uint32_t* order;  // depth-sorted Gaussian ids
   const uint32_t* touched;
@@ -272,27 +281,24 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
   __shared__ uint32_t s_ticket;
   __shared__ uint64_t s_prefix;
   __shared__ uint32_t s_c[kBinChunk];
-  __shared__ float s_iw[kBinChunk];  // 1 / (rect width in tiles), once per Gaussian
   __shared__ ushort4 s_rect[kBinChunk];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   for (int i = tid; i < a.ntiles; i += kThreads) s_cnt[i] = 0;
   if (tid == 0) s_ticket = atomicAdd(a.ticket, 1u);
   __syncthreads();
   const uint32_t b = s_ticket;
-  const int64_t start = (int64_t)b * kBinChunk;
+  const int64_t start = (int64_t)b * a.chunk;
   if (start >= a.P) return;
-  uint32_t gid[kBinItems], cnt[kBinItems];
+  const int nloc = (int)min((int64_t)a.chunk, (int64_t)a.P - start);
+  uint32_t gid[2], cnt[2];
   uint32_t tsum = 0;
 #pragma unroll
-  for (int i = 0; i < kBinItems; ++i) {
-    const int li = tid * kBinItems + i;
-    const int64_t r = start + li;
-    gid[i] = r < a.P ? a.order[r] : 0u;
-    cnt[i] = r < a.P ? a.touched[gid[i]] : 0u;
+  for (int i = 0; i < 2; ++i) {
+    const int li = tid * 2 + i;
+    gid[i] = li < nloc ? a.order[start + li] : 0u;
+    cnt[i] = li < nloc ? a.touched[gid[i]] : 0u;
     s_c[li] = cnt[i];
-    const ushort4 rc = cnt[i] ? a.rect[gid[i]] : make_ushort4(0, 0, 0, 0);
-    s_rect[li] = rc;
-    s_iw[li] = 1.0f / (float)(rc.z - rc.x + 1u);
+    s_rect[li] = cnt[i] ? a.rect[gid[i]] : make_ushort4(0, 0, 0, 0);
     tsum += cnt[i];
   }
   uint32_t btot;
@@ -300,34 +306,28 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
   // The block's total goes out at once; its tile counts, which do not need
   // the prefix, are taken while the predecessors resolve theirs.
   if (tid == 0) lookback64_publish(a.status, b, btot);
-  // Tile counts: each warp walks its Gaussians, lanes over one rect's tiles.
-  const int nloc = (int)min((int64_t)kBinChunk, (int64_t)a.P - start);
-  const int i0 = warp * (kBinChunk / 8), i1 = min(nloc, i0 + kBinChunk / 8);
-  for (int i = i0; i < i1; ++i) {
-    const uint32_t c = s_c[i];
-    if (!c) continue;
-    const ushort4 rc = s_rect[i];
-    const uint32_t wdt = rc.z - rc.x + 1u;
-    const float iw = s_iw[i];
-    for (uint32_t k = lane; k < c; k += 32) {
-      const uint32_t dy = (uint32_t)(((float)k + 0.5f) * iw), dx = k - dy * wdt;  // exact for these sizes
-      atomicAdd(&s_cnt[(rc.y + dy) * (uint32_t)a.tiles_x + rc.x + dx], 1u);
-    }
+  // Tile counts: four threads to a Gaussian, in any order.
+  for (int w = tid; w < 4 * nloc; w += kThreads) {
+    const uint32_t c = s_c[w >> 2];
+    if ((uint32_t)(w & 3) >= c) continue;
+    const ushort4 rc = s_rect[w >> 2];
+    const float iw = 1.0f / (float)(rc.z - rc.x + 1u);
+    for (uint32_t k = w & 3; k < c; k += 4) atomicAdd(&s_cnt[rect_tile(rc, iw, k, a.tiles_x)], 1u);
   }
   if (tid == 0) s_prefix = lookback64_resolve(a.status, b, btot, &a.hdr->err);
   __syncthreads();
   uint64_t run = s_prefix + texcl;
 #pragma unroll
-  for (int i = 0; i < kBinItems; ++i) {
-    const int64_t r = start + tid * kBinItems + i;
-    if (r < a.P) {
+  for (int i = 0; i < 2; ++i) {
+    const int li = tid * 2 + i;
+    if (li < nloc) {
       const uint32_t o32 = (uint32_t)min(run, (uint64_t)0xFFFFFFFFu);
-      a.offs[r] = o32;
+      a.offs[start + li] = o32;
       a.offs_by_gid[gid[i]] = o32;
     }
     run += cnt[i];
   }
-  if (start + kBinChunk >= a.P && tid == kThreads - 1) {
+  if (start + a.chunk >= a.P && tid == kThreads - 1) {
     a.offs[a.P] = (uint32_t)min(run, (uint64_t)0xFFFFFFFFu);
     a.hdr->num_dups = (uint32_t)min(run, (uint64_t)0xFFFFFFFFu);
     if (run > (uint64_t)a.cap) set_err(&a.hdr->err, kErrOverflow);
@@ -368,13 +368,24 @@ __global__ void __launch_bounds__(kThreads) table_scan_kernel(uint32_t* table, i
   }
 }
 
-// Step 4: block b (= blockIdx.x) re-walks the ranks of count block b.  Each
-// warp takes 64 consecutive Gaussians; its lanes cover one Gaussian's tiles
-// at a time (all distinct), so per-warp tile counters give stable ranks.
+// Step 4: block b (= blockIdx.x) takes the ranks of count block b, 128
+// Gaussians (a round) at a time.  Per tile it keeps a 128-bit mask of the
+// round's Gaussians that touch it (atomic ors: no order among them); then,
+// per tile, how many entries the round's later 32-Gaussian groups still add
+// (four bytes) beside the segment's position after the round, so an entry's
+// place is
+//   position after the round - entries from its group on + earlier bits of its group.
+// Entries are spread over all threads of the block, several to a Gaussian.
+// Bound by the scattered 8-byte stores and by instruction issue (two visits
+// of every entry at about ten and twenty instructions, and a sweep of the
+// tiles per round).  A warp that walked its 64 Gaussians one after another
+// with per-warp tile counters took 27 us at 1,000 Gaussians (the latency of
+// that chain; now 3), 28 at 30k (now 7), 44 at 200k (2.5 M entries; now 37)
+// and 591 at 1M (33 M; now 457).
 // Block 0 also writes the tile ranges and marks the workspace as holding a
 // forward's state.
 struct ScatterArgs {
-  int P, tiles_x, ntiles, nblocks;
+  int P, tiles_x, ntiles, nblocks, chunk;
   int64_t cap;
   const uint32_t *order, *touched, *offs, *table;
   const ushort4* rect;
@@ -382,25 +393,50 @@ struct ScatterArgs {
   uint2* ranges;
   Header* hdr;
 };
+// Threads per block: with the masks of more tiles than this only one or two
+// blocks fit on an SM, so they get more threads.
+constexpr int kScatTiles = 2048;
+constexpr int kRound = 128;  // Gaussians per round (four 32-bit mask words)
+__host__ __device__ constexpr size_t scatter_smem(int ntiles) { return (size_t)ntiles * (16 + 4 + 4); }
 
-__global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const ScatterArgs a) {
+template <int NT>
+__global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
-  uint32_t* s_base = s_dyn;                                        // [ntiles]
-  uint16_t* s_wc = reinterpret_cast<uint16_t*>(s_dyn + a.ntiles);  // [8][ntiles]
+  uint4* s_mask = reinterpret_cast<uint4*>(s_dyn);  // [ntiles]
+  uint32_t* s_word = s_dyn;                         // the same, [ntiles][4]
+  uint32_t* s_suf = s_dyn + 4 * a.ntiles;           // [ntiles]: four suffix counts
+  uint32_t* s_pos = s_suf + a.ntiles;               // [ntiles]: next position of the tile's segment
   __shared__ uint32_t s_gid[kBinChunk], s_cnt[kBinChunk], s_off[kBinChunk];
-  __shared__ float s_iw[kBinChunk];  // 1 / (rect width in tiles), once per Gaussian
+  __shared__ float s_iw[kBinChunk];  // 1 / (rect width in tiles)
   __shared__ ushort4 s_rect[kBinChunk];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int b = blockIdx.x;
-  const int64_t start = (int64_t)b * kBinChunk;
-  const int nloc = (int)min((int64_t)kBinChunk, (int64_t)a.P - start);
+  const int64_t start = (int64_t)b * a.chunk;
+  const int nloc = (int)min((int64_t)a.chunk, (int64_t)a.P - start);
   const uint64_t cap = (uint64_t)a.cap;
   // Past capacity the list is incomplete (and flagged): every range is
   // published empty so no later kernel follows an index beyond capacity.
   const bool overflow = (uint64_t)a.hdr->num_dups > cap;
   const uint64_t K = overflow ? 0 : (uint64_t)a.hdr->num_dups;
-  for (int t = tid; t < a.ntiles; t += kThreads) {
-    s_base[t] = a.table[(size_t)t * a.nblocks + b];
+  // The block's Gaussians, all rounds at once (three dependent loads).
+  const int npad = (nloc + kRound - 1) / kRound * kRound;
+  for (int j = tid; j < npad; j += NT) {
+    uint32_t g = 0, c = 0;
+    ushort4 rc = make_ushort4(0, 0, 0, 0);
+    if (j < nloc) {
+      g = a.order[start + j];
+      s_off[j] = a.offs[start + j];
+      c = a.touched[g];
+      if (c) rc = a.rect[g];
+    }
+    s_gid[j] = g;
+    s_cnt[j] = c;
+    s_rect[j] = rc;
+    s_iw[j] = 1.0f / (float)(rc.z - rc.x + 1u);
+  }
+  for (int t = tid; t < a.ntiles; t += NT) {
+    s_pos[t] = a.table[(size_t)t * a.nblocks + b];
+    s_mask[t] = make_uint4(0u, 0u, 0u, 0u);
     if (b == 0) {
       const uint64_t lo = min((uint64_t)a.table[(size_t)t * a.nblocks], K);
       const uint64_t hi = t + 1 < a.ntiles ? min((uint64_t)a.table[(size_t)(t + 1) * a.nblocks], K) : K;
@@ -408,61 +444,37 @@ __global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const ScatterArgs
     }
   }
   if (b == 0 && tid == 0) a.hdr->has_forward = 1u;
-  for (int i = tid; i < 8 * a.ntiles; i += kThreads) s_wc[i] = 0;
-  for (int i = tid; i < nloc; i += kThreads) {
-    const uint32_t g = a.order[start + i];
-    const uint32_t c = a.touched[g];
-    s_gid[i] = g;
-    s_cnt[i] = c;
-    s_off[i] = a.offs[start + i];
-    const ushort4 rc = c ? a.rect[g] : make_ushort4(0, 0, 0, 0);
-    s_rect[i] = rc;
-    s_iw[i] = 1.0f / (float)(rc.z - rc.x + 1u);
-  }
+  constexpr int TPG = NT / kRound;  // threads per Gaussian
+  const int i = tid / TPG, sub = tid % TPG;
   __syncthreads();
-  uint16_t* wc = s_wc + (size_t)warp * a.ntiles;
-  const int i0 = warp * (kBinChunk / 8), i1 = min(nloc, i0 + kBinChunk / 8);
-  for (int i = i0; i < i1; ++i) {
-    const uint32_t c = s_cnt[i];
-    if (!c) continue;
-    const ushort4 rc = s_rect[i];
-    const uint32_t wdt = rc.z - rc.x + 1u;
-    const float iw = s_iw[i];
-    for (uint32_t k = lane; k < c; k += 32) {
-      const uint32_t dy = (uint32_t)(((float)k + 0.5f) * iw), dx = k - dy * wdt;  // exact for k < 2^20
-      const uint32_t tile = (rc.y + dy) * (uint32_t)a.tiles_x + rc.x + dx;
-      wc[tile] = (uint16_t)(wc[tile] + 1u);
+  for (int r0 = 0; r0 < nloc; r0 += kRound) {
+    const uint32_t c = s_cnt[r0 + i];
+    const ushort4 rc = s_rect[r0 + i];
+    const float iw = s_iw[r0 + i];
+    for (uint32_t k = sub; k < c; k += TPG) atomicOr(&s_word[4 * rect_tile(rc, iw, k, a.tiles_x) + (i >> 5)], 1u << (i & 31));
+    __syncthreads();
+    for (int t = tid; t < a.ntiles; t += NT) {
+      const uint4 m = s_mask[t];
+      const uint32_t n3 = __popc(m.w), n2 = n3 + __popc(m.z), n1 = n2 + __popc(m.y), n0 = n1 + __popc(m.x);
+      s_suf[t] = n0 | (n1 << 8) | (n2 << 16) | (n3 << 24);
+      s_pos[t] += n0;
     }
-    __syncwarp();
-  }
-  __syncthreads();
-  for (int t = tid; t < a.ntiles; t += kThreads) {
-    uint32_t run = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      const uint32_t c = s_wc[w * a.ntiles + t];
-      s_wc[w * a.ntiles + t] = (uint16_t)run;
-      run += c;
+    __syncthreads();
+    if (sub < c) {
+      const uint32_t g = s_gid[r0 + i], e0 = s_off[r0 + i], lt = (1u << (i & 31)) - 1u;
+      const int sh = 8 * (i >> 5);
+      for (uint32_t k = sub; k < c; k += TPG) {
+        const uint32_t tile = rect_tile(rc, iw, k, a.tiles_x);
+        const uint64_t pos = (uint64_t)(s_pos[tile] - ((s_suf[tile] >> sh) & 0xFFu) + __popc(s_word[4 * tile + (i >> 5)] & lt));
+        const uint64_t e = (uint64_t)e0 + k;
+        if (pos < cap) a.sorted[pos] = make_uint2((uint32_t)e, g);
+      }
     }
-  }
-  __syncthreads();
-  for (int i = i0; i < i1; ++i) {
-    const uint32_t c = s_cnt[i];
-    if (!c) continue;
-    const ushort4 rc = s_rect[i];
-    const uint32_t wdt = rc.z - rc.x + 1u;
-    const float iw = s_iw[i];
-    const uint32_t g = s_gid[i], e0 = s_off[i];
-    for (uint32_t k = lane; k < c; k += 32) {
-      const uint32_t dy = (uint32_t)(((float)k + 0.5f) * iw), dx = k - dy * wdt;
-      const uint32_t tile = (rc.y + dy) * (uint32_t)a.tiles_x + rc.x + dx;
-      const uint32_t r = wc[tile];
-      wc[tile] = (uint16_t)(r + 1u);
-      const uint64_t pos = (uint64_t)s_base[tile] + r;
-      const uint64_t e = (uint64_t)e0 + k;
-      if (pos < cap) a.sorted[pos] = make_uint2((uint32_t)e, g);
+    __syncthreads();
+    if (r0 + kRound < nloc) {
+      for (int t = tid; t < a.ntiles; t += NT) s_mask[t] = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
     }
-    __syncwarp();
   }
 }
 
@@ -541,6 +553,7 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   ca.tiles_x = b.tiles_x;
   ca.ntiles = b.ntiles;
   ca.nblocks = bblocks;
+  ca.chunk = b.bchunk;
   ca.cap = b.cap;
   ca.order = b.dval[cur];
   ca.touched = b.touched;
@@ -566,6 +579,7 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   sa.tiles_x = b.tiles_x;
   sa.ntiles = b.ntiles;
   sa.nblocks = bblocks;
+  sa.chunk = b.bchunk;
   sa.cap = b.cap;
   sa.order = b.dval[cur];
   sa.touched = b.touched;
@@ -575,9 +589,14 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   sa.sorted = b.sorted;
   sa.ranges = b.ranges;
   sa.hdr = hdr;
-  const size_t scat_smem = (size_t)b.ntiles * 4 + (size_t)8 * b.ntiles * 2;
-  cudaFuncSetAttribute(bin_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)scat_smem);
-  bin_scatter_kernel<<<bblocks, kThreads, scat_smem, st>>>(sa);
+  const size_t smem = scatter_smem(b.ntiles);
+  if (b.ntiles <= kScatTiles) {
+    cudaFuncSetAttribute(bin_scatter_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    bin_scatter_kernel<512><<<bblocks, 512, smem, st>>>(sa);
+  } else {
+    cudaFuncSetAttribute(bin_scatter_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    bin_scatter_kernel<1024><<<bblocks, 1024, smem, st>>>(sa);
+  }
   return cudaGetLastError();
 }
 

@@ -85,10 +85,12 @@ constexpr int kSortItems = 16;
 constexpr int kSortChunk = kThreads * kSortItems;
 constexpr int kPItems = 8;
 constexpr int kPChunk = kThreads * kPItems;
-// Depth-ordered Gaussians per block of the tile count / scatter kernels
-// (each of the 8 warps walks 64 of them in order).
-constexpr int kBinItems = 2;
-constexpr int kBinChunk = kThreads * kBinItems;
+// Depth-ordered Gaussians per block of the tile count / scatter kernels: 512
+// where that gives every SM a block (longer runs of a tile's list per block,
+// a smaller (tile, block) table), else fewer, down to one round of the
+// scatter (128), so that a small scene is not left to a few blocks.
+constexpr int kBinChunk = 512;
+inline int bin_chunk(int64_t P) { return P >= 152 * 512 ? kBinChunk : (P >= 152 * 256 ? 256 : 128); }
 
 // Ticket slots in the header.
 enum : int {
@@ -103,7 +105,7 @@ enum : int {
 constexpr int kMaxTiles = 8192;
 
 struct Layout {
-  int P, D, W, H, tw, th, tiles_x, tiles_y, ntiles, pblocks, bblocks;
+  int P, D, W, H, tw, th, tiles_x, tiles_y, ntiles, pblocks, bchunk, bblocks;
   int64_t cap;
   bool with_backward;
   size_t hdr, rec, rect, touched, dkey[2], dval[2], offs, offs_by_gid, sorted, table;
@@ -128,7 +130,8 @@ inline Layout make_layout(int P, int D, int W, int H, int tw, int th, int64_t ca
   const size_t Pn = (size_t)(P > 0 ? P : 1);
   const size_t Kn = (size_t)(cap > 0 ? cap : 1);
   L.pblocks = ceil_div((int64_t)Pn, kPChunk);
-  L.bblocks = ceil_div((int64_t)Pn, kBinChunk);
+  L.bchunk = bin_chunk((int64_t)Pn);
+  L.bblocks = ceil_div((int64_t)Pn, L.bchunk);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   L.hdr = take(sizeof(Header));

@@ -59,7 +59,7 @@ cudaError_t launch_deform_mlp_bwd(const GaussArgs& a, const GaussBwdArgs& b, flo
 
 // Integer stage: binning of projected Gaussians into tile lists.
 struct BinArgs {
-  int P, ntiles, tiles_x, pblocks, bblocks;
+  int P, ntiles, tiles_x, pblocks, bchunk, bblocks;
   int64_t cap;
   const ushort4* rect;
   const uint32_t* touched;
