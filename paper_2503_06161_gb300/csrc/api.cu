@@ -164,10 +164,7 @@ BinArgs bin_args(const Layout& L, void* ws) {
 
 // Clears the per-call state: header, histograms, look-back words, ranges.
 fe_status clear_state(const Layout& L, void* ws, cudaStream_t st) {
-  FE_TRY_CUDA(cudaMemsetAsync(at<char>(ws, L.hdr), 0, sizeof(Header), st));
-  FE_TRY_CUDA(cudaMemsetAsync(at<char>(ws, L.hist), 0, (4 + 3) * 256 * 4, st));
-  FE_TRY_CUDA(cudaMemsetAsync(at<char>(ws, L.status), 0, L.status_words * 4, st));
-  FE_TRY_CUDA(cudaMemsetAsync(at<char>(ws, L.ranges), 0, (size_t)L.ntiles * 8, st));
+  FE_TRY_CUDA(cudaMemsetAsync(at<char>(ws, L.hdr), 0, L.cleared, st));
   return FE_OK;
 }
 

@@ -63,6 +63,8 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* s_warp
 // Global digit histograms of the depth keys (all four passes at once).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads) depth_hist_kernel(const uint32_t* __restrict__ keys, int n, uint32_t* hist) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ uint32_t s[4][256];
   for (int i = threadIdx.x; i < 4 * 256; i += kThreads) (&s[0][0])[i] = 0;
   __syncthreads();
@@ -104,6 +106,8 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* __re
                                                             const uint32_t* n_dev, int64_t n_cap, int shift,
                                                             const uint32_t* __restrict__ hist, uint32_t* status,
                                                             uint32_t* ticket, uint32_t* err) {
+  grid_dep_wait();
+  grid_dep_launch();
   constexpr int CHUNK = kThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PassSmem<ITEMS>& sm = *reinterpret_cast<PassSmem<ITEMS>*>(smem_raw);
@@ -276,6 +280,8 @@ struct CountArgs {
 };
 
 __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) {
+  grid_dep_wait();
+  grid_dep_launch();
   extern __shared__ uint32_t s_cnt[];  // [ntiles]
   __shared__ uint32_t s_scan[8];
   __shared__ uint32_t s_ticket;
@@ -339,6 +345,8 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
 // Step 3: in-place exclusive scan of the (tile, block) table, tile-major.
 __global__ void __launch_bounds__(kThreads) table_scan_kernel(uint32_t* table, int64_t n, uint64_t* status,
                                                              uint32_t* ticket, uint32_t* err) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ uint32_t s_scan[8];
   __shared__ uint32_t s_ticket;
   __shared__ uint64_t s_prefix;
@@ -401,6 +409,8 @@ __host__ __device__ constexpr size_t scatter_smem(int ntiles) { return (size_t)n
 
 template <int NT>
 __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
+  grid_dep_wait();
+  grid_dep_launch();
   extern __shared__ __align__(16) uint32_t s_dyn[];
   uint4* s_mask = reinterpret_cast<uint4*>(s_dyn);  // [ntiles]
   uint32_t* s_word = s_dyn;                         // the same, [ntiles][4]
@@ -533,20 +543,18 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   uint64_t* status_count = reinterpret_cast<uint64_t*>(b.status + (size_t)pblocks * 256 * 4);
   uint64_t* status_table = status_count + bblocks;
   // 1. depth sort (values: Gaussian ids)
-  depth_hist_kernel<<<pblocks, kThreads, 0, st>>>(b.dkey[0], P, b.hist);
+  if ((e = launch_pdl(depth_hist_kernel, pblocks, kThreads, 0, st, (const uint32_t*)b.dkey[0], P, b.hist)) != cudaSuccess)
+    return e;
   int cur = 0;
   for (int p = 0; p < 4; ++p) {
-    if (p == 0)
-      onesweep_kernel<true, kPItems><<<pblocks, kThreads, ppass_smem, st>>>(
-          b.dkey[cur], nullptr, b.dkey[cur ^ 1], b.dval[cur ^ 1], nullptr, P, 8 * p, b.hist + 256 * p,
-          status_depth + (size_t)p * pblocks * 256, hdr->ticket + kTicketDepth0 + p, &hdr->err);
-    else
-      onesweep_kernel<false, kPItems><<<pblocks, kThreads, ppass_smem, st>>>(
-          b.dkey[cur], b.dval[cur], b.dkey[cur ^ 1], b.dval[cur ^ 1], nullptr, P, 8 * p, b.hist + 256 * p,
-          status_depth + (size_t)p * pblocks * 256, hdr->ticket + kTicketDepth0 + p, &hdr->err);
+    e = launch_pdl(p == 0 ? onesweep_kernel<true, kPItems> : onesweep_kernel<false, kPItems>, pblocks, kThreads, ppass_smem,
+                   st, (const uint32_t*)b.dkey[cur], p == 0 ? (const uint32_t*)nullptr : (const uint32_t*)b.dval[cur],
+                   b.dkey[cur ^ 1], b.dval[cur ^ 1], (const uint32_t*)nullptr, (int64_t)P, 8 * p,
+                   (const uint32_t*)(b.hist + 256 * p), status_depth + (size_t)p * pblocks * 256,
+                   hdr->ticket + kTicketDepth0 + p, &hdr->err);
+    if (e != cudaSuccess) return e;
     cur ^= 1;
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // 2. tiles_touched scan + per-block tile counts
   CountArgs ca;
   ca.P = P;
@@ -566,13 +574,12 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   ca.hdr = hdr;
   const size_t count_smem = (size_t)b.ntiles * 4;
   cudaFuncSetAttribute(bin_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)count_smem);
-  bin_count_kernel<<<bblocks, kThreads, count_smem, st>>>(ca);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_pdl(bin_count_kernel, bblocks, kThreads, count_smem, st, ca)) != cudaSuccess) return e;
   // 3. scan of the (tile, block) table
   const int64_t tn = (int64_t)b.ntiles * bblocks;
-  table_scan_kernel<<<ceil_div(tn, kPChunk), kThreads, 0, st>>>(b.table, tn, status_table,
-                                                                hdr->ticket + kTicketTable, &hdr->err);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = launch_pdl(table_scan_kernel, ceil_div(tn, kPChunk), kThreads, 0, st, b.table, tn, status_table,
+                 hdr->ticket + kTicketTable, &hdr->err);
+  if (e != cudaSuccess) return e;
   // 4. scatter into the final list
   ScatterArgs sa;
   sa.P = P;
@@ -590,14 +597,10 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   sa.ranges = b.ranges;
   sa.hdr = hdr;
   const size_t smem = scatter_smem(b.ntiles);
-  if (b.ntiles <= kScatTiles) {
-    cudaFuncSetAttribute(bin_scatter_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    bin_scatter_kernel<512><<<bblocks, 512, smem, st>>>(sa);
-  } else {
-    cudaFuncSetAttribute(bin_scatter_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    bin_scatter_kernel<1024><<<bblocks, 1024, smem, st>>>(sa);
-  }
-  return cudaGetLastError();
+  const int nt = b.ntiles <= kScatTiles ? 512 : 1024;
+  auto scat = nt == 512 ? bin_scatter_kernel<512> : bin_scatter_kernel<1024>;
+  cudaFuncSetAttribute(scat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return launch_pdl(scat, bblocks, nt, smem, st, sa);
 }
 
 // ---------------------------------------------------------------------------

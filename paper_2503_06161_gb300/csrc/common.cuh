@@ -110,7 +110,7 @@ struct Layout {
   bool with_backward;
   size_t hdr, rec, rect, touched, dkey[2], dval[2], offs, offs_by_gid, sorted, table;
   size_t status, hist, ranges, tfinal, ncontrib, partials, pflags, cmask, dstate, fsplit, ddstate, psum;
-  size_t status_words, table_blocks;
+  size_t status_words, table_blocks, cleared;
   size_t total;
 };
 
@@ -134,7 +134,17 @@ inline Layout make_layout(int P, int D, int W, int H, int tw, int th, int64_t ca
   L.bblocks = ceil_div((int64_t)Pn, L.bchunk);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
+  const size_t table_n = (size_t)L.ntiles * L.bblocks;
+  L.table_blocks = (size_t)ceil_div((int64_t)(table_n > 0 ? table_n : 1), kPChunk);
+  // Look-back words: 4 depth passes (u32 per digit per block), then u64 per
+  // block of the tiles_touched scan and of the table scan.
+  L.status_words = (size_t)L.pblocks * 256 * 4 + 2 * (size_t)L.bblocks + 2 * L.table_blocks;
+  // What a forward clears lies together at the start (one memset).
   L.hdr = take(sizeof(Header));
+  L.hist = take((4 + 3) * 256 * 4);
+  L.status = take(L.status_words * 4);
+  L.ranges = take((size_t)L.ntiles * 8);
+  L.cleared = off;
   L.rec = take(Pn * kRec * 4);
   L.rect = take(Pn * 8);
   L.touched = take(Pn * 4);
@@ -143,15 +153,7 @@ inline Layout make_layout(int P, int D, int W, int H, int tw, int th, int64_t ca
   L.offs = take((Pn + 1) * 4);
   L.offs_by_gid = take(Pn * 4);
   L.sorted = take(Kn * 8);
-  const size_t table_n = (size_t)L.ntiles * L.bblocks;
   L.table = take(table_n * 4);
-  L.table_blocks = (size_t)ceil_div((int64_t)(table_n > 0 ? table_n : 1), kPChunk);
-  // Look-back words: 4 depth passes (u32 per digit per block), then u64 per
-  // block of the tiles_touched scan and of the table scan.
-  L.status_words = (size_t)L.pblocks * 256 * 4 + 2 * (size_t)L.bblocks + 2 * L.table_blocks;
-  L.status = take(L.status_words * 4);
-  L.hist = take((4 + 3) * 256 * 4);
-  L.ranges = take((size_t)L.ntiles * 8);
   L.tfinal = take((size_t)W * H * 4);
   L.ncontrib = take((size_t)W * H * 4);
   // Deformation state (offsets + MLP unit masks) and the HexPlane features
@@ -330,6 +332,36 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int li
   for (int i = 0; i < limit; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
+}
+
+
+// ---------------------------------------------------------------------------
+// Programmatic dependent launch.  The kernels of a pass are a chain of short
+// launches; each is launched so that it may start while the one before it
+// drains, orders itself with grid_dep_wait() before it touches memory that an
+// earlier kernel writes, and only then lets its own successor start.  So when
+// a kernel runs at all, every kernel but its direct predecessor has
+// completed: memory that the predecessor does not write (weights, parameters)
+// may be read ahead of the wait.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// A launch that may start while the previous kernel of the stream finishes
+// (programmatic stream serialization).
+template <typename... Params, typename... Args>
+cudaError_t launch_pdl(void (*k)(Params...), int grid, int block, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
 }  // namespace fe

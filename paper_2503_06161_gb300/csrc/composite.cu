@@ -348,6 +348,8 @@ __global__ void __launch_bounds__(kThreads, D <= 32 ? 3 : (D <= 64 ? 2 : 1)) com
   stage_init(s_bar);
   if (threadIdx.x == 0) s_abort[0] = s_abort[1] = 0;
   __syncthreads();
+  grid_dep_wait();
+  grid_dep_launch();
   StageState stg{{0u, 0u}, false};
   fwd_tile<D, B, kCount>(a, blockIdx.x, smem, s_bar, s_abort, stg);
 }
@@ -369,6 +371,8 @@ __global__ void __launch_bounds__(kThreads, D <= 32 ? 3 : (D <= 64 ? 2 : 1))
   __shared__ __align__(8) uint64_t s_bar[2];
   __shared__ int s_abort[2], s_item;
   stage_init(s_bar);
+  grid_dep_wait();
+  grid_dep_launch();
   StageState stg{{0u, 0u}, false};
   for (;;) {
     // Every thread is past the previous tile (its drain ended in a barrier).
@@ -936,6 +940,8 @@ __global__ void __launch_bounds__(kThreads, D <= 32 ? 2 : 1) composite_bwd_kerne
   stage_init(s_bar);
   if (threadIdx.x == 0) s_abort[0] = s_abort[1] = 0;
   __syncthreads();
+  grid_dep_wait();
+  grid_dep_launch();
   StageState stg{{0u, 0u}, false};
   bwd_tile<D>(a, blockIdx.x, smem, s_bar, s_abort, stg);
 }
@@ -948,6 +954,8 @@ __global__ void __launch_bounds__(kThreads, D <= 32 ? 2 : 1)
   __shared__ __align__(8) uint64_t s_bar[2];
   __shared__ int s_abort[2], s_item;
   stage_init(s_bar);
+  grid_dep_wait();
+  grid_dep_launch();
   StageState stg{{0u, 0u}, false};
   for (;;) {
     if (threadIdx.x == 0) {
@@ -967,8 +975,7 @@ cudaError_t launch_fwd_t(const CompositeArgs& a, cudaStream_t st) {
   const size_t smem = fwd_smem_bytes(B, D, a.feat_bf16);
   auto k = composite_fwd_kernel<D, B, kCount>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k<<<a.ntiles, kThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k, a.ntiles, kThreads, smem, st, a);
 }
 
 // Batch sizes: 32, 64, 128 Gaussians (128 only up to D = 64); the counting
@@ -992,8 +999,7 @@ cudaError_t launch_bwd_t(const CompositeArgs& a, cudaStream_t st) {
   const size_t smem = BwdCfg<D>::smem_bytes(a.feat_bf16);
   auto k = composite_bwd_kernel<D>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k<<<a.ntiles, kThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k, a.ntiles, kThreads, smem, st, a);
 }
 
 // Grid of a persistent launch: as many blocks as fit on the GPU at once
@@ -1019,8 +1025,7 @@ cudaError_t launch_fwd_batch_t(const BatchCompositeArgs& b, int bf16, cudaStream
   int grid = 1;
   if (e == cudaSuccess) e = persistent_grid(k, smem, b.nitems, grid);
   if (e != cudaSuccess) return e;
-  k<<<grid, kThreads, smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kThreads, smem, st, b);
 }
 
 template <int D>
@@ -1044,8 +1049,7 @@ cudaError_t launch_bwd_batch_t(const BatchCompositeArgs& b, int bf16, cudaStream
   int grid = 1;
   if (e == cudaSuccess) e = persistent_grid(k, smem, b.nitems, grid);
   if (e != cudaSuccess) return e;
-  k<<<grid, kThreads, smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kThreads, smem, st, b);
 }
 
 // Wide features run as several passes over `width` channels each (part h of

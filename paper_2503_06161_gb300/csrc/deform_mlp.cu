@@ -183,6 +183,9 @@ __global__ void __launch_bounds__(kMlpThreads, 2)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     tc_fence_before();
   }
+  // The weights (above) are no earlier kernel of the pass's output.
+  grid_dep_wait();
+  grid_dep_launch();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
@@ -411,6 +414,9 @@ __global__ void __launch_bounds__(kMlpBwdThreads, 2) deform_mlp_bwd_kernel(const
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     tc_fence_before();
   }
+  // The weights (above) are no earlier kernel of the pass's output.
+  grid_dep_wait();
+  grid_dep_launch();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
@@ -569,8 +575,7 @@ cudaError_t launch_mlp_bwd_t(const GaussArgs& g, const GaussBwdArgs& b, float* d
   auto k = deform_mlp_bwd_kernel<C>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::launch_bytes);
   if (e != cudaSuccess) return e;
-  k<<<grid, kMlpBwdThreads, K::launch_bytes, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kMlpBwdThreads, K::launch_bytes, st, a);
 }
 
 template <int C>
@@ -597,8 +602,7 @@ cudaError_t launch_mlp_t(const GaussArgs& g, cudaStream_t st) {
   auto k = deform_mlp_kernel<C>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::launch_bytes);
   if (e != cudaSuccess) return e;
-  k<<<grid, kMlpThreads, K::launch_bytes, st>>>(m[0], m[1], m[2], a);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, kMlpThreads, K::launch_bytes, st, m[0], m[1], m[2], a);
 }
 
 }  // namespace

@@ -304,6 +304,8 @@ __device__ __forceinline__ void project(const GaussArgs& a, int g, const float d
 // them shuffles and 4-byte loads); 1,500 Gaussians: 3 us instead of 25.
 template <int C>
 __global__ void __launch_bounds__(kThreads) hexplane_split_kernel(const GaussArgs a) {
+  grid_dep_wait();
+  grid_dep_launch();
   constexpr int LG = gather_lanes<C>();
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   const int g = (int)(tid / LG), q = (int)(tid % LG);
@@ -361,6 +363,8 @@ __device__ __forceinline__ void deform_delta(const GaussArgs& a, int g, float de
 }
 
 __global__ void __launch_bounds__(kThreads, 2) gauss_fwd_kernel(const GaussArgs a) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int g = blockIdx.x * kThreads + threadIdx.x;
   bool vis = false;
   if (g < a.P) {
@@ -434,6 +438,8 @@ __host__ __device__ constexpr int ranks_per_warp(int D) { return (partial_stride
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 3) partial_reduce_kernel(const GaussBwdArgs b, int P) {
+  grid_dep_wait();
+  grid_dep_launch();
   constexpr int NP = partial_stride(D);
   constexpr int NQ = (NP + 31) / 32;  // columns per lane
   constexpr int RG = NQ <= 2 ? 16 : (NQ <= 4 ? 8 : 4);  // rows in flight
@@ -530,6 +536,8 @@ __global__ void __launch_bounds__(kThreads, 3) partial_reduce_kernel(const Gauss
 // path through the HexPlane grid is added by gauss_bwd_deform_kernel from
 // dd = d L / d delta stored per Gaussian.
 __global__ void __launch_bounds__(kThreads, 2) gauss_bwd_proj_kernel(const GaussArgs a, const GaussBwdArgs b) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int g = blockIdx.x * kThreads + threadIdx.x;
   if (g >= a.P) return;
   float acc[kPartialScalars + 2];
@@ -720,6 +728,8 @@ __global__ void __launch_bounds__(kThreads, 2) gauss_bwd_proj_kernel(const Gauss
 template <int C>
 __global__ void __launch_bounds__(kThreads, 2) gauss_bwd_deform_kernel(const GaussArgs a, const GaussBwdArgs b,
                                                                      const float* __restrict__ df_all) {
+  grid_dep_wait();
+  grid_dep_launch();
   constexpr int LG = gather_lanes<C>();
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   const int g = (int)(tid / LG), q = (int)(tid % LG);
@@ -789,8 +799,7 @@ static int gather_blocks(int P) { return ceil_div((int64_t)P * gather_lanes<C>()
 
 template <int C>
 static cudaError_t launch_split_t(const GaussArgs& a, cudaStream_t st) {
-  hexplane_split_kernel<C><<<gather_blocks<C>(a.P), kThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(hexplane_split_kernel<C>, gather_blocks<C>(a.P), kThreads, 0, st, a);
 }
 
 // Deformed scenes: HexPlane features (split), the MLP on the tensor cores,
@@ -802,8 +811,7 @@ cudaError_t launch_gauss_fwd(const GaussArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     if ((e = launch_deform_mlp(a, st)) != cudaSuccess) return e;
   }
-  gauss_fwd_kernel<<<ceil_div(a.P, kThreads), kThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(gauss_fwd_kernel, ceil_div(a.P, kThreads), kThreads, 0, st, a);
 }
 
 // The MLP reverse on the tensor cores writes dL/df into the region of the
@@ -814,8 +822,7 @@ static cudaError_t launch_bwd_deform_t(const GaussArgs& a, const GaussBwdArgs& b
   float* df = reinterpret_cast<float*>(a.fsplit);
   cudaError_t e = launch_deform_mlp_bwd(a, b, df, st);
   if (e != cudaSuccess) return e;
-  gauss_bwd_deform_kernel<C><<<gather_blocks<C>(a.P), kThreads, 0, st>>>(a, b, df);
-  return cudaGetLastError();
+  return launch_pdl(gauss_bwd_deform_kernel<C>, gather_blocks<C>(a.P), kThreads, 0, st, a, b, (const float*)df);
 }
 
 cudaError_t launch_gauss_bwd(const GaussArgs& a, const GaussBwdArgs& b, cudaStream_t st, cudaEvent_t mid) {
@@ -823,19 +830,18 @@ cudaError_t launch_gauss_bwd(const GaussArgs& a, const GaussBwdArgs& b, cudaStre
   const int gpw = ranks_per_warp(b.D);
   const int64_t nthreads = ((int64_t)a.P + gpw - 1) / gpw * 32;  // a warp per gpw depth ranks
   const int nblk = (int)((nthreads + kThreads - 1) / kThreads);
+  cudaError_t e;
   switch (b.D) {
-    case 16: partial_reduce_kernel<16><<<nblk, kThreads, 0, st>>>(b, a.P); break;
-    case 32: partial_reduce_kernel<32><<<nblk, kThreads, 0, st>>>(b, a.P); break;
-    case 64: partial_reduce_kernel<64><<<nblk, kThreads, 0, st>>>(b, a.P); break;
-    case 128: partial_reduce_kernel<128><<<nblk, kThreads, 0, st>>>(b, a.P); break;
-    case 256: partial_reduce_kernel<256><<<nblk, kThreads, 0, st>>>(b, a.P); break;
+    case 16: e = launch_pdl(partial_reduce_kernel<16>, nblk, kThreads, 0, st, b, a.P); break;
+    case 32: e = launch_pdl(partial_reduce_kernel<32>, nblk, kThreads, 0, st, b, a.P); break;
+    case 64: e = launch_pdl(partial_reduce_kernel<64>, nblk, kThreads, 0, st, b, a.P); break;
+    case 128: e = launch_pdl(partial_reduce_kernel<128>, nblk, kThreads, 0, st, b, a.P); break;
+    case 256: e = launch_pdl(partial_reduce_kernel<256>, nblk, kThreads, 0, st, b, a.P); break;
     default: return cudaErrorInvalidValue;
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (mid && (e = cudaEventRecord(mid, st)) != cudaSuccess) return e;
-  gauss_bwd_proj_kernel<<<ceil_div(a.P, kThreads), kThreads, 0, st>>>(a, b);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_pdl(gauss_bwd_proj_kernel, ceil_div(a.P, kThreads), kThreads, 0, st, a, b)) != cudaSuccess) return e;
   if (!a.has_deform) return cudaSuccess;
   if (a.C == 32) return launch_bwd_deform_t<32>(a, b, st);
   if (a.C == 64) return launch_bwd_deform_t<64>(a, b, st);

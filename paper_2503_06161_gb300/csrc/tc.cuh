@@ -1,7 +1,7 @@
 // Helpers shared by the tcgen05 kernels: shared-memory and instruction
 // descriptors of kind::f16 (BF16 operands, FP32 accumulators), tensor-core
 // issue and commit, tensor-memory loads, TMA tensor loads and stores, and
-// the host-side tensor maps and dependent launches.
+// the host-side tensor maps.
 #pragma once
 #include <cuda.h>
 
@@ -112,12 +112,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[32]) {
       : "memory");
 }
 
-// Programmatic dependent launch: wait until the kernels this one may have
-// started beside have finished (their memory visible), and let the next
-// kernel of the stream start its set-up while this one runs.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Non-suspending poll (the tensor-core thread spins: its waits are on the
 // critical path of every tile).
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
@@ -169,24 +163,6 @@ inline int num_sms() {
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 0;
   return n;
-}
-
-// A launch that may start while the previous kernel of the stream finishes
-// (programmatic stream serialization); the kernel orders itself with
-// griddepcontrol.wait.
-template <typename... Params, typename... Args>
-cudaError_t launch_pdl(void (*k)(Params...), int grid, int block, size_t smem, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
 }  // namespace tc_host
