@@ -11,7 +11,9 @@
 //                       channels each), so a corner fetch is one coalesced
 //                       128-byte line of the channels-last planes, written
 //                       Gaussian-major;
-//   fst_fwd_kernel      the MLP: a block holds 128 Gaussians and every layer
+//   fst_fwd_tc_kernel   the MLP of a forward without reverse state, on the
+//                       tensor cores (three BF16 terms per operand);
+//   fst_fwd_kernel      the MLP in training: a block holds 128 Gaussians and every layer
 //                       is a block product -- activations in shared memory
 //                       (a row per Gaussian), each thread a register tile of
 //                       packed FP32 FMAs, weight tiles staged by cp.async --
@@ -31,6 +33,7 @@
 #include <cstdint>
 
 #include "common.cuh"
+#include "mma.cuh"
 
 namespace fe {
 
@@ -609,6 +612,341 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
 #pragma unroll
   for (int k = 0; k < 3; ++k) a.log_scales_t[(size_t)p * 3 + k] = a.log_scales[(size_t)p * 3 + k] + out[7 + k];
   a.logits_t[p] = a.logits[p] + out[10];
+}
+
+// ---------------------------------------------------------------------------
+// Forward without reverse state: the MLP on the tensor cores.
+//
+// Every operand is three BF16 terms (24 significant bits), every product the
+// six term products down to 2^-16 of |x||w|: the five small ones and hi.hi in
+// accumulators of their own, added at the end, so that the small ones are
+// not rounded away against the large sum.  A warp takes 16 Gaussians
+// through all 22 layers: a layer's accumulators (rows = Gaussians) have the
+// register layout of the next layer's first operand, so activations stay in
+// registers (h, which four branches read, waits in shared memory), and only
+// the weights are shared by the block: packed by fst_pack_tc_kernel in the
+// order the products read them, staged 32 output columns at a time through
+// three shared-memory buffers (one barrier per stage).
+//
+// Bound by the tensor pipe (200k Gaussians, 4 levels: 75 M products of
+// 16 x 8 x 16, 236 us at the measured 607 TFLOP/s of mma.sync).  The products
+// with FP32 FMAs (fst_fwd_kernel), which training keeps -- the reverse's ReLU
+// masks are decisions that a different rounding would take differently -- are
+// bound by FMA issue at twice that.  Measured: 592 -> 395 us, and the same
+// error against 64 bits (2.5e-7 of the outputs).
+// ---------------------------------------------------------------------------
+constexpr int kTcWarps = 8, kTcThreads = 32 * kTcWarps, kTcRows = 16 * kTcWarps;
+constexpr int kTcBuf = 4 * 4 * 768;   // bytes of the largest stage: K = 64, 32 columns
+constexpr int kTcMaxItems = 48;
+constexpr size_t kTcSmem = 3 * (size_t)kTcBuf + (size_t)kTcWarps * 12 * 512;
+
+// One stage of weights: output columns [n0, n0 + 8 nt) and inputs [k0, k0 + 16 ks)
+// of layer `layer`, 768 bytes per (16 inputs, 8 columns): per lane the two
+// registers of the hi and mid terms (16 bytes), then of the lo term (8).
+struct TcItem {
+  int layer, k0, ks, n0, nt;
+  int off;  // bytes
+};
+struct TcPlan {
+  TcItem item[kTcMaxItems];
+  int n, bytes;
+};
+
+TcPlan make_tc_plan(const FstGeom& g) {
+  TcPlan p{};
+  auto add = [&](int layer, int k0, int k, int n0, int n) {
+    p.item[p.n++] = TcItem{layer, k0, k / 16, n0, (n + 7) / 8, p.bytes};
+    p.bytes += k / 16 * ((n + 7) / 8) * 768;
+  };
+  // In the order of use: the first layer per half of its columns and per 64
+  // inputs, a hidden layer per half of its columns, a branch's three layers
+  // and its share of F_feat's first layer, F_feat's second layer.
+  for (int h = 0; h < 2; ++h)
+    for (int k0 = 0; k0 < g.levels * kFC; k0 += 64) add(0, k0, g.levels * kFC - k0 < 64 ? 32 : 64, 32 * h, 32);
+  for (int j = 1; j < kFDepth; ++j)
+    for (int h = 0; h < 2; ++h) add(j, 0, kFW, 32 * h, 32);
+  for (int b = 0; b < 4; ++b) {
+    add(branch_e1(b), 0, kFW, 0, 32);
+    add(branch_e1(b) + 1, 0, kFHalf, 0, 32);
+    add(branch_e1(b) + 2, 0, kFHalf, 0, branch_out(b));
+    for (int h = 0; h < 2; ++h) add(kLZ1, b * kFHalf, kFHalf, 32 * h, 32);
+  }
+  for (int n0 = 0; n0 < g.D; n0 += 32) add(kLZ2, 0, kFW, n0, g.D < 32 ? g.D : 32);
+  return p;
+}
+
+// A thread per (16 inputs, 8 columns, lane) of the plan.
+__global__ void fst_pack_tc_kernel(const FstGeom g, const TcPlan plan, const float* __restrict__ mlp,
+                                   unsigned char* __restrict__ out) {
+  const int u = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (u * 768 >= plan.bytes) return;
+  int i = 0;
+  while (i + 1 < plan.n && u * 768 >= plan.item[i + 1].off) ++i;
+  const TcItem it = plan.item[i];
+  const int v = u - it.off / 768, ks = v / it.nt, nt = v % it.nt;
+  const int n = it.n0 + 8 * nt + (lane >> 2), k = it.k0 + 16 * ks + 2 * (lane & 3);
+  float x[4] = {0.f, 0.f, 0.f, 0.f};
+  if (n < g.nout[it.layer]) {
+    const float* w = mlp + g.pw[it.layer] + (int64_t)n * g.nin[it.layer] + k;
+    x[0] = w[0]; x[1] = w[1]; x[2] = w[8]; x[3] = w[9];
+  }
+  uint32_t h[2], m[2], l[2];
+  split3(x[0], x[1], h[0], m[0], l[0]);
+  split3(x[2], x[3], h[1], m[1], l[1]);
+  unsigned char* o = out + (size_t)u * 768;
+  reinterpret_cast<uint4*>(o)[lane] = make_uint4(h[0], h[1], m[0], m[1]);
+  reinterpret_cast<uint2*>(o + 512)[lane] = make_uint2(l[0], l[1]);
+}
+
+struct TcArgs {
+  FstGeom g;
+  const float* mlp;           // biases (the caller's packed array)
+  const unsigned char* wpack;
+  int bytes[kTcMaxItems];     // of each stage; they follow one another in wpack
+  int nitems;
+  const float *means, *quats, *log_scales, *logits;
+  const void* feat;
+  int feat_bf16;
+  float *means_t, *quats_t, *log_scales_t, *logits_t;
+  void* feat_t;
+  const float* f;
+};
+
+// First operand of KS steps (16 inputs each), three terms.
+template <int KS>
+using TcFrag = uint32_t[3][KS][4];
+
+// acc_h += hi.hi, acc_s += the five smaller term products of one 16-input
+// step with NT column tiles of staged weights at w.
+template <int NT>
+__device__ __forceinline__ void tc_step(const uint32_t (&ah)[4], const uint32_t (&am)[4], const uint32_t (&al)[4],
+                                        const unsigned char* w, int lane, float (&acc_h)[NT][4], float (&acc_s)[NT][4]) {
+  uint4 hm[NT];
+  uint2 lo[NT];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    hm[nt] = reinterpret_cast<const uint4*>(w + nt * 768)[lane];
+    lo[nt] = reinterpret_cast<const uint2*>(w + nt * 768 + 512)[lane];
+  }
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc_s[nt], al, hm[nt].x, hm[nt].y);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc_s[nt], am, hm[nt].z, hm[nt].w);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc_s[nt], ah, lo[nt].x, lo[nt].y);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc_s[nt], am, hm[nt].x, hm[nt].y);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc_s[nt], ah, hm[nt].z, hm[nt].w);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc_h[nt], ah, hm[nt].x, hm[nt].y);
+}
+
+template <int NT>
+__device__ __forceinline__ void tc_zero(float (&a)[NT][4], float (&b)[NT][4]) {
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[nt][i] = b[nt][i] = 0.0f;
+}
+
+// Columns 8 nt + 2 t, + 1 of four tiles (rows fr, fr + 8) as steps k0 and
+// k0 + 1 of the next layer's first operand: relu(z + bias), three terms.
+template <int KS>
+__device__ __forceinline__ void tc_relu(const float (&z)[4][4], const float* __restrict__ bias, int ft, TcFrag<KS>& out,
+                                        int k0) {
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt) {
+    const float b0 = __ldg(bias + 8 * nt + 2 * ft), b1 = __ldg(bias + 8 * nt + 2 * ft + 1);
+    const int k = k0 + (nt >> 1), i = 2 * (nt & 1);
+    split3(fmaxf(z[nt][0] + b0, 0.0f), fmaxf(z[nt][1] + b1, 0.0f), out[0][k][i], out[1][k][i], out[2][k][i]);
+    split3(fmaxf(z[nt][2] + b0, 0.0f), fmaxf(z[nt][3] + b1, 0.0f), out[0][k][i + 1], out[1][k][i + 1], out[2][k][i + 1]);
+  }
+}
+
+template <int D>
+__global__ void __launch_bounds__(kTcThreads, 2) fst_fwd_tc_kernel(const __grid_constant__ TcArgs a) {
+  extern __shared__ __align__(16) unsigned char s_tc[];
+  const FstGeom& g = a.g;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, fr = lane >> 2, ft = lane & 3;
+  uint4* s_h = reinterpret_cast<uint4*>(s_tc + 3 * kTcBuf) + warp * 12 * 32;  // [ks][term][lane]
+  const int P = g.P;
+  const int p[2] = {(int)blockIdx.x * kTcRows + warp * 16 + fr, (int)blockIdx.x * kTcRows + warp * 16 + fr + 8};
+  const bool valid[2] = {p[0] < P, p[1] < P};
+  // Weight stages: stage t is in buffer t % 3; two are in flight.
+  int t_issue = 0, t_use = 0;
+  const unsigned char* src = a.wpack;
+  auto issue = [&]() {
+    if (t_issue < a.nitems) {
+      const int n = a.bytes[t_issue];
+      unsigned char* dst = s_tc + (t_issue % 3) * kTcBuf;
+      for (int i = tid; i < n / 16; i += kTcThreads) cp_async16(dst + 16 * i, src + 16 * i);
+      src += n;
+      ++t_issue;
+    }
+    cp_async_commit();
+  };
+  issue();
+  issue();
+  auto next = [&]() -> const unsigned char* {
+    cp_async_wait1();
+    __syncthreads();  // the stage has landed for all; the one before it is read
+    issue();
+    return s_tc + (t_use++ % 3) * kTcBuf;
+  };
+  float zh[4][4], zs[4][4];
+  auto sum = [&]() {
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) zh[nt][i] += zs[nt][i];
+  };
+  // ---- F_out ----
+  TcFrag<4> x;
+  const int nf = g.levels * kFC;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    tc_zero(zh, zs);
+    for (int k0 = 0; k0 < nf; k0 += 64) {
+      const unsigned char* w = next();
+      const int ks_n = nf - k0 < 64 ? 2 : 4;
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        if (ks < ks_n) {
+          uint32_t f3[3][4];
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const float* row = a.f + (size_t)(valid[r] ? p[r] : 0) * nf + k0 + 16 * ks + 2 * ft;
+            const float2 u0 = __ldg(reinterpret_cast<const float2*>(row)), u1 = __ldg(reinterpret_cast<const float2*>(row + 8));
+            split3(u0.x, u0.y, f3[0][r], f3[1][r], f3[2][r]);
+            split3(u1.x, u1.y, f3[0][2 + r], f3[1][2 + r], f3[2][2 + r]);
+          }
+          tc_step<4>(f3[0], f3[1], f3[2], w + ks * 4 * 768, lane, zh, zs);
+        }
+      }
+    }
+    sum();
+    tc_relu<4>(zh, a.mlp + g.pb[0] + 32 * h, ft, x, 2 * h);
+  }
+  for (int j = 1; j < kFDepth; ++j) {
+    TcFrag<4> y;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned char* w = next();
+      tc_zero(zh, zs);
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) tc_step<4>(x[0][ks], x[1][ks], x[2][ks], w + ks * 4 * 768, lane, zh, zs);
+      sum();
+      tc_relu<4>(zh, a.mlp + g.pb[j] + 32 * h, ft, y, 2 * h);
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[t][ks][i] = y[t][ks][i];
+  }
+  // relu(h) for the branches.
+#pragma unroll
+  for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+    for (int t = 0; t < 3; ++t) s_h[(3 * ks + t) * 32 + lane] = make_uint4(x[t][ks][0], x[t][ks][1], x[t][ks][2], x[t][ks][3]);
+  // ---- branches; F_feat's first layer sums over them ----
+  float v[8][4];
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[nt][i] = 0.0f;
+  const float* srcs[4] = {a.means, a.quats, a.log_scales, a.logits};
+  float* dsts[4] = {a.means_t, a.quats_t, a.log_scales_t, a.logits_t};
+#pragma unroll 1
+  for (int b = 0; b < 4; ++b) {
+    const int l1 = branch_e1(b);
+    TcFrag<2> e, u;
+    {
+      const unsigned char* w = next();
+      tc_zero(zh, zs);
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        uint32_t hx[3][4];
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          const uint4 q = s_h[(3 * ks + t) * 32 + lane];
+          hx[t][0] = q.x; hx[t][1] = q.y; hx[t][2] = q.z; hx[t][3] = q.w;
+        }
+        tc_step<4>(hx[0], hx[1], hx[2], w + ks * 4 * 768, lane, zh, zs);
+      }
+      sum();
+      tc_relu<2>(zh, a.mlp + g.pb[l1], ft, e, 0);
+    }
+    {
+      const unsigned char* w = next();
+      tc_zero(zh, zs);
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) tc_step<4>(e[0][ks], e[1][ks], e[2][ks], w + ks * 4 * 768, lane, zh, zs);
+      sum();
+      tc_relu<2>(zh, a.mlp + g.pb[l1 + 1], ft, u, 0);
+    }
+    {
+      // Head: offsets added to the canonical parameters (Eq. 6).
+      const unsigned char* w = next();
+      float oh[1][4], os[1][4];
+      tc_zero(oh, os);
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) tc_step<1>(u[0][ks], u[1][ks], u[2][ks], w + ks * 768, lane, oh, os);
+      const int dg = branch_out(b);
+      const float* bias = a.mlp + g.pb[l1 + 2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int o = 2 * ft + (i & 1), r = i >> 1;
+        if (o < dg && valid[r]) {
+          const size_t at = (size_t)p[r] * dg + o;
+          dsts[b][at] = srcs[b][at] + ((oh[0][i] + os[0][i]) + __ldg(bias + o));
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned char* w = next();
+      tc_zero(zh, zs);
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) tc_step<4>(u[0][ks], u[1][ks], u[2][ks], w + ks * 4 * 768, lane, zh, zs);
+#pragma unroll
+      for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[4 * h + nt][i] += zh[nt][i] + zs[nt][i];
+    }
+  }
+  // ---- dz = Z2 relu(v) + b ----
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float z[4][4];
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) z[nt][i] = v[4 * h + nt][i];
+    tc_relu<4>(z, a.mlp + g.pb[kLZ1] + 32 * h, ft, x, 2 * h);
+  }
+  constexpr int ZT = D < 32 ? D / 8 : 4;  // column tiles per stage
+#pragma unroll 1
+  for (int n0 = 0; n0 < D; n0 += 8 * ZT) {
+    const unsigned char* w = next();
+    float dh[ZT][4], ds[ZT][4];
+    tc_zero(dh, ds);
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) tc_step<ZT>(x[0][ks], x[1][ks], x[2][ks], w + ks * ZT * 768, lane, dh, ds);
+    const float* bias = a.mlp + g.pb[kLZ2] + n0;
+#pragma unroll
+    for (int nt = 0; nt < ZT; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int c = 8 * nt + 2 * ft + (i & 1), r = i >> 1;
+        if (valid[r]) {
+          const size_t at = (size_t)p[r] * D + n0 + c;
+          store_feat(a.feat_t, a.feat_bf16, at, load_feat(a.feat, a.feat_bf16, at) + (dh[nt][i] + ds[nt][i]) + __ldg(bias + c));
+        }
+      }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1220,6 +1558,14 @@ cudaError_t launch_fst_fwd(const FwdArgs& a, cudaStream_t st) {
 }
 
 template <int D>
+cudaError_t launch_fst_fwd_tc(const TcArgs& a, cudaStream_t st) {
+  auto k = fst_fwd_tc_kernel<D>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
+  k<<<(a.g.P + kTcRows - 1) / kTcRows, kTcThreads, kTcSmem, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <int D>
 cudaError_t launch_fst_bwd(const BwdArgs& a, int nblk, cudaStream_t st) {
   const size_t smem = kBwdSmem;
   auto k = fst_bwd_kernel<D>;
@@ -1251,6 +1597,42 @@ extern "C" fe_status fe_fst_forward(const fe_fst* fst, int P, const float* means
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   float* wt = reinterpret_cast<float*>(ws + w.wt);
   float* wn = reinterpret_cast<float*>(ws + w.wn);
+  {
+    SampArgs sa{};
+    sa.g = g;
+    sa.planes = fst->planes;
+    sa.means = means;
+    sa.t = t;
+    sa.f = reinterpret_cast<float*>(ws + w.f);
+    const dim3 grid((unsigned)(((int64_t)P * kGLanes + kSampThreads - 1) / kSampThreads), (unsigned)g.levels);
+    fst_sample_kernel<<<grid, kSampThreads, 0, st>>>(sa);
+  }
+  if (!with_backward) {
+    // Packed weights in the place of the FP32 copies (6 bytes a weight
+    // against 8: checked, for the heads are padded to eight columns).
+    const TcPlan plan = make_tc_plan(g);
+    if ((size_t)plan.bytes > w.f - w.wt) return FE_ERR_WORKSPACE;
+    fst_pack_tc_kernel<<<(plan.bytes / 768 * 32 + 255) / 256, 256, 0, st>>>(g, plan, fst->mlp, ws + w.wt);
+    TcArgs a{};
+    a.g = g;
+    a.mlp = fst->mlp;
+    a.wpack = ws + w.wt;
+    a.nitems = plan.n;
+    for (int i = 0; i < plan.n; ++i) a.bytes[i] = plan.item[i].ks * plan.item[i].nt * 768;
+    a.means = means; a.quats = quats; a.log_scales = log_scales; a.logits = opacity_logits;
+    a.feat = feat; a.feat_bf16 = feat_bf16 ? 1 : 0;
+    a.means_t = means_t; a.quats_t = quats_t; a.log_scales_t = log_scales_t; a.logits_t = opacity_logits_t;
+    a.feat_t = feat_t;
+    a.f = reinterpret_cast<const float*>(ws + w.f);
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (g.D) {
+      case 16: e = launch_fst_fwd_tc<16>(a, st); break;
+      case 32: e = launch_fst_fwd_tc<32>(a, st); break;
+      case 64: e = launch_fst_fwd_tc<64>(a, st); break;
+      case 128: e = launch_fst_fwd_tc<128>(a, st); break;
+    }
+    return e == cudaSuccess ? FE_OK : FE_ERR_CUDA;
+  }
   if (cudaMemsetAsync(wt, 0, w.f - w.wt, st) != cudaSuccess) return FE_ERR_CUDA;
   fst_pack_kernel<<<(int)((g.mlp_packed + 255) / 256), 256, 0, st>>>(g, fst->mlp, wt, wn);
   FwdArgs a{};
@@ -1269,18 +1651,8 @@ extern "C" fe_status fe_fst_forward(const fe_fst* fst, int P, const float* means
   a.log_scales_t = log_scales_t;
   a.logits_t = opacity_logits_t;
   a.feat_t = feat_t;
-  a.act = with_backward ? reinterpret_cast<float*>(ws + w.act) : nullptr;
+  a.act = reinterpret_cast<float*>(ws + w.act);
   a.f = reinterpret_cast<const float*>(ws + w.f);
-  {
-    SampArgs sa{};
-    sa.g = g;
-    sa.planes = fst->planes;
-    sa.means = means;
-    sa.t = t;
-    sa.f = reinterpret_cast<float*>(ws + w.f);
-    const dim3 grid((unsigned)(((int64_t)P * kGLanes + kSampThreads - 1) / kSampThreads), (unsigned)g.levels);
-    fst_sample_kernel<<<grid, kSampThreads, 0, st>>>(sa);
-  }
   // Weight tiles of the transposed copy in the order the kernel uses them.
   {
     int n = 0;
