@@ -182,15 +182,19 @@ def _check(fn: str, rc: int):
         raise FeError(fn, rc)
 
 
+# Addresses and stream handles go to ctypes as plain integers (every argument
+# and struct field they fill is declared c_void_p): a wrapper object for each
+# of the about sixty of a forward and reverse, and a torch Stream object for
+# each call, cost more than a short kernel.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     if stream is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return int(stream.cuda_stream if hasattr(stream, "cuda_stream") else stream)
 
 
 def make_opts(tile=(16, 16), bg=(0.0, 0.0, 0.0), max_dups=0, forward_only=False, accumulate=False, fwd_batch=0,

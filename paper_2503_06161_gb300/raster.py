@@ -219,6 +219,9 @@ class _RenderFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, rast, scene_meta, cam, deform, t, means, log_scales, quats, opacity_logits, sh, feat):
         scene = GaussianScene(means, log_scales, quats, opacity_logits, sh, feat, scene_meta)
+        # An output without an upstream gradient reaches the reverse as None
+        # (taken as zero there), not as a zero tensor filled for the call.
+        ctx.set_materialize_grads(False)
         rgb, depth, alpha, fmap = rast.forward(scene, cam, deform, t)
         ctx.rast, ctx.cam, ctx.deform, ctx.t, ctx.scene = rast, cam, deform, t, scene
         return rgb, depth, alpha, fmap
