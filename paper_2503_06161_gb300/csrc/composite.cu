@@ -22,9 +22,16 @@ namespace fe {
 
 namespace {
 
-// Gaussians per staged batch of the forward; two batches are in flight.
+// Gaussians per staged batch of the forward (two batches are in flight) and
+// blocks per SM.  Most tiles end within the first 200 entries of their list,
+// so at D = 32 batches of 64 land sooner and load less past the end (200k
+// Gaussians, 640 x 512: 170 us, 176 with 128, 182 with 32); at D = 16 two
+// blocks with room for registers beat three (30k, 333 x 251: 66 us against
+// 74), at D = 32 they are even.
 template <int D>
-constexpr int fwd_batch() { return D <= 32 ? 128 : (D <= 64 ? 64 : 32); }
+constexpr int fwd_batch() { return D == 16 ? 128 : (D <= 64 ? 64 : 32); }
+template <int D>
+constexpr int fwd_blocks() { return D == 32 ? 3 : (D <= 64 ? 2 : 1); }
 
 // Bytes of one staged batch: B render records (48 bytes each), then B
 // feature rows in their stored format (fp32 or bf16).
@@ -342,7 +349,7 @@ __device__ __forceinline__ void stage_init(uint64_t* s_bar) {
 
 // One block per tile.
 template <int D, int B, bool kCount>
-__global__ void __launch_bounds__(kThreads, D <= 32 ? 3 : (D <= 64 ? 2 : 1)) composite_fwd_kernel(const CompositeArgs a) {
+__global__ void __launch_bounds__(kThreads, fwd_blocks<D>()) composite_fwd_kernel(const CompositeArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar[2];
   __shared__ int s_abort[2];
@@ -366,7 +373,7 @@ __device__ __forceinline__ int batch_view(const BatchCompositeArgs& ba, int item
 // items from a device counter until the batch is exhausted (no block waits
 // for another: items are independent).
 template <int D, int B>
-__global__ void __launch_bounds__(kThreads, D <= 32 ? 3 : (D <= 64 ? 2 : 1))
+__global__ void __launch_bounds__(kThreads, fwd_blocks<D>())
     composite_fwd_batch_kernel(const __grid_constant__ BatchCompositeArgs ba) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar[2];
