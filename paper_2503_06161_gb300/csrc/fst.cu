@@ -19,11 +19,10 @@
 //                       packed FP32 FMAs, weight tiles staged by cp.async --
 //                       writing the deformed Gaussians and relu(z) of every
 //                       hidden layer for the reverse;
-//   fst_bwd_kernel      (persistent blocks) per layer the input gradient
-//                       delta W as the same tile product, the ReLU masks from
-//                       the stored relu(z), and the weight gradient
-//                       sum_g delta_g x_g^T as a second block product added
-//                       into the block's own partial; writes d f;
+//   fst_bwd_kernel      (persistent blocks, tensor cores) per layer the input
+//                       gradient delta W, masked by the stored relu(z), and
+//                       the weight gradient sum_g delta_g x_g^T added into
+//                       the block's own partial; writes d f;
 //   fst_hex_bwd_kernel  the HexPlane reverse: plane gradients by vector
 //                       float atomics (the only order-dependent sum of this
 //                       file), the canonical mean's gradient;
@@ -41,8 +40,7 @@ namespace {
 
 constexpr int kFW = 64, kFHalf = 32, kFDepth = 8, kFC = 32, kFMaxL = 4;
 constexpr int kFLayers = kFDepth + 12 + 2;
-constexpr int kFThreads = 128;     // threads of the reverse product kernel
-constexpr int kFM = 128;           // Gaussians per block of the product kernels
+constexpr int kFM = 128;           // Gaussians per block (chunk) of the product kernels
 constexpr int kFwdThreads = 256;   // threads of the forward product kernel
 constexpr int kFRow = 68;  // shared-memory row stride (floats) of the block products
 constexpr int kLZ1 = kFDepth + 12, kLZ2 = kFDepth + 13;
@@ -56,7 +54,7 @@ __host__ __device__ constexpr int pair_b(int k) { return k == 0 ? 1 : (k == 1 ||
 
 struct FstGeom {
   int levels, rs, rt, D, P;
-  int nslots, sf, sz, se1, shg, sv;  // activation slots ([slot][P] float32)
+  int nslots, sz, se1, shg, sv;  // a Gaussian's activations ([P][nslots] float32)
   int nout[kFLayers], nin[kFLayers];
   int64_t pw[kFLayers], pb[kFLayers];  // offsets in the caller's packed array
   int64_t aw[kFLayers], ab[kFLayers];  // offsets in the aligned copies
@@ -112,8 +110,7 @@ bool make_geom(const fe_fst* f, int P, FstGeom& g) {
   }
   for (int k = 0; k < f->levels * 6; ++k)
     if ((int64_t)g.pra[k] * g.prb[k] * kFC > (int64_t)0x7FFFFFFF) return false;  // 32-bit plane indexing
-  g.sf = 0;
-  g.sz = f->levels * kFC;
+  g.sz = 0;
   g.se1 = g.sz + kFDepth * kFW;
   g.shg = g.se1 + 4 * kFHalf;
   g.sv = g.shg + 4 * kFHalf;
@@ -134,18 +131,34 @@ __host__ __device__ int64_t plane_floats(const FstGeom& g) {
 
 // Workspace: header | transposed weights (aligned) | row-major weights
 // (aligned) | f [P][levels*32] | with the reverse: relu activations
-// [nslots][P], F_feat delta [64][P], d f [P][levels*32], per-block partials
-// of the weight gradients [nblk][mlp_aligned].
+// [P][nslots], F_feat delta [P][64], d f [P][levels*32], per-block partials
+// of the weight gradients [nblk][mlp_aligned], the reverse's packed weights.
 constexpr size_t kWsHeader = 256;
 int bwd_blocks(int P) {
-  const int chunks = (P + kFThreads - 1) / kFThreads;
+  const int chunks = (P + kFM - 1) / kFM;
   return chunks < 2 * 152 ? chunks : 2 * 152;
 }
 size_t al256(size_t x) { return (x + 255) / 256 * 256; }
+// The reverse's packed weights (fst_pack_bwd_kernel): byte offset of each
+// layer, 768 bytes per (32-column group, 16 outputs, 8 columns); the heads
+// (at most four outputs) are not packed.
+struct BwdPack {
+  int off[kFLayers + 1], bytes;
+};
+__host__ __device__ constexpr bool is_head(int l) { return l >= kFDepth && l < kLZ1 && (l - kFDepth) % 3 == 2; }
+BwdPack bwd_pack(const FstGeom& g) {
+  BwdPack p{};
+  for (int l = 0; l < kFLayers; ++l) {
+    p.off[l] = p.bytes;
+    if (!is_head(l)) p.bytes += g.nin[l] / 32 * (g.nout[l] / 16) * 4 * 768;
+  }
+  p.off[kFLayers] = p.bytes;
+  return p;
+}
 // acc: with the reverse pass, the exact plane-gradient accumulators, two
 // uint64 arrays (hi, lo) of one entry per plane float (see fixed_add).
 struct WsLayout {
-  size_t wt, wn, f, act, dv, df, part, acc, total;
+  size_t wt, wn, f, act, dv, df, part, wp, acc, total;
 };
 WsLayout ws_layout(const FstGeom& g, int with_backward) {
   WsLayout w{};
@@ -156,7 +169,8 @@ WsLayout ws_layout(const FstGeom& g, int with_backward) {
   w.dv = w.act + (with_backward ? al256((size_t)g.nslots * g.P * 4) : 0);
   w.df = w.dv + (with_backward ? al256((size_t)kFW * g.P * 4) : 0);
   w.part = w.df + (with_backward ? al256((size_t)g.levels * kFC * g.P * 4) : 0);
-  w.acc = w.part + (with_backward ? al256((size_t)bwd_blocks(g.P) * g.mlp_aligned * 4) : 0);
+  w.wp = w.part + (with_backward ? al256((size_t)bwd_blocks(g.P) * g.mlp_aligned * 4) : 0);
+  w.acc = w.wp + (with_backward ? al256((size_t)bwd_pack(g).bytes) : 0);
   w.total = w.acc + (with_backward == 2 ? al256((size_t)plane_floats(g) * 16) : 0);
   return w;
 }
@@ -196,9 +210,6 @@ __global__ void fst_pack_kernel(const FstGeom g, const float* __restrict__ mlp, 
 // its 4 weight slices are one or two wavefronts each (12 wavefronts per
 // 64 packed FMAs at TN = 8), where a warp of 32 rows and one column group
 // took 32 and was bound by them.
-//
-// Reverse (128 threads): thread (mt, nt) = (tid % 16, tid / 16) owns rows
-// mt + 16 r (r < 8) and TN consecutive columns from nt * TN.
 // ---------------------------------------------------------------------------
 template <int TN, int TM = 8>
 __device__ __forceinline__ void tile_zero(float2 (&acc)[TM][TN / 2]) {
@@ -251,11 +262,12 @@ __device__ __forceinline__ void tile_mma(const float* X, int K, const float* B, 
 }
 
 // Layer epilogue of the forward: z = acc + bias; relu(z) -> Y (shared, column
-// offset yc) and optionally -> act slots (valid rows only).  The reverse pass
-// needs only relu(z): it is the next layer's input, and z > 0 iff relu(z) > 0.
+// offset yc) and -> the Gaussians' activation rows (valid rows only).  The
+// reverse pass needs only relu(z): it is the next layer's input, and z > 0 iff
+// relu(z) > 0.
 template <int TN>
 __device__ __forceinline__ void tile_out(const float2 (&acc)[4][TN / 2], const float* __restrict__ bias, int row0,
-                                         int n0, float* act, int P, int slot, int p0, float* Y, int yc) {
+                                         int n0, float* act, int nslots, int P, int slot, int p0, float* Y, int yc) {
   float2 bb[TN / 2];
 #pragma unroll
   for (int c = 0; c < TN / 2; ++c) bb[c] = __ldg(reinterpret_cast<const float2*>(bias + n0) + c);
@@ -268,9 +280,10 @@ __device__ __forceinline__ void tile_out(const float2 (&acc)[4][TN / 2], const f
       z[2 * c] = fmaxf(acc[r][c].x + bb[c].x, 0.0f);
       z[2 * c + 1] = fmaxf(acc[r][c].y + bb[c].y, 0.0f);
     }
-    if (act && p0 + m < P) {
+    if (p0 + m < P) {
+      float4* o = reinterpret_cast<float4*>(act + (size_t)(p0 + m) * nslots + slot + n0);
 #pragma unroll
-      for (int c = 0; c < TN; ++c) act[(size_t)(slot + n0 + c) * P + p0 + m] = z[c];
+      for (int c = 0; c < TN; c += 4) o[c / 4] = make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
     }
 #pragma unroll
     for (int c = 0; c < TN; c += 4)
@@ -278,23 +291,7 @@ __device__ __forceinline__ void tile_out(const float2 (&acc)[4][TN / 2], const f
   }
 }
 
-// Row m of Y (columns [yc, yc + N)) <- rows [slot, slot + N) of the
-// [slot][P] array src at Gaussian p0 + m (zeros past the end), as 4-byte
-// asynchronous copies; complete after cp_async_wait_all() and a barrier.
-__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool valid) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(smem_addr(dst)), "l"(src), "r"(valid ? 4 : 0)
-               : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void rows_async(float* Y, int yc, const float* src, int P, int slot, int p0, int m,
-                                           int ys = kFRow) {
-  const bool valid = p0 + m < P;
-  const float* s0 = src + (size_t)slot * P + (valid ? p0 + m : 0);
-#pragma unroll 16
-  for (int q = 0; q < N; ++q) cp_async4(Y + m * ys + yc + q, s0 + (size_t)q * P, valid);
-}
-
 
 // Weight tiles staged into shared memory with cp.async, two buffers: the
 // tile of the next product is in flight while the current one runs.  (The
@@ -304,8 +301,7 @@ struct WTile {
   int rows, cols, ld;    // copied as [rows][cols] from rows of `ld` floats
 };
 constexpr int kMaxWTiles = 40;
-constexpr int kWBuf = 4096;   // floats per staging buffer (forward)
-constexpr int kWBufR = 2048;  // floats per staging buffer (reverse)
+constexpr int kWBuf = 4096;   // floats per staging buffer
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
@@ -320,12 +316,11 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // Issue the copy of tile t (if any) into buffer t & 1; always commits a
 // group so that "all but the newest group" names tile t - 1.  The caller
 // guarantees no thread still reads buffer t & 1.
-template <int kBuf = kWBuf>
 __device__ __forceinline__ void stage_tile(const WTile* tiles, int ntiles, int t, const float* __restrict__ base,
                                            float* wbuf) {
   if (t < ntiles) {
     const WTile w = tiles[t];
-    float* dst = wbuf + (t & 1) * kBuf;
+    float* dst = wbuf + (t & 1) * kWBuf;
     const int c4 = w.cols / 4, n = w.rows * c4;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       const int r = i / c4, c = i - r * c4;
@@ -336,13 +331,12 @@ __device__ __forceinline__ void stage_tile(const WTile* tiles, int ntiles, int t
 }
 
 // Tile t: start tile t + 1, wait for tile t, make it visible to the block.
-template <int kBuf = kWBuf>
 __device__ __forceinline__ const float* next_tile(const WTile* tiles, int ntiles, int& t, const float* base,
                                                   float* wbuf) {
-  stage_tile<kBuf>(tiles, ntiles, t + 1, base, wbuf);
+  stage_tile(tiles, ntiles, t + 1, base, wbuf);
   cp_async_wait1();
   __syncthreads();
-  const float* w = wbuf + (t & 1) * kBuf;
+  const float* w = wbuf + (t & 1) * kWBuf;
   ++t;
   return w;
 }
@@ -358,7 +352,7 @@ struct FwdArgs {
   float t;
   float *means_t, *quats_t, *log_scales_t, *logits_t;
   void* feat_t;
-  float* act;  // NULL: forward only
+  float* act;
   const float* f;  // [P][levels * 32] HexPlane features from fst_sample_kernel
 };
 
@@ -512,16 +506,13 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
       cp_async_wait_all();
     }
     __syncthreads();
-    if (act && valid) {
-      for (int c = 0; c < nl * kFC; ++c) act[(size_t)(g.sf + l0 * kFC + c) * P + p] = A[tid * kFRow + c];
-    }
     {
       const float* w = next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf);
       tile_mma<8, TM, 8>(A, nl * kFC, w, kFW, row0, nt * 8, acc);
     }
     __syncthreads();
   }
-  tile_out<8>(acc, a.wt + g.ab[0], row0, nt * 8, act, P, g.sz, p0, B, 0);
+  tile_out<8>(acc, a.wt + g.ab[0], row0, nt * 8, act, g.nslots, P, g.sz, p0, B, 0);
   __syncthreads();
   // z_j = W_j relu(z_{j-1}) + b_j; layer j reads (j odd ? B : A).
   for (int j = 1; j < kFDepth; ++j) {
@@ -529,7 +520,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
     float* dst = (j & 1) ? A : B;
     tile_zero<8, TM>(acc);
     tile_mma<8, TM, 8>(src, kFW, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFW, row0, nt * 8, acc);
-    tile_out<8>(acc, a.wt + g.ab[j], row0, nt * 8, act, P, g.sz + j * kFW, p0, dst, 0);
+    tile_out<8>(acc, a.wt + g.ab[j], row0, nt * 8, act, g.nslots, P, g.sz + j * kFW, p0, dst, 0);
     __syncthreads();
   }
   // relu(h) is in A.  Branches: e1 -> B[0, 32), h_g -> B[32, 64); the
@@ -544,14 +535,14 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
       float2 e[TM][2];
       tile_zero<4, TM>(e);
       tile_mma<4, TM, 8>(A, kFW, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFHalf, row0, nt * 4, e);
-      tile_out<4>(e, a.wt + g.ab[l1], row0, nt * 4, act, P, g.se1 + b * kFHalf, p0, B, 0);
+      tile_out<4>(e, a.wt + g.ab[l1], row0, nt * 4, act, g.nslots, P, g.se1 + b * kFHalf, p0, B, 0);
     }
     __syncthreads();
     {
       float2 e[TM][2];
       tile_zero<4, TM>(e);
       tile_mma<4, TM, 8>(B, kFHalf, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFHalf, row0, nt * 4, e);
-      tile_out<4>(e, a.wt + g.ab[l1 + 1], row0, nt * 4, act, P, g.shg + b * kFHalf, p0, B, kFHalf);
+      tile_out<4>(e, a.wt + g.ab[l1 + 1], row0, nt * 4, act, g.nslots, P, g.shg + b * kFHalf, p0, B, kFHalf);
     }
     __syncthreads();
     // Head (the owner thread's own Gaussian): offset = H relu(h_g) + b.
@@ -577,7 +568,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
     tile_mma<8, TM, 8>(B + kFHalf, kFHalf, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFW, row0, nt * 8, v);
     __syncthreads();
   }
-  tile_out<8>(v, a.wt + g.ab[kLZ1], row0, nt * 8, act, P, g.sv, p0, A, 0);
+  tile_out<8>(v, a.wt + g.ab[kLZ1], row0, nt * 8, act, g.nslots, P, g.sv, p0, A, 0);
   __syncthreads();
   // dz = Z2 relu(v) + b, 64 columns at a time.
   constexpr int ZN = D < 64 ? D : 64, ZT = ZN / 8;
@@ -952,124 +943,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) fst_fwd_tc_kernel(const __grid_
 // ---------------------------------------------------------------------------
 // Reverse.
 // ---------------------------------------------------------------------------
-struct BwdArgs {
-  FstGeom g;
-  const float *planes, *wn, *act;
-  const float *means;
-  float t;
-  const float *d_means_t, *d_quats_t, *d_log_scales_t, *d_logits_t, *d_feat_t;
-  float *d_means, *d_planes;
-  float* dv;    // [64][P]: delta of F_feat's first layer
-  float* df;    // [P][levels * 32]: d f, read by the HexPlane reverse kernel
-  float* part;  // [gridDim.x][mlp_aligned]
-  WTile tiles[kMaxWTiles];  // row-major weight tiles in order of use (per chunk)
-  int ntiles;
-};
-
-// pw[o * ldw + i] (+)= sum over the block's 128 Gaussians of
-// s_d[g][o] * s_x[g][i], o < NO (<= 64), i < NI (multiple of 8, <= 64);
-// pb[o] (+)= sum_g s_d[g][o] when pb is set.  Tiles of TO outputs x 8
-// inputs per thread (TO chosen so that the 128 threads have work); the bias
-// sum runs as two fixed-order halves of independent partial sums.  Starts
-// and ends with a barrier.
-template <int TO>
-__device__ __forceinline__ void outer_tiles(const float* s_d, int ds, const float* s_x, int xs, int NO, int NI,
-                                            float* pw, int ldw, bool first) {
-  const int nog = (NO + TO - 1) / TO, ntile = nog * (NI / 8);
-  for (int tile = threadIdx.x; tile < ntile; tile += kFThreads) {
-    const int o0 = (tile % nog) * TO, i0 = (tile / nog) * 8;
-    // The block's partial rows of this tile are loaded before the product,
-    // so their L2 round trip overlaps it.
-    float4 prev[TO][2];
-#pragma unroll
-    for (int r = 0; r < TO; ++r) {
-      prev[r][0] = prev[r][1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (!first && o0 + r < NO) {
-        const float4* row = reinterpret_cast<const float4*>(pw + (size_t)(o0 + r) * ldw + i0);
-        prev[r][0] = row[0];
-        prev[r][1] = row[1];
-      }
-    }
-    float2 acc[TO][4];
-#pragma unroll
-    for (int r = 0; r < TO; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
-#pragma unroll 4
-    for (int gg = 0; gg < kFThreads; ++gg) {
-      float dv[TO];
-      if (TO == 4) {
-        const float4 d = *reinterpret_cast<const float4*>(s_d + gg * ds + o0);
-        dv[0] = d.x; dv[TO > 1 ? 1 : 0] = d.y; dv[TO > 2 ? 2 : 0] = d.z; dv[TO > 3 ? 3 : 0] = d.w;
-      } else if (TO == 2) {
-        const float2 d = *reinterpret_cast<const float2*>(s_d + gg * ds + o0);
-        dv[0] = d.x; dv[TO > 1 ? 1 : 0] = d.y;
-      } else {
-        dv[0] = s_d[gg * ds + o0];
-      }
-      const float4 x0 = *reinterpret_cast<const float4*>(s_x + gg * xs + i0);
-      const float4 x1 = *reinterpret_cast<const float4*>(s_x + gg * xs + i0 + 4);
-#pragma unroll
-      for (int r = 0; r < TO; ++r) {
-        const float2 dd = make_float2(dv[r], dv[r]);
-        acc[r][0] = __ffma2_rn(dd, make_float2(x0.x, x0.y), acc[r][0]);
-        acc[r][1] = __ffma2_rn(dd, make_float2(x0.z, x0.w), acc[r][1]);
-        acc[r][2] = __ffma2_rn(dd, make_float2(x1.x, x1.y), acc[r][2]);
-        acc[r][3] = __ffma2_rn(dd, make_float2(x1.z, x1.w), acc[r][3]);
-      }
-    }
-    // Partial += this chunk's sums (the partial loaded above; zero for the
-    // block's first chunk, whose sums are stored as they are).
-#pragma unroll
-    for (int r = 0; r < TO; ++r) {
-      if (o0 + r < NO) {
-        float4* row = reinterpret_cast<float4*>(pw + (size_t)(o0 + r) * ldw + i0);
-        float4 v0 = make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
-        float4 v1 = make_float4(acc[r][2].x, acc[r][2].y, acc[r][3].x, acc[r][3].y);
-        if (!first) {
-          const float4 a0 = prev[r][0], a1 = prev[r][1];
-          v0.x += a0.x; v0.y += a0.y; v0.z += a0.z; v0.w += a0.w;
-          v1.x += a1.x; v1.y += a1.y; v1.z += a1.z; v1.w += a1.w;
-        }
-        row[0] = v0;
-        row[1] = v1;
-      }
-    }
-  }
-}
-
-__device__ void block_outer(const float* s_d, int ds, const float* s_x, int xs, int NO, int NI, float* pw, int ldw,
-                            float* pb, bool first) {
-  __shared__ float s_red[kFThreads];
-  __syncthreads();
-  if (NO >= 4 && (NO / 4) * (NI / 8) >= kFThreads)
-    outer_tiles<4>(s_d, ds, s_x, xs, NO, NI, pw, ldw, first);
-  else if (NO >= 2 && (NO / 2) * (NI / 8) >= kFThreads / 2)
-    outer_tiles<2>(s_d, ds, s_x, xs, NO, NI, pw, ldw, first);
-  else
-    outer_tiles<1>(s_d, ds, s_x, xs, NO, NI, pw, ldw, first);
-  if (pb) {
-    const int o = threadIdx.x & 63, half = threadIdx.x >> 6;
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    if (o < NO) {
-#pragma unroll 4
-      for (int gg = half * 64; gg < half * 64 + 64; gg += 4) {
-        s0 += s_d[gg * ds + o];
-        s1 += s_d[(gg + 1) * ds + o];
-        s2 += s_d[(gg + 2) * ds + o];
-        s3 += s_d[(gg + 3) * ds + o];
-      }
-    }
-    s_red[threadIdx.x] = (s0 + s1) + (s2 + s3);
-    __syncthreads();
-    if (threadIdx.x < NO) {
-      const float v = s_red[threadIdx.x] + s_red[threadIdx.x + 64];
-      pb[threadIdx.x] = first ? v : pb[threadIdx.x] + v;
-    }
-  }
-  __syncthreads();
-}
-
 // Exact, order-independent plane-gradient sums.  Each float contribution x
 // is the integer X = x 2^72 (exact for |x| >= 2^-49; smaller ones rounded to
 // the nearest multiple of 2^-72), held as hi 2^32 + lo with 0 <= lo < 2^32,
@@ -1115,180 +988,419 @@ __device__ __forceinline__ void fixed_add(unsigned long long* hi, unsigned long 
   if (l) atomicAdd(lo + i, (unsigned long long)l);
 }
 
-// Y[m][yc + n] <- (X[m][xc + n] > 0 ? acc : 0) for the thread's tile (the
-// ReLU mask read from the stored relu(z) inputs); dv rows optionally copied
-// to global [n][P].
-template <int TN>
-__device__ __forceinline__ void tile_mask(const float2 (&acc)[8][TN / 2], const float* X, int xc, float* Y, int yc,
-                                          int mt, int n0, float* rows, int P, int p0, int xs = kFRow) {
+// Packed weights of the reverse's delta W products: the second operand
+// B[k = output][n = input] in fragment order, three BF16 terms (as
+// fst_pack_tc_kernel's, with the roles of outputs and inputs exchanged), from
+// the row-major copies the forward left.
+__global__ void fst_pack_bwd_kernel(const FstGeom g, const BwdPack pk, const float* __restrict__ wn,
+                                    unsigned char* __restrict__ out) {
+  const int u = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (u * 768 >= pk.bytes) return;
+  int l = 0;
+  while (u * 768 >= pk.off[l + 1]) ++l;
+  const int v = u - pk.off[l] / 768, KS = g.nout[l] / 16, nt = v & 3, ks = (v >> 2) % KS, grp = (v >> 2) / KS;
+  const int n = 32 * grp + 8 * nt + (lane >> 2), k = 16 * ks + 2 * (lane & 3), ld = g.nin[l];
+  const float* w = wn + g.aw[l] + (int64_t)k * ld + n;
+  uint32_t h[2], m[2], lo[2];
+  split3(w[0], w[ld], h[0], m[0], lo[0]);
+  split3(w[8 * ld], w[9 * ld], h[1], m[1], lo[1]);
+  unsigned char* o = out + (size_t)u * 768;
+  reinterpret_cast<uint4*>(o)[lane] = make_uint4(h[0], h[1], m[0], m[1]);
+  reinterpret_cast<uint2*>(o + 512)[lane] = make_uint2(lo[0], lo[1]);
+}
+
+struct BwdArgs {
+  FstGeom g;
+  BwdPack pk;
+  const unsigned char* wp;    // packed weights
+  const float *wn, *act, *f;  // row-major weights (the heads), activations, HexPlane features
+  const float *d_means_t, *d_quats_t, *d_log_scales_t, *d_logits_t, *d_feat_t;
+  float* dv;    // [P][64]: delta of F_feat's first layer
+  float* df;    // [P][levels * 32]: d f, read by the HexPlane reverse kernel
+  float* part;  // [gridDim.x][mlp_aligned]
+};
+
+// A tile of 128 Gaussians x 64 columns in shared memory, three BF16 terms:
+// rows of 128 bytes, 16-byte chunk c of row r at c ^ (r & 7), so that the
+// fragment loads and stores below touch every bank once.
+constexpr int kTTerm = kFM * 128;
+__device__ __forceinline__ uint32_t t_off(int r, int chunk) { return (uint32_t)(r * 128 + ((chunk ^ (r & 7)) << 4)); }
+
+__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&v)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t (&v)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr)
+               : "memory");
+}
+
+// Lane's pair of values (columns c, c + 1; c even) of row r into a tile.
+__device__ __forceinline__ void put_pair(unsigned char* tile, int r, int c, float x, float y) {
+  uint32_t t3[3];
+  split3(x, y, t3[0], t3[1], t3[2]);
+  const uint32_t o = t_off(r, c >> 3) + 2 * (c & 7);
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int m = mt + 16 * r;
+  for (int t = 0; t < 3; ++t) *reinterpret_cast<uint32_t*>(tile + t * kTTerm + o) = t3[t];
+}
+
+// What a lane holds of its warp's 16 rows: columns 8 nt + 2 ft, + 1 of rows fr
+// (elements 0, 1) and fr + 8 (2, 3), the accumulator layout.
+template <int NT>
+__device__ __forceinline__ void load_rows(const float* a, const float* b, int ft, float (&v)[NT][4]) {
 #pragma unroll
-    for (int c = 0; c < TN / 2; ++c) {
-      const float2 x = *reinterpret_cast<const float2*>(X + m * xs + xc + n0 + 2 * c);
-      const float2 d = make_float2(x.x > 0.0f ? acc[r][c].x : 0.0f, x.y > 0.0f ? acc[r][c].y : 0.0f);
-      *reinterpret_cast<float2*>(Y + m * kFRow + yc + n0 + 2 * c) = d;
-      if (rows && p0 + m < P) {
-        rows[(size_t)(n0 + 2 * c) * P + p0 + m] = d.x;
-        rows[(size_t)(n0 + 2 * c + 1) * P + p0 + m] = d.y;
-      }
+  for (int nt = 0; nt < NT; ++nt) {
+    const float2 x = a ? __ldg(reinterpret_cast<const float2*>(a + 8 * nt + 2 * ft)) : make_float2(0.0f, 0.0f);
+    const float2 y = b ? __ldg(reinterpret_cast<const float2*>(b + 8 * nt + 2 * ft)) : make_float2(0.0f, 0.0f);
+    v[nt][0] = x.x; v[nt][1] = x.y; v[nt][2] = y.x; v[nt][3] = y.y;
+  }
+}
+template <int NT>
+__device__ __forceinline__ void put_rows(unsigned char* tile, int row, int c0, int ft, const float (&v)[NT][4]) {
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    put_pair(tile, row, c0 + 8 * nt + 2 * ft, v[nt][0], v[nt][1]);
+    put_pair(tile, row + 8, c0 + 8 * nt + 2 * ft, v[nt][2], v[nt][3]);
+  }
+}
+// v where the activation x (>= 0) is positive, else 0.
+template <int NT>
+__device__ __forceinline__ void mask_rows(float (&v)[NT][4], const float (&x)[NT][4]) {
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[nt][i] = x[nt][i] > 0.0f ? v[nt][i] : 0.0f;
+}
+
+// acc (32 columns) = delta W for the warp's rows: delta in columns
+// [16 kc, 16 (kc + KS)) of the tile, packed weights at w ([KS][4] units).
+template <int KS>
+__device__ __forceinline__ void delta_w(uint32_t tile, int warp, int kc, const unsigned char* __restrict__ w, int lane,
+                                        float (&acc)[4][4]) {
+  float zs[4][4];
+  tc_zero(acc, zs);
+  const int r = warp * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), ch = lane >> 4;
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks) {
+    uint32_t a[3][4];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) ldsm_x4(tile + t * kTTerm + t_off(r, 2 * (kc + ks) + ch), a[t]);
+    tc_step<4>(a[0], a[1], a[2], w + ks * 4 * 768, lane, acc, zs);
+  }
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[nt][i] += zs[nt][i];
+}
+
+// Weight gradient block of one warp: outputs [16 om, + 16) (columns oc0 + ...
+// of the delta tile) x inputs [8 in0, + 8 NT) (columns of the input tile),
+// summed over the tile's 128 Gaussians and added to pw (row stride ldw); with
+// pb also the bias gradient.  rows: outputs that exist.
+template <int NT>
+__device__ __forceinline__ void weight_grad(uint32_t sd, int oc, uint32_t sx, int ic, int rows, float* pw, int ldw, float* pb,
+                                            bool first, int lane) {
+  const int fr = lane >> 2, ft = lane & 3, mi = lane >> 3, r = lane & 7;
+  float2 prev[NT][2];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      prev[nt][h] = !first && fr + 8 * h < rows ? *reinterpret_cast<const float2*>(pw + (size_t)(fr + 8 * h) * ldw + 8 * nt + 2 * ft)
+                                                : make_float2(0.0f, 0.0f);
+  float zh[NT][4], zs[NT][4], bh[1][4], bs[1][4];
+  tc_zero(zh, zs);
+  tc_zero(bh, bs);
+  const uint32_t one = fr == 0 ? 0x3F803F80u : 0u;  // column 0 of the bias tile
+#pragma unroll 1
+  for (int g0 = 0; g0 < kFM; g0 += 16) {
+    uint32_t a[3][4];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) ldsm_x4_t(sd + t * kTTerm + t_off(g0 + r + 8 * (mi >> 1), oc + (mi & 1)), a[t]);
+    if (pb) {
+      mma_bf16_16816(bs[0], a[2], one, one);
+      mma_bf16_16816(bs[0], a[1], one, one);
+      mma_bf16_16816(bh[0], a[0], one, one);
     }
+    constexpr int NP = (NT + 1) / 2;
+    uint32_t b[3][NP][4];
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int q = 0; q < NP; ++q)
+        ldsm_x4_t(sx + t * kTTerm + t_off(g0 + r + 8 * (mi & 1), NT == 1 ? ic : ic + 2 * q + (mi >> 1)), b[t][q]);
+#define FST_WG(za, ta, tb)                                                                                     \
+  _Pragma("unroll") for (int nt = 0; nt < NT; ++nt)                                                            \
+      mma_bf16_16816(za[nt], a[ta], b[tb][nt >> 1][2 * (nt & 1)], b[tb][nt >> 1][2 * (nt & 1) + 1]);
+    FST_WG(zs, 2, 0)
+    FST_WG(zs, 1, 1)
+    FST_WG(zs, 0, 2)
+    FST_WG(zs, 1, 0)
+    FST_WG(zs, 0, 1)
+    FST_WG(zh, 0, 0)
+#undef FST_WG
+  }
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (fr + 8 * h < rows) {
+        const float2 v = prev[nt][h];
+        *reinterpret_cast<float2*>(pw + (size_t)(fr + 8 * h) * ldw + 8 * nt + 2 * ft) =
+            make_float2(v.x + (zh[nt][2 * h] + zs[nt][2 * h]), v.y + (zh[nt][2 * h + 1] + zs[nt][2 * h + 1]));
+      }
+  if (pb && ft == 0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (fr + 8 * h < rows) pb[fr + 8 * h] = (first ? 0.0f : pb[fr + 8 * h]) + (bh[0][2 * h] + bs[0][2 * h]);
   }
 }
 
-constexpr int kTRow = 36;  // row stride of the small third buffer
-constexpr size_t kBwdSmem = ((size_t)(2 * kFRow + kTRow) * kFThreads + 2 * kWBufR) * 4;
+constexpr int kBwdThreads = 256;
+constexpr size_t kBwdSmem = 6 * (size_t)kTTerm + 1024;
 
-
+// Reverse of the MLP for 128 Gaussians at a time (persistent blocks).  Layers
+// are walked backwards; a round holds a layer's delta and input tiles in
+// shared memory (three BF16 terms), from which the block's eight warps take
+// the weight gradient (each a 16-output block, all 128 Gaussians) and each
+// warp the input delta of its own 16 Gaussians, masked by the stored
+// relu(z).  The same term products and accumulators as the forward without
+// reverse state.
+//
+// Bound by the tensor pipe (200k Gaussians, 4 levels: 150 M products of
+// 16 x 8 x 16, 472 us at 607 TFLOP/s) and, under it, by the rounds' barriers
+// and fragment loads.  The FP32 form (8 x 8 register tiles of packed FMAs,
+// 249 registers, 8 warps per SM) took 1555 us.
 template <int D>
-__global__ void __launch_bounds__(kFThreads, 2) fst_bwd_kernel(const BwdArgs a) {
-  extern __shared__ __align__(16) float s_dyn[];
-  float* SD = s_dyn;                            // [128][kFRow]: deltas
-  float* SX = s_dyn + kFThreads * kFRow;        // [128][kFRow]: layer inputs
-  float* ST = s_dyn + 2 * kFThreads * kFRow;    // [128][kTRow]: relu(h_g) | head deltas; grid axes
-  float* wbuf = ST + kFThreads * kTRow;         // [2][kWBufR] staged weight tiles
+__global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_constant__ BwdArgs a) {
+  extern __shared__ unsigned char s_raw[];
+  unsigned char* sD = s_raw + ((1024u - (smem_addr(s_raw) & 1023u)) & 1023u);
+  unsigned char* sX = sD + 3 * kTTerm;
+  const uint32_t uD = smem_addr(sD), uX = smem_addr(sX);
   const FstGeom& g = a.g;
-  const int tid = threadIdx.x;
-  const int mt = tid & 15, nt = tid >> 4;
-  const int P = g.P;
-  const int nchunk = (P + kFThreads - 1) / kFThreads;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, fr = lane >> 2, ft = lane & 3;
+  const int P = g.P, nf = g.levels * kFC, row = warp * 16 + fr;
+  const int nchunk = (P + kFM - 1) / kFM;
   float* part = a.part + (size_t)blockIdx.x * g.mlp_aligned;
-  const float* act = a.act;
+  // Weight-gradient blocks: output tile om and input columns of this warp.
+  auto wgrad = [&](int l, int oc, int O, int ic, int I, int i0, bool bias, bool first) {
+    // Outputs O (64, 32 or 16 of the tile's columns from oc), inputs I (64 or
+    // 32 of the tile's columns from ic) that are inputs i0 .. of layer l.
+    const int om = warp % (O / 16), grp = warp / (O / 16);
+    float* pw = part + g.aw[l] + (size_t)(16 * om) * g.nin[l] + i0;
+    float* pb = bias && grp == 0 ? part + g.ab[l] + 16 * om : nullptr;
+    if (O == 64 && I == 64)
+      weight_grad<4>(uD, oc + 2 * om, uX, ic + 4 * grp, 16, pw + 32 * grp, g.nin[l], pb, first, lane);
+    else if ((O == 64 && I == 32) || (O == 32 && I == 64))
+      weight_grad<2>(uD, oc + 2 * om, uX, ic + 2 * grp, 16, pw + 16 * grp, g.nin[l], pb, first, lane);
+    else
+      weight_grad<1>(uD, oc + 2 * om, uX, ic + grp, 16, pw + 8 * grp, g.nin[l], pb, first, lane);
+  };
   for (int chunk = blockIdx.x; chunk < nchunk; chunk += gridDim.x) {
     const bool first = chunk == (int)blockIdx.x;
-    const int p0 = chunk * kFThreads;
-    const int p = p0 + tid;
-    const bool valid = p < P;
-    int wt_i = 0;
-    stage_tile<kWBufR>(a.tiles, a.ntiles, 0, a.wn, wbuf);
-    // ---- F_feat second layer: delta = d dz; input relu(v).
-    rows_async<kFW>(SX, 0, act, P, g.sv, p0, tid);
-    float2 acc[8][4];
-    tile_zero<8>(acc);
+    const int p[2] = {chunk * kFM + row, chunk * kFM + row + 8};
+    const bool valid[2] = {p[0] < P, p[1] < P};
+    const float* act[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) act[h] = valid[h] ? a.act + (size_t)p[h] * g.nslots : nullptr;
+    auto act_rows = [&](int slot, auto& v) { load_rows(act[0] ? act[0] + slot : nullptr, act[1] ? act[1] + slot : nullptr, ft, v); };
+    float d[8][4];  // delta of 64 columns (or the sum that becomes it)
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[nt][i] = 0.0f;
+    float x[8][4];
+    // ---- F_feat second layer: delta = d dz, input relu(v).
     constexpr int NC = D < 64 ? D : 64;
+    act_rows(g.sv, x);
+#pragma unroll 1
     for (int c0 = 0; c0 < D; c0 += NC) {
-      for (int q = 0; q < NC; q += 4)
-        *reinterpret_cast<float4*>(SD + tid * kFRow + q) =
-            valid ? __ldg(reinterpret_cast<const float4*>(a.d_feat_t + (size_t)p * D + c0 + q)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      cp_async_wait_all();
-      block_outer(SD, kFRow, SX, kFRow, NC, kFW, part + g.aw[kLZ2] + (size_t)c0 * kFW, kFW, part + g.ab[kLZ2] + c0, first);
-      for (int r0 = 0; r0 < NC; r0 += 32) {
-        if (r0) __syncthreads();
-        const float* w = next_tile<kWBufR>(a.tiles, a.ntiles, wt_i, a.wn, wbuf);
-        tile_mma<8, 8, 16>(SD + r0, NC - r0 < 32 ? NC - r0 : 32, w, kFW, mt, nt * 8, acc);
-      }
-      __syncthreads();
-    }
-    // delta_v (kept in SD and in the workspace for the branches).
-    tile_mask<8>(acc, SX, 0, SD, 0, mt, nt * 8, a.dv, P, p0);
-    // ---- F_feat first layer: input relu(u), u = [h_mu, h_R, h_S, h_o].
-    for (int half = 0; half < 2; ++half) {
-      __syncthreads();
-      rows_async<kFW>(SX, 0, act, P, g.shg + half * kFW, p0, tid);
-      cp_async_wait_all();
-      block_outer(SD, kFRow, SX, kFRow, kFW, kFW, part + g.aw[kLZ1] + half * kFW, 4 * kFHalf, half ? nullptr : part + g.ab[kLZ1],
-                  first);
-    }
-    // ---- Branches; d relu(h) accumulates over them.
-    float2 drh[8][4];
-    tile_zero<8>(drh);
-    const float* dsrc[4] = {a.d_means_t, a.d_quats_t, a.d_log_scales_t, a.d_logits_t};
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      constexpr int dgs[4] = {3, 4, 3, 1};
-      const int dg = dgs[b], l1 = branch_e1(b);
-      // delta_v rows -> SX; relu(h_g) and the head deltas -> ST.
-      __syncthreads();
-      rows_async<kFW>(SX, 0, a.dv, P, 0, p0, tid);
-      rows_async<kFHalf>(ST, 0, act, P, g.shg + b * kFHalf, p0, tid, kTRow);
-#pragma unroll
-      for (int o = 0; o < 4; ++o) ST[tid * kTRow + kFHalf + o] = (o < dg && valid) ? __ldg(dsrc[b] + (size_t)p * dg + o) : 0.0f;
-      cp_async_wait_all();
-      __syncthreads();
-      // d relu(h_g) = Z1[:, branch b]^T delta_v + H^T d offset, masked.
-      float2 e[8][2];
-      tile_zero<4>(e);
-      tile_mma<4, 8, 16>(SX, kFW, next_tile<kWBufR>(a.tiles, a.ntiles, wt_i, a.wn, wbuf), kFHalf, mt, nt * 4, e);
+      __syncthreads();  // the tiles are free (previous chunk or part)
       {
+        float z[NC / 8][4];
+        load_rows(valid[0] ? a.d_feat_t + (size_t)p[0] * D + c0 : nullptr, valid[1] ? a.d_feat_t + (size_t)p[1] * D + c0 : nullptr, ft, z);
+        put_rows(sD, row, 0, ft, z);
+      }
+      if (c0 == 0) put_rows(sX, row, 0, ft, x);
+      __syncthreads();
+      {
+        float* pw = part + g.aw[kLZ2] + (size_t)c0 * kFW;
+        float* pb = part + g.ab[kLZ2] + c0;
+        constexpr int OT = NC / 16;
+        const int om = warp % OT, grp = warp / OT;
+        constexpr int NTW = OT;  // 64 columns over 8 / OT groups: OT tiles each
+        weight_grad<NTW>(uD, 2 * om, uX, NTW * grp, 16, pw + (size_t)(16 * om) * kFW + 8 * NTW * grp, kFW, grp == 0 ? pb + 16 * om : nullptr, first, lane);
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float z[4][4];
+        // Packed [group][outputs / 16][4]: the outputs of this part.
+        delta_w<NC / 16>(uD, warp, 0, a.wp + a.pk.off[kLZ2] + ((size_t)h * (D / 16) + c0 / 16) * 4 * 768, lane, z);
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) d[4 * h + nt][i] += z[nt][i];
+      }
+    }
+    mask_rows(d, x);
+    // ---- F_feat first layer: input u = [h_mu, h_R, h_S, h_o] (relu).  Its
+    // delta goes to the tile and to the workspace (for the branches).
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (valid[h])
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt)
+          *reinterpret_cast<float2*>(a.dv + (size_t)p[h] * kFW + 8 * nt + 2 * ft) = make_float2(d[nt][2 * h], d[nt][2 * h + 1]);
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      act_rows(g.shg + half * kFW, x);
+      __syncthreads();
+      if (half == 0) put_rows(sD, row, 0, ft, d);
+      put_rows(sX, row, 0, ft, x);
+      __syncthreads();
+      wgrad(kLZ1, 0, 64, 0, 64, half * kFW, half == 0, first);
+    }
+    // ---- branches; d relu(h) accumulates over them.
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[nt][i] = 0.0f;
+#pragma unroll 1
+    for (int b = 0; b < 4; ++b) {
+      const int dg = branch_out(b), l1 = branch_e1(b);
+      const float* dsrc = b == 0 ? a.d_means_t : b == 1 ? a.d_quats_t : b == 2 ? a.d_log_scales_t : a.d_logits_t;
+      float off[2][4];  // head deltas of the two rows
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) off[h][o] = valid[h] && o < dg ? __ldg(dsrc + (size_t)p[h] * dg + o) : 0.0f;
+      // delta of h_g: Z1[:, branch]^T delta_v + H^T d offset, masked.
+      float du[4][4];
+      {
+        float zs[4][4];
+        tc_zero(du, zs);
+        const unsigned char* w = a.wp + a.pk.off[kLZ1] + (size_t)b * 4 * 4 * 768;
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+          uint32_t f3[3][4];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float* r = a.dv + (size_t)(valid[h] ? p[h] : 0) * kFW + 16 * ks + 2 * ft;
+            const float2 u0 = valid[h] ? *reinterpret_cast<const float2*>(r) : make_float2(0.f, 0.f);
+            const float2 u1 = valid[h] ? *reinterpret_cast<const float2*>(r + 8) : make_float2(0.f, 0.f);
+            split3(u0.x, u0.y, f3[0][h], f3[1][h], f3[2][h]);
+            split3(u1.x, u1.y, f3[0][2 + h], f3[1][2 + h], f3[2][2 + h]);
+          }
+          tc_step<4>(f3[0], f3[1], f3[2], w + ks * 4 * 768, lane, du, zs);
+        }
         const float* wh = a.wn + g.aw[l1 + 2];  // [dg][32]
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const float* dh = ST + (mt + 16 * r) * kTRow + kFHalf;
+        for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-          for (int o = 0; o < 4; ++o) {
-            if (o < dg) {
-              const float2 d2 = make_float2(dh[o], dh[o]);
+          for (int i = 0; i < 4; ++i) du[nt][i] += zs[nt][i];
 #pragma unroll
-              for (int c = 0; c < 2; ++c)
-                e[r][c] = __ffma2_rn(d2, __ldg(reinterpret_cast<const float2*>(wh + o * kFHalf + nt * 4) + c), e[r][c]);
+        for (int o = 0; o < 4; ++o)
+          if (o < dg)
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+              const float2 w2 = __ldg(reinterpret_cast<const float2*>(wh + o * kFHalf + 8 * nt + 2 * ft));
+              du[nt][0] = fmaf(off[0][o], w2.x, du[nt][0]);
+              du[nt][1] = fmaf(off[0][o], w2.y, du[nt][1]);
+              du[nt][2] = fmaf(off[1][o], w2.x, du[nt][2]);
+              du[nt][3] = fmaf(off[1][o], w2.y, du[nt][3]);
             }
-          }
-        }
       }
-      tile_mask<4>(e, ST, 0, SD, 0, mt, nt * 4, nullptr, P, p0, kTRow);   // delta_hg -> SD[0, 32)
-      // head: delta = d offset (ST[32, 36)), input relu(h_g) (ST[0, 32)).
-      block_outer(ST + kFHalf, kTRow, ST, kTRow, dg, kFHalf, part + g.aw[l1 + 2], kFHalf, part + g.ab[l1 + 2], first);
-      // E2: delta_hg (SD[0, 32)), input relu(e1).
-      rows_async<kFHalf>(SX, 0, act, P, g.se1 + b * kFHalf, p0, tid);
-      cp_async_wait_all();
-      block_outer(SD, kFRow, SX, kFRow, kFHalf, kFHalf, part + g.aw[l1 + 1], kFHalf, part + g.ab[l1 + 1], first);
-      tile_zero<4>(e);
-      tile_mma<4, 8, 16>(SD, kFHalf, next_tile<kWBufR>(a.tiles, a.ntiles, wt_i, a.wn, wbuf), kFHalf, mt, nt * 4, e);
+      float u[4][4], e1[4][4];
+      act_rows(g.shg + b * kFHalf, u);
+      act_rows(g.se1 + b * kFHalf, e1);
+      mask_rows(du, u);
       __syncthreads();
-      tile_mask<4>(e, SX, 0, SD, 0, mt, nt * 4, nullptr, P, p0);   // delta_e1 -> SD[0, 32)
+      // Round 1: delta of h_g and the head deltas (columns 32..47 of the
+      // tile, zeros past dg); inputs e1 and h_g.
+      put_rows(sD, row, 0, ft, du);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        put_pair(sD, row + 8 * h, 32 + 2 * ft, ft == 0 ? off[h][0] : ft == 1 ? off[h][2] : 0.0f,
+                 ft == 0 ? off[h][1] : ft == 1 ? off[h][3] : 0.0f);
+        put_pair(sD, row + 8 * h, 40 + 2 * ft, 0.0f, 0.0f);
+      }
+      put_rows(sX, row, 0, ft, e1);
+      put_rows(sX, row, 32, ft, u);
       __syncthreads();
-      // E1: delta_e1, input relu(h).
-      rows_async<kFW>(SX, 0, act, P, g.sz + (kFDepth - 1) * kFW, p0, tid);
-      cp_async_wait_all();
-      block_outer(SD, kFRow, SX, kFRow, kFHalf, kFW, part + g.aw[l1], kFW, part + g.ab[l1], first);
-      tile_mma<8, 8, 16>(SD, kFHalf, next_tile<kWBufR>(a.tiles, a.ntiles, wt_i, a.wn, wbuf), kFW, mt, nt * 8, drh);
+      wgrad(l1 + 1, 0, 32, 0, 32, 0, true, first);
+      if (warp < 4)
+        weight_grad<1>(uD, 4, uX, 4 + warp, dg, part + g.aw[l1 + 2] + 8 * warp, kFHalf, warp == 0 ? part + g.ab[l1 + 2] : nullptr, first, lane);
+      float de[4][4];
+      delta_w<2>(uD, warp, 0, a.wp + a.pk.off[l1 + 1], lane, de);
+      mask_rows(de, e1);
+      act_rows(g.sz + (kFDepth - 1) * kFW, x);
+      __syncthreads();
+      // Round 2: delta of e1, input relu(h).
+      put_rows(sD, row, 0, ft, de);
+      put_rows(sX, row, 0, ft, x);
+      __syncthreads();
+      wgrad(l1, 0, 32, 0, 64, 0, true, first);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float z[4][4];
+        delta_w<2>(uD, warp, 0, a.wp + a.pk.off[l1] + (size_t)h * 2 * 4 * 768, lane, z);
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) d[4 * h + nt][i] += z[nt][i];
+      }
     }
-    // ---- F_out, last layer first.  SX holds relu(h).
-    __syncthreads();
-    tile_mask<8>(drh, SX, 0, SD, 0, mt, nt * 8, nullptr, P, p0);
+    // ---- F_out, last layer first (x holds relu(h)).
+    mask_rows(d, x);
+#pragma unroll 1
     for (int j = kFDepth - 1; j >= 1; --j) {
+      act_rows(g.sz + (j - 1) * kFW, x);
       __syncthreads();
-      rows_async<kFW>(SX, 0, act, P, g.sz + (j - 1) * kFW, p0, tid);
-      cp_async_wait_all();
-      block_outer(SD, kFRow, SX, kFRow, kFW, kFW, part + g.aw[j], kFW, part + g.ab[j], first);
-      tile_zero<8>(acc);
-      tile_mma<8, 8, 16>(SD, 32, next_tile<kWBufR>(a.tiles, a.ntiles, wt_i, a.wn, wbuf), kFW, mt, nt * 8, acc);
+      put_rows(sD, row, 0, ft, d);
+      put_rows(sX, row, 0, ft, x);
       __syncthreads();
-      tile_mma<8, 8, 16>(SD + 32, 32, next_tile<kWBufR>(a.tiles, a.ntiles, wt_i, a.wn, wbuf), kFW, mt, nt * 8, acc);
-      __syncthreads();
-      tile_mask<8>(acc, SX, 0, SD, 0, mt, nt * 8, nullptr, P, p0);
-    }
-    // First layer: input f.
-    const int nf = g.levels * kFC;
-    for (int c0 = 0; c0 < nf; c0 += kFW) {
-      const int nc = nf - c0 < kFW ? nf - c0 : kFW;
-      __syncthreads();
-      if (nc == kFW) rows_async<kFW>(SX, 0, act, P, g.sf + c0, p0, tid);
-      else rows_async<kFC>(SX, 0, act, P, g.sf + c0, p0, tid);
-      cp_async_wait_all();
-      block_outer(SD, kFRow, SX, kFRow, kFW, nc, part + g.aw[0] + c0, nf, c0 ? nullptr : part + g.ab[0], first);
-    }
-    // ---- d f = W0^T delta_0, 32 columns per level, staged in SX and
-    // written Gaussian-major for the HexPlane reverse kernel.
-    for (int lv = 0; lv < g.levels; ++lv) {
-      float2 e[8][2];
-      tile_zero<4>(e);
-      tile_mma<4, 8, 16>(SD, kFW, next_tile<kWBufR>(a.tiles, a.ntiles, wt_i, a.wn, wbuf), kFC, mt, nt * 4, e);
-      __syncthreads();
+      wgrad(j, 0, 64, 0, 64, 0, true, first);
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
+      for (int h = 0; h < 2; ++h) {
+        float z[4][4];
+        delta_w<4>(uD, warp, 0, a.wp + a.pk.off[j] + (size_t)h * 4 * 4 * 768, lane, z);
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-          *reinterpret_cast<float2*>(SX + (mt + 16 * r) * kFRow + nt * 4 + 2 * c) = e[r][c];
-      __syncthreads();
-      if (valid) {
-        float4* dst = reinterpret_cast<float4*>(a.df + (size_t)p * nf + lv * kFC);
+        for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-        for (int q = 0; q < kFC / 4; ++q) dst[q] = *reinterpret_cast<const float4*>(SX + tid * kFRow + 4 * q);
+          for (int i = 0; i < 4; ++i) d[4 * h + nt][i] = x[4 * h + nt][i] > 0.0f ? z[nt][i] : 0.0f;
       }
     }
-    __syncthreads();  // the buffers are rewritten by the next chunk
+    // First layer: input f, 64 columns (two levels) at a time; d f.
+#pragma unroll 1
+    for (int c0 = 0; c0 < nf; c0 += kFW) {
+      const bool wide = nf - c0 >= kFW;
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) {
+        const bool in = wide || nt < 4;
+        const float2 u0 = in && valid[0] ? __ldg(reinterpret_cast<const float2*>(a.f + (size_t)p[0] * nf + c0 + 8 * nt + 2 * ft)) : make_float2(0.f, 0.f);
+        const float2 u1 = in && valid[1] ? __ldg(reinterpret_cast<const float2*>(a.f + (size_t)p[1] * nf + c0 + 8 * nt + 2 * ft)) : make_float2(0.f, 0.f);
+        x[nt][0] = u0.x; x[nt][1] = u0.y; x[nt][2] = u1.x; x[nt][3] = u1.y;
+      }
+      __syncthreads();
+      if (c0 == 0) put_rows(sD, row, 0, ft, d);
+      put_rows(sX, row, 0, ft, x);
+      __syncthreads();
+      wgrad(0, 0, 64, 0, wide ? 64 : 32, c0, c0 == 0, first);
+      for (int h = 0; h < (wide ? 2 : 1); ++h) {
+        float z[4][4];
+        delta_w<4>(uD, warp, 0, a.wp + a.pk.off[0] + (size_t)(c0 / 32 + h) * 4 * 4 * 768, lane, z);
+#pragma unroll
+        for (int r2 = 0; r2 < 2; ++r2)
+          if (valid[r2])
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+              *reinterpret_cast<float2*>(a.df + (size_t)p[r2] * nf + c0 + 32 * h + 8 * nt + 2 * ft) = make_float2(z[nt][2 * r2], z[nt][2 * r2 + 1]);
+      }
+    }
   }
 }
 
@@ -1570,7 +1682,7 @@ cudaError_t launch_fst_bwd(const BwdArgs& a, int nblk, cudaStream_t st) {
   const size_t smem = kBwdSmem;
   auto k = fst_bwd_kernel<D>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k<<<nblk, kFThreads, smem, st>>>(a);
+  k<<<nblk, kBwdThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1715,42 +1827,20 @@ extern "C" fe_status fe_fst_backward(const fe_fst* fst, int P, const float* mean
   }
   BwdArgs a{};
   a.g = g;
-  a.planes = fst->planes;
+  a.pk = bwd_pack(g);
+  a.wp = ws + w.wp;
   a.wn = reinterpret_cast<const float*>(ws + w.wn);
   a.act = reinterpret_cast<const float*>(ws + w.act);
-  a.means = means;
-  a.t = t;
+  a.f = reinterpret_cast<const float*>(ws + w.f);
   a.d_means_t = d_means_t;
   a.d_quats_t = d_quats_t;
   a.d_log_scales_t = d_log_scales_t;
   a.d_logits_t = d_opacity_logits_t;
   a.d_feat_t = d_feat_t;
-  a.d_means = d_means;
-  a.d_planes = d_planes;
   a.dv = reinterpret_cast<float*>(ws + w.dv);
   a.df = reinterpret_cast<float*>(ws + w.df);
   a.part = reinterpret_cast<float*>(ws + w.part);
-  // Row-major weight tiles (at most 2048 floats) in the order the kernel
-  // uses them for every chunk.
-  {
-    int n = 0;
-    auto add = [&](int64_t off, int rows, int cols, int ld) { a.tiles[n++] = WTile{off, rows, cols, ld}; };
-    const int nc = g.D < 64 ? g.D : 64;
-    for (int c0 = 0; c0 < g.D; c0 += nc)
-      for (int r0 = 0; r0 < nc; r0 += 32) add(g.aw[kLZ2] + (int64_t)(c0 + r0) * kFW, nc - r0 < 32 ? nc - r0 : 32, kFW, kFW);
-    for (int b = 0; b < 4; ++b) {
-      add(g.aw[kLZ1] + b * kFHalf, kFW, kFHalf, 4 * kFHalf);
-      add(g.aw[branch_e1(b) + 1], kFHalf, kFHalf, kFHalf);
-      add(g.aw[branch_e1(b)], kFHalf, kFW, kFW);
-    }
-    for (int j = kFDepth - 1; j >= 1; --j) {
-      add(g.aw[j], 32, kFW, kFW);
-      add(g.aw[j] + 32 * kFW, 32, kFW, kFW);
-    }
-    const int nf = g.levels * kFC;
-    for (int lv = 0; lv < g.levels; ++lv) add(g.aw[0] + lv * kFC, kFW, kFC, nf);
-    a.ntiles = n;
-  }
+  fst_pack_bwd_kernel<<<(a.pk.bytes / 768 * 32 + 255) / 256, 256, 0, st>>>(g, a.pk, a.wn, ws + w.wp);
   const int nblk = bwd_blocks(P);
   cudaError_t e = cudaErrorInvalidValue;
   switch (g.D) {
