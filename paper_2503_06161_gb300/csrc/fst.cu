@@ -1161,7 +1161,8 @@ __device__ __forceinline__ void weight_grad(uint32_t sd, int oc, uint32_t sx, in
 }
 
 constexpr int kBwdThreads = 256;
-constexpr size_t kBwdSmem = 6 * (size_t)kTTerm + 1024;
+constexpr int kBwdW = 4 * 4 * 768;  // staged weights: 64 outputs x 32 columns
+constexpr size_t kBwdSmem = 6 * (size_t)kTTerm + kBwdW + 1024;
 
 // Reverse of the MLP for 128 Gaussians at a time (persistent blocks).  Layers
 // are walked backwards; a round holds a layer's delta and input tiles in
@@ -1180,6 +1181,7 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
   extern __shared__ unsigned char s_raw[];
   unsigned char* sD = s_raw + ((1024u - (smem_addr(s_raw) & 1023u)) & 1023u);
   unsigned char* sX = sD + 3 * kTTerm;
+  unsigned char* sW = sX + 3 * kTTerm;
   const uint32_t uD = smem_addr(sD), uX = smem_addr(sX);
   const FstGeom& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, fr = lane >> 2, ft = lane & 3;
@@ -1200,6 +1202,17 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
     else
       weight_grad<1>(uD, oc + 2 * om, uX, ic + grp, 16, pw + 8 * grp, g.nin[l], pb, first, lane);
   };
+  // Weights of the next delta W product into sW (every thread is past the
+  // product before it); landed() completes the copy for the whole block, with
+  // the tiles written meanwhile.
+  auto stage = [&](int l, int off, int bytes) {
+    const unsigned char* src = a.wp + a.pk.off[l] + off;
+    for (int i = tid; i < bytes / 16; i += kBwdThreads) cp_async16(sW + 16 * i, src + 16 * i);
+  };
+  auto landed = [&]() {
+    cp_async_wait_all();
+    __syncthreads();
+  };
   for (int chunk = blockIdx.x; chunk < nchunk; chunk += gridDim.x) {
     const bool first = chunk == (int)blockIdx.x;
     const int p[2] = {chunk * kFM + row, chunk * kFM + row + 8};
@@ -1207,6 +1220,12 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
     const float* act[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) act[h] = valid[h] ? a.act + (size_t)p[h] * g.nslots : nullptr;
+    // A round's activation rows are fetched to L2 a round ahead: a lane takes
+    // one 128-byte line of its warp's 16 rows of 64 floats.
+    const int pf = chunk * kFM + warp * 16 + (lane >> 1);
+    auto fetch = [&](int slot) {
+      if (pf < P) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.act + (size_t)pf * g.nslots + slot + 32 * (lane & 1)));
+    };
     auto act_rows = [&](int slot, auto& v) { load_rows(act[0] ? act[0] + slot : nullptr, act[1] ? act[1] + slot : nullptr, ft, v); };
     float d[8][4];  // delta of 64 columns (or the sum that becomes it)
 #pragma unroll
@@ -1220,13 +1239,27 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
 #pragma unroll 1
     for (int c0 = 0; c0 < D; c0 += NC) {
       __syncthreads();  // the tiles are free (previous chunk or part)
+      // Packed [group][outputs / 16][4]: the outputs of this part.
+      stage(kLZ2, (c0 / 16) * 4 * 768, NC / 16 * 4 * 768);
       {
         float z[NC / 8][4];
         load_rows(valid[0] ? a.d_feat_t + (size_t)p[0] * D + c0 : nullptr, valid[1] ? a.d_feat_t + (size_t)p[1] * D + c0 : nullptr, ft, z);
         put_rows(sD, row, 0, ft, z);
       }
       if (c0 == 0) put_rows(sX, row, 0, ft, x);
+      fetch(g.shg);
+      landed();
+      auto product = [&](int h) {
+        float z[4][4];
+        delta_w<NC / 16>(uD, warp, 0, sW, lane, z);
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) d[4 * h + nt][i] += z[nt][i];
+      };
+      product(0);
       __syncthreads();
+      stage(kLZ2, (D / 16 + c0 / 16) * 4 * 768, NC / 16 * 4 * 768);
       {
         float* pw = part + g.aw[kLZ2] + (size_t)c0 * kFW;
         float* pb = part + g.ab[kLZ2] + c0;
@@ -1235,16 +1268,8 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
         constexpr int NTW = OT;  // 64 columns over 8 / OT groups: OT tiles each
         weight_grad<NTW>(uD, 2 * om, uX, NTW * grp, 16, pw + (size_t)(16 * om) * kFW + 8 * NTW * grp, kFW, grp == 0 ? pb + 16 * om : nullptr, first, lane);
       }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float z[4][4];
-        // Packed [group][outputs / 16][4]: the outputs of this part.
-        delta_w<NC / 16>(uD, warp, 0, a.wp + a.pk.off[kLZ2] + ((size_t)h * (D / 16) + c0 / 16) * 4 * 768, lane, z);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) d[4 * h + nt][i] += z[nt][i];
-      }
+      landed();
+      product(1);
     }
     mask_rows(d, x);
     // ---- F_feat first layer: input u = [h_mu, h_R, h_S, h_o] (relu).  Its
@@ -1258,6 +1283,7 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
       act_rows(g.shg + half * kFW, x);
+      fetch(half == 0 ? g.shg + kFW : g.se1);
       __syncthreads();
       if (half == 0) put_rows(sD, row, 0, ft, d);
       put_rows(sX, row, 0, ft, x);
@@ -1279,11 +1305,13 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
 #pragma unroll
         for (int o = 0; o < 4; ++o) off[h][o] = valid[h] && o < dg ? __ldg(dsrc + (size_t)p[h] * dg + o) : 0.0f;
       // delta of h_g: Z1[:, branch]^T delta_v + H^T d offset, masked.
+      __syncthreads();
+      stage(kLZ1, b * 4 * 4 * 768, 4 * 4 * 768);
+      landed();
       float du[4][4];
       {
         float zs[4][4];
         tc_zero(du, zs);
-        const unsigned char* w = a.wp + a.pk.off[kLZ1] + (size_t)b * 4 * 4 * 768;
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
           uint32_t f3[3][4];
@@ -1295,7 +1323,7 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
             split3(u0.x, u0.y, f3[0][h], f3[1][h], f3[2][h]);
             split3(u1.x, u1.y, f3[0][2 + h], f3[1][2 + h], f3[2][2 + h]);
           }
-          tc_step<4>(f3[0], f3[1], f3[2], w + ks * 4 * 768, lane, du, zs);
+          tc_step<4>(f3[0], f3[1], f3[2], sW + ks * 4 * 768, lane, du, zs);
         }
         const float* wh = a.wn + g.aw[l1 + 2];  // [dg][32]
 #pragma unroll
@@ -1319,6 +1347,7 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
       act_rows(g.se1 + b * kFHalf, e1);
       mask_rows(du, u);
       __syncthreads();
+      stage(l1 + 1, 0, 2 * 4 * 768);
       // Round 1: delta of h_g and the head deltas (columns 32..47 of the
       // tile, zeros past dg); inputs e1 and h_g.
       put_rows(sD, row, 0, ft, du);
@@ -1330,24 +1359,27 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
       }
       put_rows(sX, row, 0, ft, e1);
       put_rows(sX, row, 32, ft, u);
-      __syncthreads();
+      fetch(g.sz + (kFDepth - 1) * kFW);
+      landed();
       wgrad(l1 + 1, 0, 32, 0, 32, 0, true, first);
       if (warp < 4)
         weight_grad<1>(uD, 4, uX, 4 + warp, dg, part + g.aw[l1 + 2] + 8 * warp, kFHalf, warp == 0 ? part + g.ab[l1 + 2] : nullptr, first, lane);
       float de[4][4];
-      delta_w<2>(uD, warp, 0, a.wp + a.pk.off[l1 + 1], lane, de);
+      delta_w<2>(uD, warp, 0, sW, lane, de);
       mask_rows(de, e1);
       act_rows(g.sz + (kFDepth - 1) * kFW, x);
       __syncthreads();
+      stage(l1, 0, 2 * 2 * 4 * 768);
       // Round 2: delta of e1, input relu(h).
       put_rows(sD, row, 0, ft, de);
       put_rows(sX, row, 0, ft, x);
-      __syncthreads();
+      fetch(b < 3 ? (b == 1 ? g.se1 + kFW : g.se1) : g.sz + (kFDepth - 2) * kFW);
+      landed();
       wgrad(l1, 0, 32, 0, 64, 0, true, first);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         float z[4][4];
-        delta_w<2>(uD, warp, 0, a.wp + a.pk.off[l1] + (size_t)h * 2 * 4 * 768, lane, z);
+        delta_w<2>(uD, warp, 0, sW + h * 2 * 4 * 768, lane, z);
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
@@ -1360,19 +1392,25 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
     for (int j = kFDepth - 1; j >= 1; --j) {
       act_rows(g.sz + (j - 1) * kFW, x);
       __syncthreads();
+      stage(j, 0, kBwdW);
       put_rows(sD, row, 0, ft, d);
       put_rows(sX, row, 0, ft, x);
-      __syncthreads();
-      wgrad(j, 0, 64, 0, 64, 0, true, first);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      if (j >= 2) fetch(g.sz + (j - 2) * kFW);
+      landed();
+      auto product = [&](int h) {
         float z[4][4];
-        delta_w<4>(uD, warp, 0, a.wp + a.pk.off[j] + (size_t)h * 4 * 4 * 768, lane, z);
+        delta_w<4>(uD, warp, 0, sW, lane, z);
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
           for (int i = 0; i < 4; ++i) d[4 * h + nt][i] = x[4 * h + nt][i] > 0.0f ? z[nt][i] : 0.0f;
-      }
+      };
+      product(0);
+      __syncthreads();
+      stage(j, kBwdW, kBwdW);
+      wgrad(j, 0, 64, 0, 64, 0, true, first);
+      landed();
+      product(1);
     }
     // First layer: input f, 64 columns (two levels) at a time; d f.
 #pragma unroll 1
@@ -1386,19 +1424,25 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
         x[nt][0] = u0.x; x[nt][1] = u0.y; x[nt][2] = u1.x; x[nt][3] = u1.y;
       }
       __syncthreads();
+      stage(0, c0 / 32 * kBwdW, kBwdW);
       if (c0 == 0) put_rows(sD, row, 0, ft, d);
       put_rows(sX, row, 0, ft, x);
-      __syncthreads();
-      wgrad(0, 0, 64, 0, wide ? 64 : 32, c0, c0 == 0, first);
+      landed();
       for (int h = 0; h < (wide ? 2 : 1); ++h) {
+        if (h == 1) landed();
         float z[4][4];
-        delta_w<4>(uD, warp, 0, a.wp + a.pk.off[0] + (size_t)(c0 / 32 + h) * 4 * 4 * 768, lane, z);
+        delta_w<4>(uD, warp, 0, sW, lane, z);
 #pragma unroll
         for (int r2 = 0; r2 < 2; ++r2)
           if (valid[r2])
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt)
               *reinterpret_cast<float2*>(a.df + (size_t)p[r2] * nf + c0 + 32 * h + 8 * nt + 2 * ft) = make_float2(z[nt][2 * r2], z[nt][2 * r2 + 1]);
+        if (h == 0) {
+          __syncthreads();
+          if (wide) stage(0, (c0 / 32 + 1) * kBwdW, kBwdW);
+          wgrad(0, 0, 64, 0, wide ? 64 : 32, c0, c0 == 0, first);
+        }
       }
     }
   }
