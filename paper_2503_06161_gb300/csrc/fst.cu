@@ -202,19 +202,17 @@ __global__ void fst_pack_kernel(const FstGeom g, const float* __restrict__ mlp, 
 // Block products.  A block holds 128 Gaussians; activations live in shared
 // memory row-major per Gaussian ([128][kFRow] floats).
 //
-// Forward (256 threads): a warp owns a 32-row x (4 TN)-column tile, lane
-// (lane / 4, lane % 4) its rows row0 + 8 r (r < 4) and TN consecutive columns
-// from n0.  Per step of four inputs a lane reads four 16-byte row slices and
-// TN weights per input and issues 4 TN / 2 packed FMAs per input.  The
-// square warp tile is what the shared-memory pipe wants: its 8 row slices and
-// its 4 weight slices are one or two wavefronts each (12 wavefronts per
-// 64 packed FMAs at TN = 8), where a warp of 32 rows and one column group
-// took 32 and was bound by them.
+// Eight warps: warp w owns TN consecutive columns from w TN, lane l the rows
+// l + 32 r (r < 4).  Per step of four inputs a lane reads four 16-byte row
+// slices (four wavefronts each) and, uniformly over the warp, TN weights per
+// input (16-byte broadcasts, one wavefront each), and issues 4 TN / 2 packed
+// FMAs per input.  The shared-memory pipe decides the shape: at TN = 8 it is
+// 24 wavefronts per 64 FMAs.
 // ---------------------------------------------------------------------------
-template <int TN, int TM = 8>
-__device__ __forceinline__ void tile_zero(float2 (&acc)[TM][TN / 2]) {
+template <int TN>
+__device__ __forceinline__ void tile_zero(float2 (&acc)[4][TN / 2]) {
 #pragma unroll
-  for (int r = 0; r < TM; ++r)
+  for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < TN / 2; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
 }
@@ -235,23 +233,23 @@ __device__ __forceinline__ void lds_pairs(const float* p, float2 (&v)[N / 2]) {
   }
 }
 
-// acc[r][c] += sum_k X[(row0 + RS r) * kFRow + k] * B[k * ldb + n0 + (2c, 2c+1)],
+// acc[r][c] += sum_k X[(row0 + 32 r) * kFRow + k] * B[k * ldb + n0 + (2c, 2c+1)],
 // k < K (multiple of 8) in increasing order; B in shared memory, its rows
 // aligned to the widest load at n0.
-template <int TN, int TM, int RS>
+template <int TN>
 __device__ __forceinline__ void tile_mma(const float* X, int K, const float* B, int ldb, int row0, int n0,
-                                         float2 (&acc)[TM][TN / 2]) {
+                                         float2 (&acc)[4][TN / 2]) {
 #pragma unroll 2
   for (int k = 0; k < K; k += 4) {
-    float4 xv[TM];
+    float4 xv[4];
 #pragma unroll
-    for (int r = 0; r < TM; ++r) xv[r] = *reinterpret_cast<const float4*>(X + (row0 + RS * r) * kFRow + k);
+    for (int r = 0; r < 4; ++r) xv[r] = *reinterpret_cast<const float4*>(X + (row0 + 32 * r) * kFRow + k);
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
       float2 b[TN / 2];
       lds_pairs<TN>(B + (size_t)(k + kk) * ldb + n0, b);
 #pragma unroll
-      for (int r = 0; r < TM; ++r) {
+      for (int r = 0; r < 4; ++r) {
         const float xk = kk == 0 ? xv[r].x : (kk == 1 ? xv[r].y : (kk == 2 ? xv[r].z : xv[r].w));
         const float2 x2 = make_float2(xk, xk);
 #pragma unroll
@@ -262,32 +260,39 @@ __device__ __forceinline__ void tile_mma(const float* X, int K, const float* B, 
 }
 
 // Layer epilogue of the forward: z = acc + bias; relu(z) -> Y (shared, column
-// offset yc) and -> the Gaussians' activation rows (valid rows only).  The
-// reverse pass needs only relu(z): it is the next layer's input, and z > 0 iff
-// relu(z) > 0.
+// offset yc).
 template <int TN>
 __device__ __forceinline__ void tile_out(const float2 (&acc)[4][TN / 2], const float* __restrict__ bias, int row0,
-                                         int n0, float* act, int nslots, int P, int slot, int p0, float* Y, int yc) {
+                                         int n0, float* Y, int yc) {
   float2 bb[TN / 2];
 #pragma unroll
   for (int c = 0; c < TN / 2; ++c) bb[c] = __ldg(reinterpret_cast<const float2*>(bias + n0) + c);
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
-    const int m = row0 + 8 * r;
     float z[TN];
 #pragma unroll
     for (int c = 0; c < TN / 2; ++c) {
       z[2 * c] = fmaxf(acc[r][c].x + bb[c].x, 0.0f);
       z[2 * c + 1] = fmaxf(acc[r][c].y + bb[c].y, 0.0f);
     }
-    if (p0 + m < P) {
-      float4* o = reinterpret_cast<float4*>(act + (size_t)(p0 + m) * nslots + slot + n0);
-#pragma unroll
-      for (int c = 0; c < TN; c += 4) o[c / 4] = make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
-    }
 #pragma unroll
     for (int c = 0; c < TN; c += 4)
-      *reinterpret_cast<float4*>(Y + m * kFRow + yc + n0 + c) = make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
+      *reinterpret_cast<float4*>(Y + (row0 + 32 * r) * kFRow + yc + n0 + c) = make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
+  }
+}
+
+// Columns [yc, yc + N) of the block's rows of Y -> the Gaussians' activation
+// rows from `slot` (whole 16-byte units, consecutive lanes along a row).  The
+// reverse pass needs only relu(z): it is the next layer's input, and z > 0 iff
+// relu(z) > 0.
+template <int N>
+__device__ __forceinline__ void keep_rows(const float* Y, int yc, float* act, int nslots, int slot, int p0, int P) {
+#pragma unroll 4
+  for (int i = threadIdx.x; i < kFM * (N / 4); i += kFwdThreads) {
+    const int r = i / (N / 4), q = i % (N / 4);
+    if (p0 + r < P)
+      *reinterpret_cast<float4*>(act + (size_t)(p0 + r) * nslots + slot + 4 * q) =
+          *reinterpret_cast<const float4*>(Y + r * kFRow + yc + 4 * q);
   }
 }
 
@@ -467,11 +472,9 @@ constexpr size_t kFwdSmem = ((size_t)2 * kFM * kFRow + 2 * kWBuf) * 4;
 
 template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a) {
-  // 256 threads over 128 Gaussians: warp w owns rows [32 (w / 2), + 32) and
-  // half (w % 2) of the columns of every product (see above); threads below
-  // 128 also own Gaussian p0 + tid for the per-Gaussian parts (f rows, heads,
-  // outputs).
-  constexpr int TM = 4;
+  // 256 threads over 128 Gaussians: rows and columns of the products as above;
+  // threads below 128 also own Gaussian p0 + tid for the per-Gaussian parts (f
+  // rows, heads, outputs).
   extern __shared__ __align__(16) float s_buf[];
   float* A = s_buf;                        // [128][kFRow]
   float* B = s_buf + kFM * kFRow;          // [128][kFRow]
@@ -480,11 +483,10 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
   stage_tile(a.tiles, a.ntiles, 0, a.wt, wbuf);
   const FstGeom& g = a.g;
   const int tid = threadIdx.x;
-  const int warp = tid >> 5, lane = tid & 31;
-  const int row0 = 32 * (warp >> 1) + (lane >> 2), nt = 4 * (warp & 1) + (lane & 3);
-  const bool owner = tid < kFM;
+  const int row0 = tid & 31, nt = tid >> 5;
   const int p0 = blockIdx.x * kFM;
   const int p = p0 + tid;
+  const bool owner = tid < kFM;
   const bool valid = owner && p < g.P;
   const int P = g.P;
   float* act = a.act;
@@ -496,8 +498,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
   // F_out layer 0 over f (written Gaussian-major by the sampling kernel),
   // two levels (64 columns) at a time, copied into A asynchronously.
   const int nf = g.levels * kFC;
-  float2 acc[TM][4];
-  tile_zero<8, TM>(acc);
+  float2 acc[4][4];
+  tile_zero<8>(acc);
   for (int l0 = 0; l0 < g.levels; l0 += 2) {
     const int nl = g.levels - l0 < 2 ? g.levels - l0 : 2;
     if (owner) {
@@ -508,43 +510,47 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
     __syncthreads();
     {
       const float* w = next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf);
-      tile_mma<8, TM, 8>(A, nl * kFC, w, kFW, row0, nt * 8, acc);
+      tile_mma<8>(A, nl * kFC, w, kFW, row0, nt * 8, acc);
     }
     __syncthreads();
   }
-  tile_out<8>(acc, a.wt + g.ab[0], row0, nt * 8, act, g.nslots, P, g.sz, p0, B, 0);
+  tile_out<8>(acc, a.wt + g.ab[0], row0, nt * 8, B, 0);
   __syncthreads();
+  keep_rows<kFW>(B, 0, act, g.nslots, g.sz, p0, P);
   // z_j = W_j relu(z_{j-1}) + b_j; layer j reads (j odd ? B : A).
   for (int j = 1; j < kFDepth; ++j) {
     float* src = (j & 1) ? B : A;
     float* dst = (j & 1) ? A : B;
-    tile_zero<8, TM>(acc);
-    tile_mma<8, TM, 8>(src, kFW, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFW, row0, nt * 8, acc);
-    tile_out<8>(acc, a.wt + g.ab[j], row0, nt * 8, act, g.nslots, P, g.sz + j * kFW, p0, dst, 0);
+    tile_zero<8>(acc);
+    tile_mma<8>(src, kFW, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFW, row0, nt * 8, acc);
+    tile_out<8>(acc, a.wt + g.ab[j], row0, nt * 8, dst, 0);
     __syncthreads();
+    keep_rows<kFW>(dst, 0, act, g.nslots, g.sz + j * kFW, p0, P);
   }
   // relu(h) is in A.  Branches: e1 -> B[0, 32), h_g -> B[32, 64); the
   // semantic updater's first layer accumulates over the branches.
-  float2 v[TM][4];
-  tile_zero<8, TM>(v);
+  float2 v[4][4];
+  tile_zero<8>(v);
   float out[11];
 #pragma unroll
   for (int b = 0; b < 4; ++b) {
     const int l1 = branch_e1(b);
     {
-      float2 e[TM][2];
-      tile_zero<4, TM>(e);
-      tile_mma<4, TM, 8>(A, kFW, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFHalf, row0, nt * 4, e);
-      tile_out<4>(e, a.wt + g.ab[l1], row0, nt * 4, act, g.nslots, P, g.se1 + b * kFHalf, p0, B, 0);
+      float2 e[4][2];
+      tile_zero<4>(e);
+      tile_mma<4>(A, kFW, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFHalf, row0, nt * 4, e);
+      tile_out<4>(e, a.wt + g.ab[l1], row0, nt * 4, B, 0);
     }
     __syncthreads();
     {
-      float2 e[TM][2];
-      tile_zero<4, TM>(e);
-      tile_mma<4, TM, 8>(B, kFHalf, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFHalf, row0, nt * 4, e);
-      tile_out<4>(e, a.wt + g.ab[l1 + 1], row0, nt * 4, act, g.nslots, P, g.shg + b * kFHalf, p0, B, kFHalf);
+      float2 e[4][2];
+      tile_zero<4>(e);
+      tile_mma<4>(B, kFHalf, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFHalf, row0, nt * 4, e);
+      tile_out<4>(e, a.wt + g.ab[l1 + 1], row0, nt * 4, B, kFHalf);
     }
     __syncthreads();
+    keep_rows<kFHalf>(B, 0, act, g.nslots, g.se1 + b * kFHalf, p0, P);
+    keep_rows<kFHalf>(B, kFHalf, act, g.nslots, g.shg + b * kFHalf, p0, P);
     // Head (the owner thread's own Gaussian): offset = H relu(h_g) + b.
     constexpr int dgs[4] = {3, 4, 3, 1}, oos[4] = {0, 3, 7, 10};
     if (owner) {
@@ -565,24 +571,25 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
             if (o < dgs[b]) out[oos[b] + o] = fmaf(__ldg(wt_h + (i4 + i) * dgs[b] + o), hv[i], out[oos[b] + o]);
       }
     }
-    tile_mma<8, TM, 8>(B + kFHalf, kFHalf, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFW, row0, nt * 8, v);
+    tile_mma<8>(B + kFHalf, kFHalf, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), kFW, row0, nt * 8, v);
     __syncthreads();
   }
-  tile_out<8>(v, a.wt + g.ab[kLZ1], row0, nt * 8, act, g.nslots, P, g.sv, p0, A, 0);
+  tile_out<8>(v, a.wt + g.ab[kLZ1], row0, nt * 8, A, 0);
   __syncthreads();
+  keep_rows<kFW>(A, 0, act, g.nslots, g.sv, p0, P);
   // dz = Z2 relu(v) + b, 64 columns at a time.
   constexpr int ZN = D < 64 ? D : 64, ZT = ZN / 8;
 #pragma unroll
   for (int c0 = 0; c0 < D; c0 += ZN) {
-    float2 z[TM][ZT / 2];
-    tile_zero<ZT, TM>(z);
-    tile_mma<ZT, TM, 8>(A, kFW, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), ZN, row0, nt * ZT, z);
+    float2 z[4][ZT / 2];
+    tile_zero<ZT>(z);
+    tile_mma<ZT>(A, kFW, next_tile(a.tiles, a.ntiles, wt_i, a.wt, wbuf), ZN, row0, nt * ZT, z);
     float2 bb[ZT / 2];
 #pragma unroll
     for (int c = 0; c < ZT / 2; ++c) bb[c] = __ldg(reinterpret_cast<const float2*>(a.wt + g.ab[kLZ2] + c0 + nt * ZT) + c);
 #pragma unroll
-    for (int r = 0; r < TM; ++r) {
-      const int pm = p0 + row0 + 8 * r;
+    for (int r = 0; r < 4; ++r) {
+      const int pm = p0 + row0 + 32 * r;
       if (pm < P) {
 #pragma unroll
         for (int c = 0; c < ZT / 2; ++c) {
