@@ -427,23 +427,30 @@ __global__ void __launch_bounds__(kThreads, 2) gauss_fwd_kernel(const GaussArgs 
 // sums to psum[g].  The entries of consecutive depth ranks occupy
 // consecutive emission ranges, so one warp takes ranks_per_warp(D) consecutive
 // ranks: one coalesced load of their ranges, one of the bitmask words of
-// the whole range (read back by shuffle), then the written rows streamed RG
+// the whole range, from which the lanes together list the written rows (most
+// entries have none: nothing reached them).  The rows are then streamed RG
 // at a time (all RG rows' loads in flight before any is added), lane c
 // adding column c (and c + 32, ...).  Each Gaussian's rows are added one
 // after another in increasing emission order: a fixed order, so the result
-// is bitwise reproducible.
+// is bitwise reproducible.  Bound by the latency of each warp's three
+// dependent loads (ranges, words, rows), so the chip is kept full of warps;
+// finding the next set bit row by row had it at 217 warp instructions per
+// Gaussian (1M Gaussians, D = 64: 256 us, now 218 from launch to end,
+// overlapping the kernel before it).
 // Ranks per warp: 8 for rows of at most 64 floats (D <= 52), else 4
 // (measured best at D = 32 and D = 128).
 __host__ __device__ constexpr int ranks_per_warp(int D) { return (partial_stride(D) + 31) / 32 <= 2 ? 8 : 4; }
 
 template <int D>
-__global__ void __launch_bounds__(kThreads, 3) partial_reduce_kernel(const GaussBwdArgs b, int P) {
+__global__ void __launch_bounds__(kThreads, 4) partial_reduce_kernel(const GaussBwdArgs b, int P) {
   grid_dep_wait();
   grid_dep_launch();
   constexpr int NP = partial_stride(D);
   constexpr int NQ = (NP + 31) / 32;  // columns per lane
-  constexpr int RG = NQ <= 2 ? 16 : (NQ <= 4 ? 8 : 4);  // rows in flight
+  constexpr int RG = NQ <= 4 ? 8 : 4;  // rows in flight
+  __shared__ uint16_t s_rows[kThreads / 32][1024];  // written rows of 32 bitmask words
   const int lane = threadIdx.x & 31;
+  uint16_t* rows = s_rows[threadIdx.x >> 5];
   constexpr int GPW = ranks_per_warp(D);
   const int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * GPW;
   if (r0 >= P) return;
@@ -456,16 +463,6 @@ __global__ void __launch_bounds__(kThreads, 3) partial_reduce_kernel(const Gauss
   const uint32_t eend = mine ? (uint32_t)min((uint64_t)b.offs[r0 + lane + 1], cap) : 0u;
   const uint32_t E0 = __shfl_sync(0xFFFFFFFFu, ebeg, 0);
   const uint32_t E1 = __shfl_sync(0xFFFFFFFFu, eend, nvalid - 1);
-  // Bitmask words of the range: word wbase + l in lane l (the rest, for a
-  // range of more than 32 words, read when reached).
-  const uint32_t wbase = E0 >> 5;
-  const uint32_t wlast = E0 < E1 ? (E1 - 1) >> 5 : wbase;
-  const uint32_t wl = (E0 < E1 && wbase + (uint32_t)lane <= wlast) ? __ldg(b.pflags + wbase + lane) : 0u;
-  auto word = [&](uint32_t w) -> uint32_t {
-    const uint32_t k = w - wbase;
-    const uint32_t v = __shfl_sync(0xFFFFFFFFu, wl, (int)(k & 31u));
-    return k < 32u ? v : __ldg(b.pflags + w);
-  };
   float acc[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) acc[q] = 0.0f;
@@ -488,42 +485,46 @@ __global__ void __launch_bounds__(kThreads, 3) partial_reduce_kernel(const Gauss
     ++j;
     jend = __shfl_sync(0xFFFFFFFFu, eend, j < nvalid ? j : nvalid - 1);
   };
-  // Word w of the bitmask, m its bits not yet taken.
-  uint32_t w = wbase;
-  uint32_t m = E0 < E1 ? word(w) & (~0u << (E0 & 31u)) : 0u;
-  bool done = E0 >= E1;
-  while (!done) {
-    // The next RG written rows (warp-uniform; slot u holds one if has[u]).
-    uint32_t idx[RG];
-    bool has[RG];
+  const uint32_t wlast = E0 < E1 ? (E1 - 1) >> 5 : 0u;
+  for (uint32_t w0 = E0 >> 5; E0 < E1 && w0 <= wlast; w0 += 32) {
+    const uint32_t w = w0 + (uint32_t)lane;
+    uint32_t m = w <= wlast ? __ldg(b.pflags + w) : 0u;
+    if (w == E0 >> 5) m &= ~0u << (E0 & 31u);
+    if (w == wlast && (E1 & 31u)) m &= (1u << (E1 & 31u)) - 1u;
+    uint32_t pos = (uint32_t)__popc(m);
+    const uint32_t mine_n = pos;
 #pragma unroll
-    for (int u = 0; u < RG; ++u) {
-      while (!done && m == 0u) {
-        ++w;
-        if (w > wlast) done = true;
-        else m = word(w);
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, pos, o);
+      if (lane >= o) pos += y;
+    }
+    const int n = (int)__shfl_sync(0xFFFFFFFFu, pos, 31);
+    pos -= mine_n;
+    while (m) {
+      rows[pos++] = (uint16_t)(lane * 32 + __ffs(m) - 1);
+      m &= m - 1u;
+    }
+    __syncwarp();
+    for (int r = 0; r < n; r += RG) {
+      uint32_t idx[RG];
+      float x[RG][NQ];
+#pragma unroll
+      for (int u = 0; u < RG; ++u) {
+        idx[u] = (w0 << 5) + rows[min(r + u, n - 1)];
+        const float* row = b.partials + (size_t)idx[u] * NP;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) x[u][q] = (r + u < n && lane + 32 * q < NP) ? __ldg(row + lane + 32 * q) : 0.0f;
       }
-      const uint32_t e = (w << 5) + (uint32_t)(__ffs(m) - 1);
-      has[u] = !done && e < E1;
-      if (!done && e >= E1) done = true;
-      idx[u] = has[u] ? e : 0u;
-      if (has[u]) m &= m - 1u;
-    }
-    float x[RG][NQ];
 #pragma unroll
-    for (int u = 0; u < RG; ++u) {
-      const float* row = b.partials + (size_t)idx[u] * NP;
+      for (int u = 0; u < RG; ++u) {
+        if (r + u < n) {
+          while (idx[u] >= jend) flush();  // rows belong to the Gaussians in order
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) x[u][q] = (has[u] && lane + 32 * q < NP) ? __ldg(row + lane + 32 * q) : 0.0f;
-    }
-#pragma unroll
-    for (int u = 0; u < RG; ++u) {
-      if (has[u]) {
-        while (idx[u] >= jend) flush();  // rows belong to the Gaussians in order
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) acc[q] += x[u][q];
+          for (int q = 0; q < NQ; ++q) acc[q] += x[u][q];
+        }
       }
     }
+    __syncwarp();
   }
   while (j < nvalid) flush();  // the last Gaussian with rows, and any after it without
 }
