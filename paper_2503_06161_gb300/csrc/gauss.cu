@@ -722,12 +722,15 @@ __global__ void __launch_bounds__(kThreads, 2) gauss_bwd_proj_kernel(const Gauss
 // Mean gradient through the HexPlane grid (Sec. 3.2, Eq. 4-6): dL/df (written
 // by the MLP reverse) through the product of the six bilinear samples to the
 // three coordinates.  The lanes of a Gaussian (see gather_lanes) each take
-// four channels: the products of the other five planes by prefix / suffix
-// products (no division), summed per axis, then over the lanes by a fixed
-// shuffle tree.  200k Gaussians, C = 32: 59 us, 86 us with lanes over channels
-// and twelve warp sums per Gaussian; 1,500 Gaussians: 3 us instead of 21.
+// four channels: the product and its three derivatives carried from plane to
+// plane (product rule, no division), summed over the channels, then over the
+// lanes by a fixed shuffle tree.  Bound by the latency of the texel gathers,
+// so registers decide: at 64 (four blocks per SM) 1M Gaussians, C = 32, take
+// 257 us, 286 at 80 registers, 385 at 124; prefix and suffix products of all
+// planes held 72 floats more.  200k: 86 us with lanes over channels and twelve
+// warp sums per Gaussian, 59 with two blocks.
 template <int C>
-__global__ void __launch_bounds__(kThreads, 2) gauss_bwd_deform_kernel(const GaussArgs a, const GaussBwdArgs b,
+__global__ void __launch_bounds__(kThreads, 4) gauss_bwd_deform_kernel(const GaussArgs a, const GaussBwdArgs b,
                                                                      const float* __restrict__ df_all) {
   grid_dep_wait();
   grid_dep_launch();
@@ -744,36 +747,38 @@ __global__ void __launch_bounds__(kThreads, 2) gauss_bwd_deform_kernel(const Gau
     const AxisPos ap = axis_pos(a, mu);
     const float4 df4 = __ldg(reinterpret_cast<const float4*>(df_all) + (size_t)g * LG + q);
     const float df[4] = {df4.x, df4.y, df4.z, df4.w};
-    float sv[6][4], d0[6][4], d1[6][4];
+    // The product of the six planes and its derivatives by x, y, z, one
+    // plane after another.
+    float pr[4], dp[3][4];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      const float f0 = ap.f[pair_a(k)], f1 = ap.f[pair_b(k)];
+      const int ia = pair_a(k), ib = pair_b(k);
+      const float f0 = ap.f[ia], f1 = ap.f[ib];
       float4 x[4];  // 00, 01, 10, 11
       corners<C>(a, ap, k, q, x);
       const float x00[4] = {x[0].x, x[0].y, x[0].z, x[0].w}, x01[4] = {x[1].x, x[1].y, x[1].z, x[1].w};
       const float x10[4] = {x[2].x, x[2].y, x[2].z, x[2].w}, x11[4] = {x[3].x, x[3].y, x[3].z, x[3].w};
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        sv[k][c] = (1.f - f0) * (1.f - f1) * x00[c] + f0 * (1.f - f1) * x10[c] + (1.f - f0) * f1 * x01[c] + f0 * f1 * x11[c];
-        d0[k][c] = (1.f - f1) * (x10[c] - x00[c]) + f1 * (x11[c] - x01[c]);
-        d1[k][c] = (1.f - f0) * (x01[c] - x00[c]) + f0 * (x11[c] - x10[c]);
+        const float sv = (1.f - f0) * (1.f - f1) * x00[c] + f0 * (1.f - f1) * x10[c] + (1.f - f0) * f1 * x01[c] + f0 * f1 * x11[c];
+        const float da = (1.f - f1) * (x10[c] - x00[c]) + f1 * (x11[c] - x01[c]);
+        const float db = (1.f - f0) * (x01[c] - x00[c]) + f0 * (x11[c] - x10[c]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const bool on_a = i == ia, on_b = i == ib;  // (axis 3 is time)
+          if (k == 0) {
+            dp[i][c] = on_a ? da : on_b ? db : 0.0f;
+          } else {
+            const float t = dp[i][c] * sv;
+            dp[i][c] = on_a ? fmaf(pr[c], da, t) : on_b ? fmaf(pr[c], db, t) : t;
+          }
+        }
+        pr[c] = k == 0 ? sv : pr[c] * sv;
       }
     }
-    float dg[4] = {0.f, 0.f, 0.f, 0.f};  // d L / d(grid position) of each axis
+    float dg[3];  // d L / d(grid position) of each axis
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float pre[6], suf = df[c];
-      pre[0] = 1.0f;
-#pragma unroll
-      for (int k = 1; k < 6; ++k) pre[k] = pre[k - 1] * sv[k - 1][c];
-#pragma unroll
-      for (int k = 5; k >= 0; --k) {
-        const float ds = pre[k] * suf;
-        dg[pair_a(k)] = fmaf(ds, d0[k][c], dg[pair_a(k)]);
-        dg[pair_b(k)] = fmaf(ds, d1[k][c], dg[pair_b(k)]);
-        suf *= sv[k][c];
-      }
-    }
+    for (int i = 0; i < 3; ++i) dg[i] = df[0] * dp[i][0] + df[1] * dp[i][1] + df[2] * dp[i][2] + df[3] * dp[i][3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) dc[i] = ap.clamped[i] ? 0.0f : dg[i];
   }
