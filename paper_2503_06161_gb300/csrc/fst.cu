@@ -1585,8 +1585,17 @@ __global__ void fst_reduce_kernel(const FstGeom g, const float* __restrict__ par
     int k = 0;
     while (k + 1 < kFLayers && e >= g.pw[k + 1]) ++k;
     const int64_t src = e < g.pb[k] ? g.aw[k] + (e - g.pw[k]) : g.ab[k] + (e - g.pb[k]);
+    // Sixteen loads in flight, added in block order.
     float s = 0.0f;
-    for (int b = 0; b < nblk; ++b) s += part[(size_t)b * g.mlp_aligned + src];
+    int b = 0;
+    for (; b + 16 <= nblk; b += 16) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = __ldg(part + (size_t)(b + u) * g.mlp_aligned + src);
+#pragma unroll
+      for (int u = 0; u < 16; ++u) s += v[u];
+    }
+    for (; b < nblk; ++b) s += part[(size_t)b * g.mlp_aligned + src];
     out[e] = s;
   }
 }
@@ -1655,9 +1664,13 @@ __global__ void __launch_bounds__(256) fst_tv_kernel(const TvArgs a) {
 }
 
 __global__ void fst_tv_finish(const float* __restrict__ partial, int n, float weight, float* __restrict__ loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
+  // Staged by the whole block, then added in order by one thread.
+  __shared__ float s_part[kTvMaxBlocks];
+  for (int b = threadIdx.x; b < n; b += blockDim.x) s_part[b] = partial[b];
+  __syncthreads();
+  if (threadIdx.x == 0) {
     float s = 0.0f;
-    for (int b = 0; b < n; ++b) s += partial[b];
+    for (int b = 0; b < n; ++b) s += s_part[b];
     *loss = weight * s;
   }
 }
@@ -1960,6 +1973,6 @@ extern "C" fe_status fe_fst_tv(const fe_fst* fst, float weight, float* loss, flo
   }
   const int nblk = a.bstart[np];
   fst_tv_kernel<<<nblk, 256, 0, st>>>(a);
-  fst_tv_finish<<<1, 32, 0, st>>>(scratch, nblk, weight, loss);
+  fst_tv_finish<<<1, 256, 0, st>>>(scratch, nblk, weight, loss);
   return cudaGetLastError() == cudaSuccess ? FE_OK : FE_ERR_CUDA;
 }
