@@ -25,9 +25,10 @@ namespace {
 // Gaussians per staged batch of the forward (two batches are in flight) and
 // blocks per SM.  Most tiles end within the first 200 entries of their list,
 // so at D = 32 batches of 64 land sooner and load less past the end (200k
-// Gaussians, 640 x 512: 170 us, 176 with 128, 182 with 32); at D = 16 two
-// blocks with room for registers beat three (30k, 333 x 251: 66 us against
-// 74), at D = 32 they are even.
+// Gaussians, 640 x 512: 167 us, 176 with 128, 182 with 32); at D = 16 two
+// blocks with room for registers and batches of 128 are the faster (30k,
+// 333 x 251: 57 us; three blocks 68, batches of 64 66), at D = 32 two and
+// three blocks are even.
 template <int D>
 constexpr int fwd_batch() { return D == 16 ? 128 : (D <= 64 ? 64 : 32); }
 template <int D>
@@ -255,27 +256,35 @@ __device__ __forceinline__ void fwd_tile(const CompositeArgs& a, const int tile,
         // Groups of 32 entries; the entries the warp's block may blend are
         // taken in order, two at a time: both evaluated ahead of their
         // (ordered) blending -- the two evaluations are independent, only
-        // the blend carries T.
+        // the blend carries T.  One code path for full and half pairs and one
+        // exit (a second path for a single last entry and breaks out of each
+        // cost 5 to 14%: 30k Gaussians at 333 x 251, D = 16, 66 -> 57 us;
+        // 90k, D = 128, 483 -> 453; 1M at 1280 x 1024, D = 64, 744 -> 717).
+        // Bound by the latency of this loop (evaluation, then the blends in
+        // order); four at a time are no faster, and evaluating a pair ahead
+        // of the previous one's blends is slower (61 us for the 57).
         for (int g = 0; g < NG && !done; ++g) {
           uint32_t t = g == 0 ? em0 : g == 1 ? em1 : g == 2 ? em2 : em3;
           cur = 0u;
           while (t) {
-            const int ja = 32 * g + __ffs(t) - 1;
-            t &= t - 1u;
-            PairEval p0, p1;
             // Evaluations without early exits, so that they interleave
-            // (identical arithmetic and decisions to eval_pair).
-            const bool h0 = eval_pair_flat(s_rec + ja * kRec, pxc, pyc, p0);
-            if (t) {
-              const int jb = 32 * g + __ffs(t) - 1;
+            // (identical arithmetic and decisions to eval_pair); a missing
+            // second entry evaluates the group's first and is not blended.
+            int j[2];
+            bool h[2];
+            PairEval pe[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const bool have = t != 0u;
+              j[u] = 32 * g + (have ? __ffs(t) - 1 : 0);
               t &= t - 1u;
-              const bool h1 = eval_pair_flat(s_rec + jb * kRec, pxc, pyc, p1);
-              if (h0 && blend(ja, p0)) break;
-              if (h1 && blend(jb, p1)) break;
-            } else if (h0 && blend(ja, p0)) {
-              break;
+              h[u] = eval_pair_flat(s_rec + j[u] * kRec, pxc, pyc, pe[u]) && have;
             }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+              if (h[u] && blend(j[u], pe[u])) goto ended;
           }
+        ended:
           cm0 |= g == 0 ? cur : 0u;
           if (NG > 1) cm1 |= g == 1 ? cur : 0u;
           if (NG > 2) cm2 |= g == 2 ? cur : 0u;
