@@ -106,15 +106,17 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* __re
                                                             const uint32_t* n_dev, int64_t n_cap, int shift,
                                                             const uint32_t* __restrict__ hist, uint32_t* status,
                                                             uint32_t* ticket, uint32_t* err) {
-  grid_dep_wait();
-  grid_dep_launch();
   constexpr int CHUNK = kThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PassSmem<ITEMS>& sm = *reinterpret_cast<PassSmem<ITEMS>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // Before the wait for the previous pass: the counters' zeros and the
+  // ticket (its counter is cleared ahead of the whole chain of launches).
   for (int i = tid; i < 8 * 256; i += kThreads) (&sm.wcnt[0][0])[i] = 0;
   if (tid == 0) sm.ticket = atomicAdd(ticket, 1u);
   __syncthreads();
+  grid_dep_wait();
+  grid_dep_launch();
   const uint32_t b = sm.ticket;
   const uint64_t n = n_dev ? min((uint64_t)*n_dev, (uint64_t)n_cap) : (uint64_t)n_cap;
   const uint64_t start = (uint64_t)b * CHUNK;
@@ -124,12 +126,18 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* __re
   uint32_t k[ITEMS], v[ITEMS], rk[ITEMS];
   int dg[ITEMS];
   const uint64_t wbase = start + (uint64_t)warp * (CHUNK / 8);
+  // All loads in flight before the first key is ranked.
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const uint64_t idx = wbase + (uint64_t)r * 32 + lane;
+    k[r] = idx < n ? keys_in[idx] : 0u;
+    v[r] = idx < n ? (kIdentVals ? (uint32_t)idx : vals_in[idx]) : 0u;
+  }
 #pragma unroll
   for (int r = 0; r < ITEMS; ++r) {
     const uint64_t idx = wbase + (uint64_t)r * 32 + lane;
     const bool valid = idx < n;
-    const uint32_t key = valid ? keys_in[idx] : 0u;
-    const uint32_t val = valid ? (kIdentVals ? (uint32_t)idx : vals_in[idx]) : 0u;
+    const uint32_t key = k[r];
     const int d = valid ? (int)((key >> shift) & 255u) : 256;
     const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
     const int lead = __ffs(peers) - 1;
@@ -139,8 +147,6 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* __re
     if (valid && lane == lead) sm.wcnt[warp][d] = base + __popc(peers);
     __syncwarp();
     rk[r] = base + __popc(peers & lanemask_lt());
-    k[r] = key;
-    v[r] = val;
     dg[r] = d;
   }
   __syncthreads();
