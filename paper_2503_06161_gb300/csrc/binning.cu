@@ -14,6 +14,8 @@
 // ties by index, built with one write per entry instead of radix passes over
 // 64-bit keys.  Every inter-block wait is a bounded spin that records
 // kErrTimeout and carries on, so no launch can hang.
+#include <atomic>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -214,6 +216,211 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* __re
     keys_out[gp] = key;
     vals_out[gp] = sm.vals[i];
   }
+}
+
+// ---------------------------------------------------------------------------
+// The same sort in one launch, for the few keys that one cluster of blocks
+// holds in registers: per pass every block ranks its keys, the blocks exchange
+// their digit counts through distributed shared memory behind a cluster
+// barrier, and the keys move by way of L2, in runs ordered in shared memory.
+// Bound by the latency of a pass (1.6 us in one block, 2.8 in sixteen with two
+// keys a thread); the five launches above, four of them with a chain of
+// look-back, are too, at 20 us for 1,000 keys and 37 for 30k, where this one
+// takes 6 and 11.  With more keys a thread the sixteen SMs fall behind the
+// whole chip (100k: 38 us against 35), so the line lies at three a thread
+// (640 x 512 frames, this sort against the passes: 1,000 Gaussians 53 and
+// 57 us, 10k 104 and 111, 32k 177 and 179, 48k 196 and 198, 64k 209 and 208).
+// ---------------------------------------------------------------------------
+constexpr int kSortThreads = 1024, kSortWarps = kSortThreads / 32;
+constexpr int kSortBlocks = 16;  // more than the eight that every device takes: see sort_blocks
+constexpr int kSortMaxItems = 3;
+
+template <int ITEMS>
+struct SortSmem {
+  uint32_t wcnt[kSortWarps][256];  // digit counts, then prefixes, per warp
+  uint32_t cnt[256];               // the block's digit counts (read by the cluster)
+  uint32_t gbase[256], bstart[256];
+  uint64_t scan[8];
+  uint32_t keys[kSortThreads * ITEMS], vals[kSortThreads * ITEMS];
+};
+
+struct SortArgs {
+  uint32_t *key0, *key1, *val0, *val1;  // key0: input; result in val0 (the last pass writes no keys)
+  int n;
+};
+
+// Word of block `rank` of the cluster at this block's shared address p.
+__device__ __forceinline__ uint32_t ld_cluster(const uint32_t* p, uint32_t rank) {
+  uint32_t a, v;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Block b of the cluster holds elements [b * 1024 items, ...), warp w of it 32
+// items consecutive ones; items <= ITEMS and gridDim.x * 1024 * items >= n.
+template <int ITEMS>
+__global__ void __launch_bounds__(kSortThreads, 1) cluster_sort_kernel(const SortArgs a, const int items) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SortSmem<ITEMS>& sm = *reinterpret_cast<SortSmem<ITEMS>*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t b = blockIdx.x, nb = gridDim.x;
+  const int first = (int)b * kSortThreads * items;
+  const int cnt = max(0, min(kSortThreads * items, a.n - first));
+  const int wfirst = warp * 32 * items + lane;  // within the block
+  grid_dep_wait();
+  grid_dep_launch();
+#pragma unroll 1
+  for (int p = 0; p < 4; ++p) {
+    const int shift = 8 * p;
+    const bool odd = p & 1;
+    const uint32_t* kin = odd ? a.key1 : a.key0;
+    const uint32_t* vin = odd ? a.val1 : a.val0;
+    uint32_t* kout = odd ? a.key0 : a.key1;
+    uint32_t* vout = odd ? a.val0 : a.val1;
+    uint32_t k[ITEMS], v[ITEMS], rk[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      const int i = wfirst + 32 * r;
+      const bool valid = r < items && i < cnt;
+      k[r] = valid ? __ldcg(kin + first + i) : 0u;
+      v[r] = valid ? (p == 0 ? (uint32_t)(first + i) : __ldcg(vin + first + i)) : 0u;
+    }
+    for (int i = tid; i < kSortWarps * 256; i += kSortThreads) (&sm.wcnt[0][0])[i] = 0u;
+    __syncthreads();
+    uint32_t* wc = sm.wcnt[warp];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      rk[r] = 0u;
+      if (r < items) {
+        const bool valid = wfirst + 32 * r < cnt;
+        const int d = valid ? (int)((k[r] >> shift) & 255u) : 256;
+        const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+        const uint32_t base = valid ? wc[d] : 0u;
+        __syncwarp();
+        if (valid && lane == __ffs(peers) - 1) wc[d] = base + __popc(peers);
+        __syncwarp();
+        rk[r] = base + __popc(peers & lanemask_lt());
+      }
+    }
+    __syncthreads();
+    // Digit tid: prefix over the warps and the block's count.
+    uint32_t bcount = 0;
+    if (tid < 256) {
+#pragma unroll
+      for (int w = 0; w < kSortWarps; ++w) {
+        const uint32_t c = sm.wcnt[w][tid];
+        sm.wcnt[w][tid] = bcount;
+        bcount += c;
+      }
+      sm.cnt[tid] = bcount;
+    }
+    cluster_barrier();
+    // Digit tid's count in the cluster and in the blocks before this one;
+    // exclusive scans over the digits of the cluster's and the block's counts.
+    uint32_t tot = 0, before = 0;
+    uint64_t own = 0, incl = 0;
+    if (tid < 256) {
+#pragma unroll
+      for (int c = 0; c < kSortBlocks; ++c) {
+        const uint32_t x = c < (int)nb ? ld_cluster(&sm.cnt[tid], (uint32_t)c) : 0u;
+        tot += x;
+        if (c < (int)b) before += x;
+      }
+      incl = own = ((uint64_t)tot << 32) | bcount;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (lane == 31) sm.scan[warp] = incl;
+    }
+    __syncthreads();
+    if (tid < 256) {
+      uint64_t ex = incl - own;
+      for (int w = 0; w < warp; ++w) ex += sm.scan[w];
+      sm.gbase[tid] = (uint32_t)(ex >> 32) + before;
+      sm.bstart[tid] = (uint32_t)ex;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      if (r < items && wfirst + 32 * r < cnt) {
+        const uint32_t d = (k[r] >> shift) & 255u;
+        const uint32_t lp = sm.bstart[d] + wc[d] + rk[r];
+        sm.keys[lp] = k[r];
+        sm.vals[lp] = v[r];
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < cnt; i += kSortThreads) {
+      const uint32_t key = sm.keys[i], d = (key >> shift) & 255u;
+      const uint32_t gp = sm.gbase[d] + ((uint32_t)i - sm.bstart[d]);
+      if (p < 3) kout[gp] = key;
+      vout[gp] = sm.vals[i];
+    }
+    // The pass's output is in place, and no block of the cluster still reads
+    // this one's counts.
+    cluster_barrier();
+  }
+}
+
+template <int ITEMS>
+void sort_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int nb, cudaStream_t st) {
+  cfg = cudaLaunchConfig_t{};
+  cfg.gridDim = dim3((unsigned)nb);
+  cfg.blockDim = dim3(kSortThreads);
+  cfg.dynamicSmemBytes = sizeof(SortSmem<ITEMS>);
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)nb;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+}
+
+template <int ITEMS>
+cudaError_t sort_attributes() {
+  auto k = cluster_sort_kernel<ITEMS>;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem<ITEMS>));
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+// Blocks a cluster of the sort can have on the current device: kSortBlocks if
+// the device can hold such a cluster, else the portable eight.
+int sort_blocks() {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
+  int nb = known[dev].load(std::memory_order_relaxed);
+  if (nb) return nb;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  sort_config<kSortMaxItems>(cfg, attr, kSortBlocks, nullptr);
+  int n = 0;
+  const bool fits = sort_attributes<kSortMaxItems>() == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&n, cluster_sort_kernel<kSortMaxItems>, &cfg) == cudaSuccess && n > 0;
+  if (!fits) cudaGetLastError();
+  nb = fits ? kSortBlocks : 8;
+  known[dev].store(nb, std::memory_order_relaxed);
+  return nb;
+}
+
+template <int ITEMS>
+cudaError_t launch_cluster_sort(const SortArgs& a, int nb, int items, cudaStream_t st) {
+  const cudaError_t e = sort_attributes<ITEMS>();
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  sort_config<ITEMS>(cfg, attr, nb, st);
+  return cudaLaunchKernelEx(&cfg, cluster_sort_kernel<ITEMS>, a, items);
 }
 
 // ---------------------------------------------------------------------------
@@ -567,18 +774,32 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   const int bblocks = b.bblocks;
   uint64_t* status_count = reinterpret_cast<uint64_t*>(b.status + (size_t)pblocks * 256 * 4);
   uint64_t* status_table = status_count + bblocks;
-  // 1. depth sort (values: Gaussian ids)
-  if ((e = launch_pdl(depth_hist_kernel, pblocks, kThreads, 0, st, (const uint32_t*)b.dkey[0], P, b.hist)) != cudaSuccess)
-    return e;
-  int cur = 0;
-  for (int p = 0; p < 4; ++p) {
-    e = launch_pdl(p == 0 ? onesweep_kernel<true, kPItems> : onesweep_kernel<false, kPItems>, pblocks, kThreads, ppass_smem,
-                   st, (const uint32_t*)b.dkey[cur], p == 0 ? (const uint32_t*)nullptr : (const uint32_t*)b.dval[cur],
-                   b.dkey[cur ^ 1], b.dval[cur ^ 1], (const uint32_t*)nullptr, (int64_t)P, 8 * p,
-                   (const uint32_t*)(b.hist + 256 * p), status_depth + (size_t)p * pblocks * 256,
-                   hdr->ticket + kTicketDepth0 + p, &hdr->err);
+  // 1. depth sort (values: Gaussian ids; an even number of passes, so the
+  // result is in dval[0] either way)
+  const int max_nb = P <= kSortBlocks * kSortThreads * kSortMaxItems ? sort_blocks() : 0;
+  if (P <= max_nb * kSortThreads * kSortMaxItems) {
+    SortArgs so;
+    so.key0 = b.dkey[0];
+    so.key1 = b.dkey[1];
+    so.val0 = b.dval[0];
+    so.val1 = b.dval[1];
+    so.n = P;
+    int nb = 1;  // blocks: one key a thread first, then more keys a thread
+    while (nb < max_nb && nb * kSortThreads < P) nb *= 2;
+    const int items = ceil_div(P, nb * kSortThreads);
+    e = items <= 1 ? launch_cluster_sort<1>(so, nb, items, st) : launch_cluster_sort<kSortMaxItems>(so, nb, items, st);
     if (e != cudaSuccess) return e;
-    cur ^= 1;
+  } else {
+    if ((e = launch_pdl(depth_hist_kernel, pblocks, kThreads, 0, st, (const uint32_t*)b.dkey[0], P, b.hist)) != cudaSuccess)
+      return e;
+    for (int p = 0; p < 4; ++p) {
+      const int i = p & 1, o = i ^ 1;
+      e = launch_pdl(p == 0 ? onesweep_kernel<true, kPItems> : onesweep_kernel<false, kPItems>, pblocks, kThreads,
+                     ppass_smem, st, (const uint32_t*)b.dkey[i], p == 0 ? (const uint32_t*)nullptr : (const uint32_t*)b.dval[i],
+                     b.dkey[o], b.dval[o], (const uint32_t*)nullptr, (int64_t)P, 8 * p, (const uint32_t*)(b.hist + 256 * p),
+                     status_depth + (size_t)p * pblocks * 256, hdr->ticket + kTicketDepth0 + p, &hdr->err);
+      if (e != cudaSuccess) return e;
+    }
   }
   // 2. tiles_touched scan + per-block tile counts
   CountArgs ca;
@@ -588,7 +809,7 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   ca.nblocks = bblocks;
   ca.chunk = b.bchunk;
   ca.cap = b.cap;
-  ca.order = b.dval[cur];
+  ca.order = b.dval[0];
   ca.touched = b.touched;
   ca.rect = b.rect;
   ca.offs = b.offs;
@@ -613,7 +834,7 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   sa.nblocks = bblocks;
   sa.chunk = b.bchunk;
   sa.cap = b.cap;
-  sa.order = b.dval[cur];
+  sa.order = b.dval[0];
   sa.touched = b.touched;
   sa.offs = b.offs;
   sa.table = b.table;
