@@ -155,10 +155,12 @@ BwdPack bwd_pack(const FstGeom& g) {
   p.off[kFLayers] = p.bytes;
   return p;
 }
+// The time planes' gradient lines: three axes per level, kFC floats a position.
+size_t line_bytes(const FstGeom& g) { return (size_t)3 * g.rs * ((1u << g.levels) - 1u) * kFC * 4; }
 // acc: with the reverse pass, the exact plane-gradient accumulators, two
 // uint64 arrays (hi, lo) of one entry per plane float (see fixed_add).
 struct WsLayout {
-  size_t wt, wn, f, act, dv, df, part, wp, acc, total;
+  size_t wt, wn, f, act, dv, df, part, wp, lines, acc, total;
 };
 WsLayout ws_layout(const FstGeom& g, int with_backward) {
   WsLayout w{};
@@ -170,7 +172,8 @@ WsLayout ws_layout(const FstGeom& g, int with_backward) {
   w.df = w.dv + (with_backward ? al256((size_t)kFW * g.P * 4) : 0);
   w.part = w.df + (with_backward ? al256((size_t)g.levels * kFC * g.P * 4) : 0);
   w.wp = w.part + (with_backward ? al256((size_t)bwd_blocks(g.P) * g.mlp_aligned * 4) : 0);
-  w.acc = w.wp + (with_backward ? al256((size_t)bwd_pack(g).bytes) : 0);
+  w.lines = w.wp + (with_backward ? al256((size_t)bwd_pack(g).bytes) : 0);
+  w.acc = w.lines + (with_backward ? al256(line_bytes(g)) : 0);
   w.total = w.acc + (with_backward == 2 ? al256((size_t)plane_floats(g) * 16) : 0);
   return w;
 }
@@ -1458,9 +1461,18 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
 // HexPlane reverse: per Gaussian and level, d f (Gaussian-major rows) through
 // the channel-wise product and the bilinear weights -- plane gradients by
 // 16-byte vector atomics (a corner is one 128-byte line), the canonical mean's
-// gradient summed over the lanes by a fixed shuffle tree (reproducible).  200k
-// Gaussians, 4 levels: 432 us (2.46 GB of atomic adds at 5.7 TB/s), 633 us
-// with lanes over channels, 4-byte atomics and five shuffles per sum.
+// gradient (the product's derivatives, carried from plane to plane) summed
+// over the lanes by a fixed shuffle tree (reproducible).  Every Gaussian has
+// the same time, so a time plane's gradient is a line over the spatial axis
+// times the two time weights: the lines are added here (two corners instead
+// of four) and spread over the planes by fst_lines_out_kernel.  The exact sums
+// keep the four corners.  Bound by the gathers (250 us of it without the
+// atomics) and the 18 atomic lines per level: 200k Gaussians, 4 levels: 357 us,
+// 432 with four corners for every plane, 633 with lanes over channels, 4-byte
+// atomics and five shuffles per sum.  At three blocks per SM (80 registers)
+// it spills: 410 us; a block row per level, which the forward takes, meets
+// the coarse levels' atomics all at once: 396 to 411; four copies of the
+// lines: 348 of the 357.
 constexpr int kHexThreads = 256;
 struct HexArgs {
   FstGeom g;
@@ -1468,9 +1480,34 @@ struct HexArgs {
   float t;
   float* d_means;
   float* d_planes;                      // float-atomic plane sums (acc_hi == NULL)
+  float4* lines;                        // and those of the time planes' lines
   unsigned long long *acc_hi, *acc_lo;  // or exact plane-gradient sums (fixed_add)
   uint32_t* err;
 };
+
+// Line of axis a of level lv (in 16-byte units; a position is kGLanes of them).
+__host__ __device__ __forceinline__ size_t line_off(const FstGeom& g, int lv, int a) {
+  return ((size_t)3 * g.rs * ((1u << lv) - 1u) + (size_t)a * (g.rs << lv)) * kGLanes;
+}
+
+// The time planes' gradients from the lines: the two time rows around t.
+__global__ void __launch_bounds__(256) fst_lines_out_kernel(const FstGeom g, const float4* __restrict__ lines, float t,
+                                                            float* __restrict__ d_planes, int64_t n) {
+  const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (e >= n) return;
+  int lv = 0;
+  while (lv + 1 < g.levels && e >= (int64_t)line_off(g, lv + 1, 0)) ++lv;
+  const int64_t r = e - (int64_t)line_off(g, lv, 0);
+  const int64_t per = (int64_t)(g.rs << lv) * kGLanes;
+  const int a = (int)(r / per), i = (int)(r % per) / kGLanes, q = (int)(r % kGLanes);
+  const Node nt = node_of(2.0f * t - 1.0f, g.rt);
+  const float4 v = lines[e];
+  // Plane 3 + a is (axis a, time).
+  float* o = d_planes + g.poff[lv * 6 + 3 + a] + ((int64_t)i * g.rt + nt.i) * kFC + 4 * q;
+  const float w0 = 1.0f - nt.f, w1 = nt.f;
+  o[0] = w0 * v.x; o[1] = w0 * v.y; o[2] = w0 * v.z; o[3] = w0 * v.w;
+  o[kFC] = w1 * v.x; o[kFC + 1] = w1 * v.y; o[kFC + 2] = w1 * v.z; o[kFC + 3] = w1 * v.w;
+}
 
 // d_planes[i] = the exact sum hi 2^32 + lo, times 2^-72, rounded to float.
 __global__ void __launch_bounds__(256) fst_planes_out_kernel(const unsigned long long* __restrict__ hi,
@@ -1506,27 +1543,43 @@ __global__ void __launch_bounds__(kHexThreads, 2) fst_hex_bwd_kernel(const HexAr
       const float df[4] = {df4.x, df4.y, df4.z, df4.w};
       Node n[4];
       level_nodes(g, c, lv, n);
-      // Samples of the six planes and their derivatives along both axes.
-      size_t off[6];
-      uint32_t row[6];
-      float smp[6][4], da[6][4], db[6][4];
+      // Samples of the six planes; their product's derivatives along x, y, z
+      // (product rule, plane by plane).
+      uint32_t loc[6];  // the first corner within its plane (16-byte units)
+      float smp[6][4], pr[4], dp[3][4];
 #pragma unroll
       for (int k = 0; k < 6; ++k) {
-        off[k] = corner_off(g, lv, k, n, q, row[k]);
-        const float4* base = planes + off[k];
-        const float4 v00 = __ldg(base), v01 = __ldg(base + kGLanes), v10 = __ldg(base + row[k]),
-                     v11 = __ldg(base + row[k] + kGLanes);
+        const int ia = pair_a(k), ib = pair_b(k);
+        const uint32_t row = (uint32_t)g.prb[lv * 6 + k] * kGLanes;
+        loc[k] = (uint32_t)n[ia].i * row + (uint32_t)n[ib].i * kGLanes + q;
+        const float4* base = planes + g.poff[lv * 6 + k] / 4 + loc[k];
+        const float4 v00 = __ldg(base), v01 = __ldg(base + kGLanes), v10 = __ldg(base + row),
+                     v11 = __ldg(base + row + kGLanes);
         const float p00[4] = {v00.x, v00.y, v00.z, v00.w}, p01[4] = {v01.x, v01.y, v01.z, v01.w};
         const float p10[4] = {v10.x, v10.y, v10.z, v10.w}, p11[4] = {v11.x, v11.y, v11.z, v11.w};
-        const float fa = n[pair_a(k)].f, fb = n[pair_b(k)].f;
+        const float fa = n[ia].f, fb = n[ib].f;
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
-          smp[k][ch] = (1.0f - fa) * ((1.0f - fb) * p00[ch] + fb * p01[ch]) + fa * ((1.0f - fb) * p10[ch] + fb * p11[ch]);
-          da[k][ch] = (1.0f - fb) * (p10[ch] - p00[ch]) + fb * (p11[ch] - p01[ch]);
-          db[k][ch] = (1.0f - fa) * (p01[ch] - p00[ch]) + fa * (p11[ch] - p10[ch]);
+          const float sv = (1.0f - fa) * ((1.0f - fb) * p00[ch] + fb * p01[ch]) + fa * ((1.0f - fb) * p10[ch] + fb * p11[ch]);
+          const float da = (1.0f - fb) * (p10[ch] - p00[ch]) + fb * (p11[ch] - p01[ch]);
+          const float db = (1.0f - fa) * (p01[ch] - p00[ch]) + fa * (p11[ch] - p10[ch]);
+          smp[k][ch] = sv;
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            const bool on_a = i == ia, on_b = i == ib;  // (axis 3 is time)
+            if (k == 0) {
+              dp[i][ch] = on_a ? da : on_b ? db : 0.0f;
+            } else {
+              const float t = dp[i][ch] * sv;
+              dp[i][ch] = on_a ? fmaf(pr[ch], da, t) : on_b ? fmaf(pr[ch], db, t) : t;
+            }
+          }
+          pr[ch] = k == 0 ? sv : pr[ch] * sv;
         }
       }
-      float dg[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // d L / d(grid position) per axis, over this lane's channels
+      float dg[3];  // d L / d(grid position) per axis, over this lane's channels
+#pragma unroll
+      for (int i = 0; i < 3; ++i) dg[i] = df[0] * dp[i][0] + df[1] * dp[i][1] + df[2] * dp[i][2] + df[3] * dp[i][3];
       float ds[6][4];
 #pragma unroll
       for (int ch = 0; ch < 4; ++ch) {
@@ -1538,8 +1591,6 @@ __global__ void __launch_bounds__(kHexThreads, 2) fst_hex_bwd_kernel(const HexAr
 #pragma unroll
         for (int k = 5; k >= 0; --k) {
           ds[k][ch] = pre[k] * suf;
-          dg[pair_a(k)] = fmaf(ds[k][ch], da[k][ch], dg[pair_a(k)]);
-          dg[pair_b(k)] = fmaf(ds[k][ch], db[k][ch], dg[pair_b(k)]);
           suf *= smp[k][ch];
         }
       }
@@ -1549,8 +1600,17 @@ __global__ void __launch_bounds__(kHexThreads, 2) fst_hex_bwd_kernel(const HexAr
 #pragma unroll
       for (int k = 0; k < 6; ++k) {
         const float fa = n[pair_a(k)].f, fb = n[pair_b(k)].f;
+        if (kAdd != PlaneAdd::kExact && pair_b(k) == 3) {
+          float4* line = a.lines + line_off(g, lv, pair_a(k)) + (size_t)n[pair_a(k)].i * kGLanes + q;
+          const float w0 = 1.0f - fa;
+          red_add4(line, w0 * ds[k][0], w0 * ds[k][1], w0 * ds[k][2], w0 * ds[k][3]);
+          red_add4(line + kGLanes, fa * ds[k][0], fa * ds[k][1], fa * ds[k][2], fa * ds[k][3]);
+          continue;
+        }
         const float w[4] = {(1.0f - fa) * (1.0f - fb), (1.0f - fa) * fb, fa * (1.0f - fb), fa * fb};
-        const size_t at[4] = {off[k], off[k] + kGLanes, off[k] + row[k], off[k] + row[k] + kGLanes};
+        const uint32_t row = (uint32_t)g.prb[lv * 6 + k] * kGLanes;
+        const size_t at0 = (size_t)(g.poff[lv * 6 + k] / 4) + loc[k];
+        const size_t at[4] = {at0, at0 + kGLanes, at0 + row, at0 + row + kGLanes};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float x[4] = {w[e] * ds[k][0], w[e] * ds[k][1], w[e] * ds[k][2], w[e] * ds[k][3]};
@@ -1924,6 +1984,7 @@ extern "C" fe_status fe_fst_backward(const fe_fst* fst, int P, const float* mean
     h.t = t;
     h.d_means = d_means;
     h.d_planes = d_planes;
+    h.lines = reinterpret_cast<float4*>(ws + w.lines);
     h.acc_hi = acc_hi;
     h.acc_lo = acc_lo;
     h.err = reinterpret_cast<uint32_t*>(ws);
@@ -1932,10 +1993,13 @@ extern "C" fe_status fe_fst_backward(const fe_fst* fst, int P, const float* mean
       fst_hex_bwd_kernel<PlaneAdd::kExact><<<hb, kHexThreads, 0, st>>>(h);
       const int64_t nb = (npl + 255) / 256;
       fst_planes_out_kernel<<<(int)(nb < 152 * 16 ? nb : 152 * 16), 256, 0, st>>>(acc_hi, acc_lo, npl, d_planes);
-    } else if (al16p(d_planes)) {
-      fst_hex_bwd_kernel<PlaneAdd::kVector><<<hb, kHexThreads, 0, st>>>(h);
     } else {
-      fst_hex_bwd_kernel<PlaneAdd::kScalar><<<hb, kHexThreads, 0, st>>>(h);
+      const size_t lb = line_bytes(g);
+      if (cudaMemsetAsync(h.lines, 0, lb, st) != cudaSuccess) return FE_ERR_CUDA;
+      if (al16p(d_planes)) fst_hex_bwd_kernel<PlaneAdd::kVector><<<hb, kHexThreads, 0, st>>>(h);
+      else fst_hex_bwd_kernel<PlaneAdd::kScalar><<<hb, kHexThreads, 0, st>>>(h);
+      const int64_t nl = (int64_t)(lb / 16);
+      fst_lines_out_kernel<<<(int)((nl + 255) / 256), 256, 0, st>>>(g, h.lines, t, d_planes, nl);
     }
   }
   fst_reduce_kernel<<<(int)((g.mlp_packed + 255) / 256), 256, 0, st>>>(g, a.part, nblk, d_mlp);
