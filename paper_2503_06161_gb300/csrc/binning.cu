@@ -473,7 +473,7 @@ __device__ __forceinline__ uint32_t rect_tile(const ushort4 rc, float iw, uint32
 }
 
 // Step 2: block b (ticket) owns depth ranks [chunk b, chunk b + chunk), chunk
-// <= 512; thread t scans ranks 2t and 2t + 1.  Writes offs / offs_by_gid and
+// <= 256 ITEMS; thread t scans ranks ITEMS t, ...  Writes offs / offs_by_gid and
 // column b of the tile-major count table.
 struct CountArgs {
   int P, tiles_x, ntiles, nblocks, chunk;
@@ -487,6 +487,7 @@ struct CountArgs {
   Header* hdr;
 };
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) {
   grid_dep_wait();
   grid_dep_launch();
@@ -494,8 +495,8 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
   __shared__ uint32_t s_scan[8];
   __shared__ uint32_t s_ticket;
   __shared__ uint64_t s_prefix;
-  __shared__ uint32_t s_c[kBinChunk];
-  __shared__ ushort4 s_rect[kBinChunk];
+  __shared__ uint32_t s_c[kThreads * ITEMS];
+  __shared__ ushort4 s_rect[kThreads * ITEMS];
   const int tid = threadIdx.x;
   for (int i = tid; i < a.ntiles; i += kThreads) s_cnt[i] = 0;
   if (tid == 0) s_ticket = atomicAdd(a.ticket, 1u);
@@ -504,11 +505,11 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
   const int64_t start = (int64_t)b * a.chunk;
   if (start >= a.P) return;
   const int nloc = (int)min((int64_t)a.chunk, (int64_t)a.P - start);
-  uint32_t gid[2], cnt[2];
+  uint32_t gid[ITEMS], cnt[ITEMS];
   uint32_t tsum = 0;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int li = tid * 2 + i;
+  for (int i = 0; i < ITEMS; ++i) {
+    const int li = tid * ITEMS + i;
     gid[i] = li < nloc ? a.order[start + li] : 0u;
     cnt[i] = li < nloc ? a.touched[gid[i]] : 0u;
     s_c[li] = cnt[i];
@@ -536,8 +537,8 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
   __syncthreads();
   uint64_t run = s_prefix + texcl;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int li = tid * 2 + i;
+  for (int i = 0; i < ITEMS; ++i) {
+    const int li = tid * ITEMS + i;
     if (li < nloc) {
       const uint32_t o32 = (uint32_t)min(run, (uint64_t)0xFFFFFFFFu);
       a.offs[start + li] = o32;
@@ -610,18 +611,21 @@ __global__ void __launch_bounds__(kThreads) table_scan_kernel(uint32_t* table, i
 
 // Step 4: block b (= blockIdx.x) takes the ranks of count block b, 128
 // Gaussians (a round) at a time.  Per tile it keeps a 128-bit mask of the
-// round's Gaussians that touch it (atomic ors: no order among them); then,
-// per tile, how many entries the round's later 32-Gaussian groups still add
-// (four bytes) beside the segment's position after the round, so an entry's
-// place is
-//   position after the round - entries from its group on + earlier bits of its group.
-// Entries are spread over all threads of the block, several to a Gaussian.
-// Bound by the scattered 8-byte stores and by instruction issue (two visits
-// of every entry at about ten and twenty instructions, and a sweep of the
-// tiles per round).  A warp that walked its 64 Gaussians one after another
-// with per-warp tile counters took 27 us at 1,000 Gaussians (the latency of
-// that chain; now 3), 28 at 30k (now 7), 44 at 200k (2.5 M entries; now 37)
-// and 591 at 1M (33 M; now 457).
+// round's Gaussians that touch it (atomic ors: no order among them), and the
+// position in the list where the round's entries of the tile begin; an
+// entry's place is that position plus the mask bits of earlier Gaussians.
+// Gaussian i of the round is bit i / 4 of word i % 4: a warp's Gaussians lie
+// in different words and a Gaussian's threads on consecutive tiles, so the
+// ors of a warp spread over all banks, and the second visit reads a mask with
+// one 16-byte load.  Entries are spread over all threads of the block, several
+// to a Gaussian; the next round's Gaussians (three dependent loads) are
+// fetched while a round is worked on.
+// Bound by the scattered 8-byte stores (a third to half of it: one sector
+// each) and by issue (two visits of every entry and a sweep of the tiles per
+// round).  1M Gaussians at 1280 x 1024, 33 M entries: 522 us from its early
+// launch, 543 with suffix counts beside the masks and blocks of 512; 100k at
+// 640 x 512, 1.6 M entries, the stage alone: 24 us instead of 32; 1,000
+// Gaussians: 3 us, 27 with a warp walking its 64 Gaussians one after another.
 // Block 0 also writes the tile ranges and marks the workspace as holding a
 // forward's state.
 struct ScatterArgs {
@@ -637,7 +641,7 @@ struct ScatterArgs {
 // blocks fit on an SM, so they get more threads.
 constexpr int kScatTiles = 2048;
 constexpr int kRound = 128;  // Gaussians per round (four 32-bit mask words)
-__host__ __device__ constexpr size_t scatter_smem(int ntiles) { return (size_t)ntiles * (16 + 4 + 4); }
+__host__ __device__ constexpr size_t scatter_smem(int ntiles) { return (size_t)ntiles * (16 + 4); }
 
 template <int NT>
 __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
@@ -646,11 +650,9 @@ __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
   uint4* s_mask = reinterpret_cast<uint4*>(s_dyn);  // [ntiles]
   uint32_t* s_word = s_dyn;                         // the same, [ntiles][4]
-  uint32_t* s_suf = s_dyn + 4 * a.ntiles;           // [ntiles]: four suffix counts
-  uint32_t* s_pos = s_suf + a.ntiles;               // [ntiles]: next position of the tile's segment
-  __shared__ uint32_t s_gid[kBinChunk], s_cnt[kBinChunk], s_off[kBinChunk];
-  __shared__ float s_iw[kBinChunk];  // 1 / (rect width in tiles)
-  __shared__ ushort4 s_rect[kBinChunk];
+  uint32_t* s_pos = s_dyn + 4 * a.ntiles;           // [ntiles]: next position of the tile's segment
+  __shared__ uint2 s_id[2][kRound];  // id, first emission index
+  __shared__ ushort4 s_rect[2][kRound];
   const int tid = threadIdx.x;
   const int b = blockIdx.x;
   const int64_t start = (int64_t)b * a.chunk;
@@ -660,21 +662,15 @@ __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
   // published empty so no later kernel follows an index beyond capacity.
   const bool overflow = (uint64_t)a.hdr->num_dups > cap;
   const uint64_t K = overflow ? 0 : (uint64_t)a.hdr->num_dups;
-  // The block's Gaussians, all rounds at once (three dependent loads).
-  const int npad = (nloc + kRound - 1) / kRound * kRound;
-  for (int j = tid; j < npad; j += NT) {
-    uint32_t g = 0, c = 0;
-    ushort4 rc = make_ushort4(0, 0, 0, 0);
-    if (j < nloc) {
-      g = a.order[start + j];
-      s_off[j] = a.offs[start + j];
-      c = a.touched[g];
-      if (c) rc = a.rect[g];
-    }
-    s_gid[j] = g;
-    s_cnt[j] = c;
-    s_rect[j] = rc;
-    s_iw[j] = 1.0f / (float)(rc.z - rc.x + 1u);
+  // Rectangle of Gaussian g (width 0 where it touches no tile).
+  const auto rect_of = [&](bool have, uint32_t g) {
+    return have && a.touched[g] != 0u ? a.rect[g] : make_ushort4(1, 0, 0, 0);
+  };
+  if (tid < kRound) {
+    const bool have = tid < nloc;
+    const uint32_t g = have ? a.order[start + tid] : 0u;
+    s_id[0][tid] = make_uint2(g, have ? a.offs[start + tid] : 0u);
+    s_rect[0][tid] = rect_of(have, g);
   }
   for (int t = tid; t < a.ntiles; t += NT) {
     s_pos[t] = a.table[(size_t)t * a.nblocks + b];
@@ -688,35 +684,45 @@ __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
   if (b == 0 && tid == 0) a.hdr->has_forward = 1u;
   constexpr int TPG = NT / kRound;  // threads per Gaussian
   const int i = tid / TPG, sub = tid % TPG;
+  const int word = i & 3, bit = i >> 2;
+  // Bits of the Gaussians before i in the four words.
+  const uint32_t below = (1u << bit) - 1u, upto = (2u << bit) - 1u;
+  const uint32_t m0 = word > 0 ? upto : below, m1 = word > 1 ? upto : below, m2 = word > 2 ? upto : below;
   __syncthreads();
-  for (int r0 = 0; r0 < nloc; r0 += kRound) {
-    const uint32_t c = s_cnt[r0 + i];
-    const ushort4 rc = s_rect[r0 + i];
-    const float iw = s_iw[r0 + i];
-    for (uint32_t k = sub; k < c; k += TPG) atomicOr(&s_word[4 * rect_tile(rc, iw, k, a.tiles_x) + (i >> 5)], 1u << (i & 31));
+  int buf = 0;
+  for (int r0 = 0; r0 < nloc; r0 += kRound, buf ^= 1) {
+    // The next round's Gaussian of this thread: ids now, rectangles below.
+    const int rn = r0 + kRound + tid;
+    const bool have = tid < kRound && rn < nloc;
+    uint2 nid = make_uint2(0u, 0u);
+    if (have) nid = make_uint2(a.order[start + rn], a.offs[start + rn]);
+    const ushort4 rc = s_rect[buf][i];
+    const uint32_t width = (uint32_t)(rc.z + 1) - rc.x, c = width * ((uint32_t)(rc.w + 1) - rc.y);
+    const float iw = 1.0f / (float)width;
+    for (uint32_t k = sub; k < c; k += TPG) atomicOr(&s_word[4 * rect_tile(rc, iw, k, a.tiles_x) + word], 1u << bit);
+    __syncthreads();
+    const ushort4 nrc = rect_of(have, nid.x);
+    if (sub < c) {
+      const uint2 id = s_id[buf][i];
+      for (uint32_t k = sub; k < c; k += TPG) {
+        const uint32_t tile = rect_tile(rc, iw, k, a.tiles_x);
+        const uint4 m = s_mask[tile];
+        const uint32_t pos = s_pos[tile] + __popc(m.x & m0) + __popc(m.y & m1) + __popc(m.z & m2) + __popc(m.w & below);
+        if ((uint64_t)pos < cap) a.sorted[pos] = make_uint2(id.y + k, id.x);
+      }
+    }
+    if (r0 + kRound >= nloc) break;
+    if (tid < kRound) {
+      s_id[buf ^ 1][tid] = nid;
+      s_rect[buf ^ 1][tid] = nrc;
+    }
     __syncthreads();
     for (int t = tid; t < a.ntiles; t += NT) {
       const uint4 m = s_mask[t];
-      const uint32_t n3 = __popc(m.w), n2 = n3 + __popc(m.z), n1 = n2 + __popc(m.y), n0 = n1 + __popc(m.x);
-      s_suf[t] = n0 | (n1 << 8) | (n2 << 16) | (n3 << 24);
-      s_pos[t] += n0;
+      s_pos[t] += __popc(m.x) + __popc(m.y) + __popc(m.z) + __popc(m.w);
+      s_mask[t] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
-    if (sub < c) {
-      const uint32_t g = s_gid[r0 + i], e0 = s_off[r0 + i], lt = (1u << (i & 31)) - 1u;
-      const int sh = 8 * (i >> 5);
-      for (uint32_t k = sub; k < c; k += TPG) {
-        const uint32_t tile = rect_tile(rc, iw, k, a.tiles_x);
-        const uint64_t pos = (uint64_t)(s_pos[tile] - ((s_suf[tile] >> sh) & 0xFFu) + __popc(s_word[4 * tile + (i >> 5)] & lt));
-        const uint64_t e = (uint64_t)e0 + k;
-        if (pos < cap) a.sorted[pos] = make_uint2((uint32_t)e, g);
-      }
-    }
-    __syncthreads();
-    if (r0 + kRound < nloc) {
-      for (int t = tid; t < a.ntiles; t += NT) s_mask[t] = make_uint4(0u, 0u, 0u, 0u);
-      __syncthreads();
-    }
   }
 }
 
@@ -819,8 +825,9 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
   ca.ticket = hdr->ticket + kTicketScan;
   ca.hdr = hdr;
   const size_t count_smem = (size_t)b.ntiles * 4;
-  cudaFuncSetAttribute(bin_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)count_smem);
-  if ((e = launch_pdl(bin_count_kernel, bblocks, kThreads, count_smem, st, ca)) != cudaSuccess) return e;
+  auto count = b.bchunk <= 2 * kThreads ? bin_count_kernel<2> : bin_count_kernel<kBinChunk / kThreads>;
+  cudaFuncSetAttribute(count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)count_smem);
+  if ((e = launch_pdl(count, bblocks, kThreads, count_smem, st, ca)) != cudaSuccess) return e;
   // 3. scan of the (tile, block) table
   const int64_t tn = (int64_t)b.ntiles * bblocks;
   e = launch_pdl(table_scan_kernel, ceil_div(tn, kPChunk), kThreads, 0, st, b.table, tn, status_table,

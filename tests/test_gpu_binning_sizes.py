@@ -19,7 +19,8 @@ from test_gpu_render import _tile_bin_gpu  # noqa: E402
     (1025, 97, 61, (16, 16)), (2049, 97, 61, (16, 16)), (16384, 203, 157, (16, 16)), (16385, 203, 157, (16, 16)),
     (32769, 203, 157, (16, 16)), (38912, 203, 157, (16, 16)), (49152, 203, 157, (16, 16)),
     (49153, 203, 157, (16, 16)), (77823, 203, 157, (16, 16)), (77825, 203, 157, (16, 16)),
-    (3000, 1100, 520, (16, 16)), (20001, 1100, 520, (16, 16)), (79000, 1100, 520, (16, 16))])
+    (3000, 1100, 520, (16, 16)), (20001, 1100, 520, (16, 16)), (79000, 1100, 520, (16, 16)),
+    (622591, 97, 61, (16, 16)), (622593, 203, 157, (16, 16))])
 def test_tile_lists_bit_exact(P, W, H, tile):
     rng = np.random.default_rng(P)
     uv = np.c_[rng.uniform(-20, W + 20, P), rng.uniform(-20, H + 20, P)].astype(np.float32)
