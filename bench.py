@@ -587,14 +587,15 @@ def run_ours(args, world, rank, local):
                "d2h_bytes_per_step": int(d2h), "ms_per_step": round(e2e_ms, 4),
                "pipeline": "two buffer sets; uploads and read-backs on two copy streams overlap the compute"}
 
-    # forward: deform+project, depth histogram, 4 depth passes, count, table
-    # scan, scatter, composite; L1 x2 (2 kernels each); reverse: composite,
-    # feature sums, projection chain (+ deformation chain).
-    # (With a decoder, its kernel and fixed-order sum replace the two
-    # feature-L1 kernels.)
-    # Training adds the depth L1 (2 kernels) and the Adam launch.
-    launches_per_step = (10 + 4 + 3 + (1 if deform is not None else 0) + (1 if opt is not None else 0)
-                         + (2 if tgt_depth is not None else 0))
+    # forward: projection, depth sort (histogram and 4 passes, one launch for
+    # few Gaussians), count, table scan, scatter, composite; L1 x2 (2 kernels
+    # each); reverse: composite (a pass per 64 channels), feature sums,
+    # projection chain; the deformation adds its sample and MLP and their
+    # reverses.  (With a decoder, its kernel and fixed-order sum replace the two
+    # feature-L1 kernels.)  Training adds the depth L1 (2 kernels) and the Adam
+    # launch.
+    launches_per_step = ((6 if P <= 49152 else 10) + 4 + 2 + max(1, D // 64) + (4 if deform is not None else 0)
+                         + (1 if opt is not None else 0) + (2 if tgt_depth is not None else 0))
     result = {
         "metric": METRIC, "value": round(world * 1000.0 / ms, 3), "unit": "it/s", "n_gpus": world,
         "steps": K_steps, "warmup": args.warmup, "ms_per_step": round(ms, 4), "higher_is_better": True,
@@ -960,10 +961,11 @@ def run_train_fst(args, world, rank, local, cfg):
         "e2e": {"value": round(world * 1000.0 / e2e_ms, 3), "unit": "it/s", "h2d_bytes_per_step": int(h2d),
                 "d2h_bytes_per_step": 16, "ms_per_step": round(e2e_ms, 4)},
         "device_errors": int(tr.rast.stats()["device_errors"]), "clocks": clk,
-        # per step: FST forward 2 (pack, forward); render forward 10; L1 rgb 2,
-        # decoder 2, depth L1 2; render reverse 3; FST reverse 2 (reverse,
-        # reduce); TV 2; Adam 2 (Gaussians + decoder, planes + MLP)
-        "gpu_launches": 27 * K,
+        # per step: FST forward 3 (pack, sample, MLP); render forward 10; L1 rgb
+        # 2, decoder 2, depth L1 2; render reverse 3; FST reverse 5 (pack, MLP,
+        # HexPlane, lines, reduce); TV 2; Adam 2 (Gaussians + decoder, planes +
+        # MLP)
+        "gpu_launches": 31 * K,
     }
     if rank == 0:
         print(json.dumps(result))
