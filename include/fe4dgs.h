@@ -372,7 +372,7 @@ int64_t fe_fst_mlp_floats(int levels, int D);
  * planes of levels x (rs, rt) nodes.  with_backward = 0: forward only
  * (inference; the HexPlane features, 0.5 KB per Gaussian at 4 levels); 1:
  * the forward also keeps the per-Gaussian activations the reverse pass
- * reads, and the reverse's own per-Gaussian buffers (about 5.1 KB per
+ * reads, and the reverse's own per-Gaussian buffers (about 4.6 KB per
  * Gaussian at 4 levels in all) and per-block partial sums of the weight
  * gradients; 2: as 1, plus the exact plane-gradient accumulators that
  * fe_fst.exact_planes = 1 needs (16 bytes per plane float).  The first 4

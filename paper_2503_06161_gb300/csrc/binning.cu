@@ -1,6 +1,7 @@
 // Integer stage of the pass: the tile-based binning of 3DGS that the paper
 // builds on (Sec. 2.1), reorganised for one GPU:
-//   1. stable LSD radix sort of the P depth keys (4 x 8-bit passes);
+//   1. stable LSD radix sort of the P depth keys (4 x 8-bit passes, in one
+//      launch for few keys);
 //   2. exclusive scan of tiles_touched in depth order (decoupled look-back)
 //      and, per block of depth-ordered Gaussians, its count of entries per
 //      tile (a tile-major (tile, block) table);

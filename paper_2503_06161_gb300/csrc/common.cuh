@@ -104,7 +104,7 @@ enum : int {
   kNumTickets = 8,
 };
 
-// Largest tile count of the counting scatter (its per-warp counters live in
+// Largest tile count of the counting scatter (its masks of the tiles live in
 // shared memory).
 constexpr int kMaxTiles = 8192;
 

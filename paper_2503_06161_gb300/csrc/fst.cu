@@ -13,9 +13,9 @@
 //                       Gaussian-major;
 //   fst_fwd_tc_kernel   the MLP of a forward without reverse state, on the
 //                       tensor cores (three BF16 terms per operand);
-//   fst_fwd_kernel      the MLP in training: a block holds 128 Gaussians and every layer
-//                       is a block product -- activations in shared memory
-//                       (a row per Gaussian), each thread a register tile of
+//   fst_fwd_kernel      the MLP in training: a block holds 128 Gaussians and
+//                       every layer is a block product -- activations in
+//                       shared memory (a row per Gaussian), lanes over rows,
 //                       packed FP32 FMAs, weight tiles staged by cp.async --
 //                       writing the deformed Gaussians and relu(z) of every
 //                       hidden layer for the reverse;
@@ -25,7 +25,9 @@
 //                       the block's own partial; writes d f;
 //   fst_hex_bwd_kernel  the HexPlane reverse: plane gradients by vector
 //                       float atomics (the only order-dependent sum of this
-//                       file), the canonical mean's gradient;
+//                       file), the time planes' as lines over the spatial
+//                       axis (spread by fst_lines_out_kernel), and the
+//                       canonical mean's gradient;
 //   fst_reduce_kernel   the weight gradients: the blocks' partials summed in
 //                       block order (reproducible bit for bit);
 //   fst_tv_kernel       the TV term and its plane gradient.
@@ -1938,7 +1940,7 @@ extern "C" fe_status fe_fst_backward(const fe_fst* fst, int P, const float* mean
     return cudaMemsetAsync(d_mlp, 0, (size_t)g.mlp_packed * 4, st) == cudaSuccess ? FE_OK : FE_ERR_CUDA;
   }
   if (!fst->planes || !means || !d_means_t || !d_quats_t || !d_log_scales_t || !d_opacity_logits_t || !d_feat_t ||
-      !d_means || !al16p(d_feat_t))
+      !d_means || !al16p(d_feat_t) || !al16p(fst->planes))
     return FE_ERR_INVALID_ARG;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   unsigned long long* acc_hi = exact ? reinterpret_cast<unsigned long long*>(ws + w.acc) : nullptr;
