@@ -157,8 +157,11 @@ BwdPack bwd_pack(const FstGeom& g) {
   p.off[kFLayers] = p.bytes;
   return p;
 }
-// The time planes' gradient lines: three axes per level, kFC floats a position.
-size_t line_bytes(const FstGeom& g) { return (size_t)3 * g.rs * ((1u << g.levels) - 1u) * kFC * 4; }
+// The time planes' gradient lines: three axes per level, kFC floats a
+// position, in kLineCopies copies that blocks take in turn (a line's few
+// positions get terms from every Gaussian: shorter sums round less).
+constexpr int kLineCopies = 16;
+size_t line_bytes(const FstGeom& g) { return (size_t)kLineCopies * 3 * g.rs * ((1u << g.levels) - 1u) * kFC * 4; }
 // acc: with the reverse pass, the exact plane-gradient accumulators, two
 // uint64 arrays (hi, lo) of one entry per plane float (see fixed_add).
 struct WsLayout {
@@ -1469,12 +1472,12 @@ __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_co
 // times the two time weights: the lines are added here (two corners instead
 // of four) and spread over the planes by fst_lines_out_kernel.  The exact sums
 // keep the four corners.  Bound by the gathers (250 us of it without the
-// atomics) and the 18 atomic lines per level: 200k Gaussians, 4 levels: 357 us,
+// atomics) and the 18 atomic lines per level: 200k Gaussians, 4 levels: 349 us,
 // 432 with four corners for every plane, 633 with lanes over channels, 4-byte
 // atomics and five shuffles per sum.  At three blocks per SM (80 registers)
 // it spills: 410 us; a block row per level, which the forward takes, meets
-// the coarse levels' atomics all at once: 396 to 411; four copies of the
-// lines: 348 of the 357.
+// the coarse levels' atomics all at once: 396 to 411; with one copy of the
+// lines: 357.
 constexpr int kHexThreads = 256;
 struct HexArgs {
   FstGeom g;
@@ -1492,7 +1495,8 @@ __host__ __device__ __forceinline__ size_t line_off(const FstGeom& g, int lv, in
   return ((size_t)3 * g.rs * ((1u << lv) - 1u) + (size_t)a * (g.rs << lv)) * kGLanes;
 }
 
-// The time planes' gradients from the lines: the two time rows around t.
+// The time planes' gradients from the lines (n 16-byte units a copy): the two
+// time rows around t.
 __global__ void __launch_bounds__(256) fst_lines_out_kernel(const FstGeom g, const float4* __restrict__ lines, float t,
                                                             float* __restrict__ d_planes, int64_t n) {
   const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -1503,7 +1507,12 @@ __global__ void __launch_bounds__(256) fst_lines_out_kernel(const FstGeom g, con
   const int64_t per = (int64_t)(g.rs << lv) * kGLanes;
   const int a = (int)(r / per), i = (int)(r % per) / kGLanes, q = (int)(r % kGLanes);
   const Node nt = node_of(2.0f * t - 1.0f, g.rt);
-  const float4 v = lines[e];
+  float4 v = lines[e];
+#pragma unroll
+  for (int c = 1; c < kLineCopies; ++c) {
+    const float4 x = __ldg(lines + e + c * n);
+    v = make_float4(v.x + x.x, v.y + x.y, v.z + x.z, v.w + x.w);
+  }
   // Plane 3 + a is (axis a, time).
   float* o = d_planes + g.poff[lv * 6 + 3 + a] + ((int64_t)i * g.rt + nt.i) * kFC + 4 * q;
   const float w0 = 1.0f - nt.f, w1 = nt.f;
@@ -1603,7 +1612,8 @@ __global__ void __launch_bounds__(kHexThreads, 2) fst_hex_bwd_kernel(const HexAr
       for (int k = 0; k < 6; ++k) {
         const float fa = n[pair_a(k)].f, fb = n[pair_b(k)].f;
         if (kAdd != PlaneAdd::kExact && pair_b(k) == 3) {
-          float4* line = a.lines + line_off(g, lv, pair_a(k)) + (size_t)n[pair_a(k)].i * kGLanes + q;
+          float4* line = a.lines + (size_t)(blockIdx.x % kLineCopies) * line_off(g, g.levels, 0) +
+                         line_off(g, lv, pair_a(k)) + (size_t)n[pair_a(k)].i * kGLanes + q;
           const float w0 = 1.0f - fa;
           red_add4(line, w0 * ds[k][0], w0 * ds[k][1], w0 * ds[k][2], w0 * ds[k][3]);
           red_add4(line + kGLanes, fa * ds[k][0], fa * ds[k][1], fa * ds[k][2], fa * ds[k][3]);
@@ -2000,7 +2010,7 @@ extern "C" fe_status fe_fst_backward(const fe_fst* fst, int P, const float* mean
       if (cudaMemsetAsync(h.lines, 0, lb, st) != cudaSuccess) return FE_ERR_CUDA;
       if (al16p(d_planes)) fst_hex_bwd_kernel<PlaneAdd::kVector><<<hb, kHexThreads, 0, st>>>(h);
       else fst_hex_bwd_kernel<PlaneAdd::kScalar><<<hb, kHexThreads, 0, st>>>(h);
-      const int64_t nl = (int64_t)(lb / 16);
+      const int64_t nl = (int64_t)(lb / 16 / kLineCopies);
       fst_lines_out_kernel<<<(int)((nl + 255) / 256), 256, 0, st>>>(g, h.lines, t, d_planes, nl);
     }
   }
