@@ -228,9 +228,10 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* __re
 // keys a thread); the five launches above, four of them with a chain of
 // look-back, are too, at 20 us for 1,000 keys and 37 for 30k, where this one
 // takes 6 and 11.  With more keys a thread the sixteen SMs fall behind the
-// whole chip (100k: 38 us against 35), so the line lies at three a thread
-// (640 x 512 frames, this sort against the passes: 1,000 Gaussians 53 and
-// 57 us, 10k 104 and 111, 32k 177 and 179, 48k 196 and 198, 64k 209 and 208).
+// whole chip (a frame of 100k 8 us slower, of 200k 48), so the line lies at
+// three a thread (640 x 512 frames, this sort against the passes: 1,000
+// Gaussians 53 and 57 us, 10k 104 and 111, 32k 177 and 179, 48k 196 and 198,
+// 64k 209 and 208).
 // ---------------------------------------------------------------------------
 constexpr int kSortThreads = 1024, kSortWarps = kSortThreads / 32;
 constexpr int kSortBlocks = 16;  // more than the eight that every device takes: see sort_blocks
