@@ -65,7 +65,7 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* s_warp
 // ---------------------------------------------------------------------------
 // Global digit histograms of the depth keys (all four passes at once).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) depth_hist_kernel(const uint32_t* __restrict__ keys, int n, uint32_t* hist) {
+__global__ void __launch_bounds__(kThreads) depth_hist_kernel(const uint32_t* keys, int n, uint32_t* hist) {
   grid_dep_wait();
   grid_dep_launch();
   __shared__ uint32_t s[4][256];
@@ -102,12 +102,10 @@ struct PassSmem {
 };
 
 template <bool kIdentVals, int ITEMS>
-__global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* __restrict__ keys_in,
-                                                            const uint32_t* __restrict__ vals_in,
-                                                            uint32_t* __restrict__ keys_out,
-                                                            uint32_t* __restrict__ vals_out,
+__global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* keys_in, const uint32_t* vals_in,
+                                                            uint32_t* keys_out, uint32_t* vals_out,
                                                             const uint32_t* n_dev, int64_t n_cap, int shift,
-                                                            const uint32_t* __restrict__ hist, uint32_t* status,
+                                                            const uint32_t* hist, uint32_t* status,
                                                             uint32_t* ticket, uint32_t* err) {
   constexpr int CHUNK = kThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];

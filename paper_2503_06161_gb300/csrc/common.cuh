@@ -347,6 +347,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int li
 // a kernel runs at all, every kernel but its direct predecessor has
 // completed: memory that the predecessor does not write (weights, parameters)
 // may be read ahead of the wait.
+// A kernel can be running while its predecessor still writes, so what a pass
+// writes is read by plain loads alone: __ldg and const __restrict__ parameters
+// promise data that nobody writes while the kernel runs, which lets a load
+// move above the wait or hit a line cached before it.  __ldg is for what no
+// kernel of the pass writes (parameters, planes, weights, upstream gradients).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

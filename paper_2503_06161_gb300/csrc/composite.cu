@@ -145,7 +145,7 @@ __device__ __forceinline__ void fwd_tile(const CompositeArgs& a, const int tile,
   // Gaussian of this thread's slot in batch k (prefetched a batch ahead).
   auto slot_gid = [&](uint32_t k) -> uint32_t {
     const uint32_t p = k * B + (uint32_t)tid;
-    return (k < nbatch && tid < B && p < n) ? __ldg(&a.sorted[rg.x + p].y) : 0u;
+    return (k < nbatch && tid < B && p < n) ? a.sorted[rg.x + p].y : 0u;
   };
   auto batch_len = [&](uint32_t k) -> int { return (int)min((uint32_t)B, n - k * B); };
   uint32_t issued = 0;
@@ -547,7 +547,7 @@ __device__ __forceinline__ void bwd_tile(const CompositeArgs& a, const int tile,
     g = 0u;
     if (k < nbatch && tid < batch_len(k)) {
       const uint32_t p = rg.x + batch_lo(k) + (uint32_t)tid;
-      const uint2 eg = __ldg(a.sorted + p);
+      const uint2 eg = a.sorted[p];
       e = eg.x;
       g = eg.y;
     }
@@ -556,7 +556,7 @@ __device__ __forceinline__ void bwd_tile(const CompositeArgs& a, const int tile,
   // pixel of its block blended (read a batch ahead, so its global latency
   // overlaps the previous batch).
   auto mask_word = [&](uint32_t k) -> uint32_t {
-    return (k < nbatch && batch_lo(k) < wmax) ? __ldg(a.cmask + (cslot0 + batch_lo(k) / 32) * 8 + warp) : 0u;
+    return (k < nbatch && batch_lo(k) < wmax) ? a.cmask[(cslot0 + batch_lo(k) / 32) * 8 + warp] : 0u;
   };
   uint32_t mask_next = mask_word(0);
   uint32_t e_next, g_next;

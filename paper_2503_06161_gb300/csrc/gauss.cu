@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 4) partial_reduce_kernel(const Gauss
   const uint32_t wlast = E0 < E1 ? (E1 - 1) >> 5 : 0u;
   for (uint32_t w0 = E0 >> 5; E0 < E1 && w0 <= wlast; w0 += 32) {
     const uint32_t w = w0 + (uint32_t)lane;
-    uint32_t m = w <= wlast ? __ldg(b.pflags + w) : 0u;
+    uint32_t m = w <= wlast ? b.pflags[w] : 0u;
     if (w == E0 >> 5) m &= ~0u << (E0 & 31u);
     if (w == wlast && (E1 & 31u)) m &= (1u << (E1 & 31u)) - 1u;
     uint32_t pos = (uint32_t)__popc(m);
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(kThreads, 4) partial_reduce_kernel(const Gauss
         idx[u] = (w0 << 5) + rows[min(r + u, n - 1)];
         const float* row = b.partials + (size_t)idx[u] * NP;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) x[u][q] = (r + u < n && lane + 32 * q < NP) ? __ldg(row + lane + 32 * q) : 0.0f;
+        for (int q = 0; q < NQ; ++q) x[u][q] = (r + u < n && lane + 32 * q < NP) ? row[lane + 32 * q] : 0.0f;
       }
 #pragma unroll
       for (int u = 0; u < RG; ++u) {
@@ -731,21 +731,21 @@ __global__ void __launch_bounds__(kThreads, 2) gauss_bwd_proj_kernel(const Gauss
 // warp sums per Gaussian, 59 with two blocks.
 template <int C>
 __global__ void __launch_bounds__(kThreads, 4) gauss_bwd_deform_kernel(const GaussArgs a, const GaussBwdArgs b,
-                                                                     const float* __restrict__ df_all) {
+                                                                     const float* df_all) {
   grid_dep_wait();
   grid_dep_launch();
   constexpr int LG = gather_lanes<C>();
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   const int g = (int)(tid / LG), q = (int)(tid % LG);
   const float* dd = b.ddstate + (size_t)g * 12;
-  const bool active = g < a.P && __ldg(dd + 11) != 0.0f;
+  const bool active = g < a.P && dd[11] != 0.0f;
   if (!__any_sync(0xFFFFFFFFu, active)) return;  // whole warp idle
   float dc[3] = {0.f, 0.f, 0.f};
   if (active) {
     const float mu[3] = {__ldg(a.means + 3 * (size_t)g), __ldg(a.means + 3 * (size_t)g + 1),
                          __ldg(a.means + 3 * (size_t)g + 2)};
     const AxisPos ap = axis_pos(a, mu);
-    const float4 df4 = __ldg(reinterpret_cast<const float4*>(df_all) + (size_t)g * LG + q);
+    const float4 df4 = reinterpret_cast<const float4*>(df_all)[(size_t)g * LG + q];
     const float df[4] = {df4.x, df4.y, df4.z, df4.w};
     // The product of the six planes and its derivatives by x, y, z, one
     // plane after another.
@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(kThreads, 4) gauss_bwd_deform_kernel(const Gau
     const float part = (q == 0 ? dc[0] : q == 1 ? dc[1] : dc[2]) * (0.5f * (float)(a.R - 1)) *
                        (q == 0 ? a.bscale[0] : q == 1 ? a.bscale[1] : a.bscale[2]);
     float* o = b.d_means + 3 * (size_t)g + q;
-    *o += b.accumulate ? __ldg(dd + q) + part : part;
+    *o += b.accumulate ? dd[q] + part : part;
   }
 }
 
