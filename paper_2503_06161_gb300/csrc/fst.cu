@@ -1041,19 +1041,6 @@ struct BwdArgs {
 constexpr int kTTerm = kFM * 128;
 __device__ __forceinline__ uint32_t t_off(int r, int chunk) { return (uint32_t)(r * 128 + ((chunk ^ (r & 7)) << 4)); }
 
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&v)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-               : "r"(addr)
-               : "memory");
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t (&v)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-               : "r"(addr)
-               : "memory");
-}
-
 // Lane's pair of values (columns c, c + 1; c even) of row r into a tile.
 __device__ __forceinline__ void put_pair(unsigned char* tile, int r, int c, float x, float y) {
   uint32_t t3[3];
@@ -1103,7 +1090,7 @@ __device__ __forceinline__ void delta_w(uint32_t tile, int warp, int kc, const u
   for (int ks = 0; ks < KS; ++ks) {
     uint32_t a[3][4];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) ldsm_x4(tile + t * kTTerm + t_off(r, 2 * (kc + ks) + ch), a[t]);
+    for (int t = 0; t < 3; ++t) ldmatrix_x4(tile + t * kTTerm + t_off(r, 2 * (kc + ks) + ch), a[t]);
     tc_step<4>(a[0], a[1], a[2], w + ks * 4 * 768, lane, acc, zs);
   }
 #pragma unroll
@@ -1135,7 +1122,7 @@ __device__ __forceinline__ void weight_grad(uint32_t sd, int oc, uint32_t sx, in
   for (int g0 = 0; g0 < kFM; g0 += 16) {
     uint32_t a[3][4];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) ldsm_x4_t(sd + t * kTTerm + t_off(g0 + r + 8 * (mi >> 1), oc + (mi & 1)), a[t]);
+    for (int t = 0; t < 3; ++t) ldmatrix_x4_trans(sd + t * kTTerm + t_off(g0 + r + 8 * (mi >> 1), oc + (mi & 1)), a[t]);
     if (pb) {
       mma_bf16_16816(bs[0], a[2], one, one);
       mma_bf16_16816(bs[0], a[1], one, one);
@@ -1147,7 +1134,7 @@ __device__ __forceinline__ void weight_grad(uint32_t sd, int oc, uint32_t sx, in
     for (int t = 0; t < 3; ++t)
 #pragma unroll
       for (int q = 0; q < NP; ++q)
-        ldsm_x4_t(sx + t * kTTerm + t_off(g0 + r + 8 * (mi & 1), NT == 1 ? ic : ic + 2 * q + (mi >> 1)), b[t][q]);
+        ldmatrix_x4_trans(sx + t * kTTerm + t_off(g0 + r + 8 * (mi & 1), NT == 1 ? ic : ic + 2 * q + (mi >> 1)), b[t][q]);
 #define FST_WG(za, ta, tb)                                                                                     \
   _Pragma("unroll") for (int nt = 0; nt < NT; ++nt)                                                            \
       mma_bf16_16816(za[nt], a[ta], b[tb][nt >> 1][2 * (nt & 1)], b[tb][nt >> 1][2 * (nt & 1) + 1]);

@@ -50,3 +50,17 @@ def test_non_coherent_loads_read_inputs_only(name):
     text = _source(name)
     for m in re.finditer(r"__ldg\(", text):
         assert _argument(text, m.end()) in INPUTS, _argument(text, m.end())
+
+
+def test_inline_memory_accesses_are_ordered():
+    # An instruction with an address operand is tied to the stores before it
+    # only by the clobber (a prefetch moves no data).
+    accesses = 0
+    for name in sorted(os.listdir(CSRC)):
+        text = _source(name)
+        for m in re.finditer(r"\basm(?:\s+volatile)?\s*\(", text):
+            stmt = _argument(text, m.end())
+            if re.search(r"\[%", stmt) and not stmt.startswith('"prefetch'):
+                accesses += 1
+                assert '"memory"' in stmt, (name, stmt)
+    assert accesses > 20
