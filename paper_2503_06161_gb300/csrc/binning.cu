@@ -465,12 +465,70 @@ __device__ __forceinline__ uint64_t lookback64_resolve(uint64_t* status, uint32_
   return excl;
 }
 
-// Tile of item k (row-major) of a Gaussian's tile rectangle, iw = 1 / width
-// (exact for k < 2^20).
-__device__ __forceinline__ uint32_t rect_tile(const ushort4 rc, float iw, uint32_t k, int tiles_x) {
-  const uint32_t dy = (uint32_t)(((float)k + 0.5f) * iw), dx = k - dy * (rc.z - rc.x + 1u);
-  return (rc.y + dy) * (uint32_t)tiles_x + rc.x + dx;
+// Tiles of a rectangle (first and last tile of each axis; none: last < first).
+__device__ __forceinline__ uint32_t rect_tiles(const ushort4 rc) {
+  return ((uint32_t)(rc.z + 1) - rc.x) * ((uint32_t)(rc.w + 1) - rc.y);
 }
+
+// Row-major walk over the tiles of a rectangle by T threads: thread `sub` takes
+// tiles sub, sub + T, ...  One division per walk, a few additions per step (with
+// a division per step the scatter of 1.2 M entries took 35 us from its early
+// launch, now 27).
+struct TileWalk {
+  uint32_t dx, tile, width, r, inc, skip;
+  __device__ __forceinline__ TileWalk(const ushort4 rc, uint32_t sub, uint32_t T, uint32_t tiles_x) {
+    width = (uint32_t)(rc.z + 1) - rc.x;
+    // Exact: sub, T < 2^12 lie at least 0.5 / 2^12 of themselves from the next quotient.
+    const float iw = __fdividef(1.0f, (float)width);
+    const uint32_t dy = (uint32_t)(((float)sub + 0.5f) * iw), q = (uint32_t)(((float)T + 0.5f) * iw);
+    dx = sub - dy * width;
+    tile = (rc.y + dy) * tiles_x + rc.x + dx;
+    r = T - q * width;
+    inc = q * tiles_x + r;
+    skip = tiles_x - width;
+  }
+  __device__ __forceinline__ void next() {
+    dx += r;
+    tile += inc;
+    if (dx >= width) {
+      dx -= width;
+      tile += skip;
+    }
+  }
+};
+
+// The Gaussians of a block (or round) that cover many tiles.  The few threads
+// that a Gaussian has in the two kernels below would walk a screen-sized
+// rectangle in hundreds of dependent steps with the whole block waiting for
+// them, so beyond kNarrow steps a thread a Gaussian goes to a whole warp (they
+// are dealt to the warps in turn), beyond kHuge tiles to all of the block.
+// The binning stage of 100k Gaussians at 640 x 512, 0.5% of them screen-sized:
+// 104 us, 287 without the lists (equal footprints with as many entries: 92);
+// 200k at 1280 x 1024: 225 and 937 us (205).  A limit of 16 or 64 steps is even
+// (a frame of 100k Gaussians of 55 tiles on average: 285 us at 32, 290 at 16
+// and at 64); kHuge only matters for a few in a block, as many make every warp
+// busy either way.
+template <int N>
+struct WideList {
+  uint32_t n[2];    // wide ones from the front of id, huge ones from its end
+  uint16_t id[N];
+  __device__ __forceinline__ void clear() { n[0] = n[1] = 0u; }
+  __device__ __forceinline__ void add(int i, bool huge) {
+    const int at = (int)atomicAdd(&n[huge], 1u);
+    id[huge ? N - 1 - at : at] = (uint16_t)i;
+  }
+  // Number of a warp's items, and the j-th of them.
+  __device__ __forceinline__ int mine(int warp, int warps) const { return ((int)n[0] - warp + warps - 1) / warps; }
+  __device__ __forceinline__ int items(int warp, int warps) const { return mine(warp, warps) + (int)n[1]; }
+  __device__ __forceinline__ int item(int j, int warp, int warps, bool& huge) const {
+    const int m = mine(warp, warps);
+    huge = j >= m;
+    return id[huge ? N - 1 - (j - m) : warp + j * warps];
+  }
+};
+constexpr int kNarrow = 32;     // steps of a thread
+constexpr int kHuge = 2048;     // tiles
+constexpr int kCountTPG = 4;    // threads per Gaussian in the count kernel
 
 // Step 2: block b (ticket) owns depth ranks [chunk b, chunk b + chunk), chunk
 // <= 256 ITEMS; thread t scans ranks ITEMS t, ...  Writes offs / offs_by_gid and
@@ -497,9 +555,13 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
   __shared__ uint64_t s_prefix;
   __shared__ uint32_t s_c[kThreads * ITEMS];
   __shared__ ushort4 s_rect[kThreads * ITEMS];
-  const int tid = threadIdx.x;
+  __shared__ WideList<kThreads * ITEMS> s_wide;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < a.ntiles; i += kThreads) s_cnt[i] = 0;
-  if (tid == 0) s_ticket = atomicAdd(a.ticket, 1u);
+  if (tid == 0) {
+    s_ticket = atomicAdd(a.ticket, 1u);
+    s_wide.clear();
+  }
   __syncthreads();
   const uint32_t b = s_ticket;
   const int64_t start = (int64_t)b * a.chunk;
@@ -514,6 +576,7 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
     cnt[i] = li < nloc ? a.touched[gid[i]] : 0u;
     s_c[li] = cnt[i];
     s_rect[li] = cnt[i] ? a.rect[gid[i]] : make_ushort4(0, 0, 0, 0);
+    if (cnt[i] > kNarrow * kCountTPG) s_wide.add(li, cnt[i] > kHuge);
     tsum += cnt[i];
   }
   uint32_t btot;
@@ -521,13 +584,21 @@ __global__ void __launch_bounds__(kThreads) bin_count_kernel(const CountArgs a) 
   // The block's total goes out at once; its tile counts, which do not need
   // the prefix, are taken while the predecessors resolve theirs.
   if (tid == 0) lookback64_publish(a.status, b, btot);
-  // Tile counts: four threads to a Gaussian, in any order.
-  for (int w = tid; w < 4 * nloc; w += kThreads) {
-    const uint32_t c = s_c[w >> 2];
-    if ((uint32_t)(w & 3) >= c) continue;
-    const ushort4 rc = s_rect[w >> 2];
-    const float iw = 1.0f / (float)(rc.z - rc.x + 1u);
-    for (uint32_t k = w & 3; k < c; k += 4) atomicAdd(&s_cnt[rect_tile(rc, iw, k, a.tiles_x)], 1u);
+  // Tile counts, in any order: four threads to a Gaussian, a warp or the block
+  // to a wide one.
+  for (int w = tid; w < kCountTPG * nloc; w += kThreads) {
+    const uint32_t c = s_c[w / kCountTPG], sub = (uint32_t)w % kCountTPG;
+    if (sub >= c || c > kNarrow * kCountTPG) continue;
+    TileWalk t(s_rect[w / kCountTPG], sub, kCountTPG, a.tiles_x);
+    for (uint32_t k = sub; k < c; k += kCountTPG, t.next()) atomicAdd(&s_cnt[t.tile], 1u);
+  }
+  const int items = s_wide.items(warp, kThreads / 32);
+  for (int j = 0; j < items; ++j) {
+    bool huge;
+    const int i = s_wide.item(j, warp, kThreads / 32, huge);
+    const uint32_t c = s_c[i], sub = huge ? tid : lane, T = huge ? kThreads : 32;
+    TileWalk t(s_rect[i], sub, T, a.tiles_x);
+    for (uint32_t k = sub; k < c; k += T, t.next()) atomicAdd(&s_cnt[t.tile], 1u);
   }
   if (tid < 32) {
     __syncwarp();
@@ -617,15 +688,15 @@ __global__ void __launch_bounds__(kThreads) table_scan_kernel(uint32_t* table, i
 // Gaussian i of the round is bit i / 4 of word i % 4: a warp's Gaussians lie
 // in different words and a Gaussian's threads on consecutive tiles, so the
 // ors of a warp spread over all banks, and the second visit reads a mask with
-// one 16-byte load.  Entries are spread over all threads of the block, several
-// to a Gaussian; the next round's Gaussians (three dependent loads) are
-// fetched while a round is worked on.
+// one 16-byte load.  Several threads take a Gaussian's entries, a warp or the
+// block those of a wide one (WideList); the next round's Gaussians (three
+// dependent loads) are fetched while a round is worked on.
 // Bound by the scattered 8-byte stores (a third to half of it: one sector
 // each) and by issue (two visits of every entry and a sweep of the tiles per
-// round).  1M Gaussians at 1280 x 1024, 33 M entries: 522 us from its early
+// round).  1M Gaussians at 1280 x 1024, 33 M entries: 512 us from its early
 // launch, 543 with suffix counts beside the masks and blocks of 512; 100k at
-// 640 x 512, 1.6 M entries, the stage alone: 24 us instead of 32; 1,000
-// Gaussians: 3 us, 27 with a warp walking its 64 Gaussians one after another.
+// 640 x 512, 1.2 M entries: 27 us; 1,000 Gaussians: 3 us, 27 with a warp walking
+// its 64 Gaussians one after another.
 // Block 0 also writes the tile ranges and marks the workspace as holding a
 // forward's state.
 struct ScatterArgs {
@@ -653,7 +724,9 @@ __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
   uint32_t* s_pos = s_dyn + 4 * a.ntiles;           // [ntiles]: next position of the tile's segment
   __shared__ uint2 s_id[2][kRound];  // id, first emission index
   __shared__ ushort4 s_rect[2][kRound];
-  const int tid = threadIdx.x;
+  __shared__ WideList<kRound> s_wide[2];
+  constexpr int TPG = NT / kRound;  // threads per Gaussian
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   const int64_t start = (int64_t)b * a.chunk;
   const int nloc = (int)min((int64_t)a.chunk, (int64_t)a.P - start);
@@ -666,11 +739,18 @@ __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
   const auto rect_of = [&](bool have, uint32_t g) {
     return have && a.touched[g] != 0u ? a.rect[g] : make_ushort4(1, 0, 0, 0);
   };
+  const auto put = [&](int to, const uint2 id, const ushort4 rc) {
+    s_id[to][tid] = id;
+    s_rect[to][tid] = rc;
+    const uint32_t c = rect_tiles(rc);
+    if (c > kNarrow * TPG) s_wide[to].add(tid, c > kHuge);
+  };
+  if (tid < 2) s_wide[tid].clear();
+  __syncthreads();
   if (tid < kRound) {
     const bool have = tid < nloc;
     const uint32_t g = have ? a.order[start + tid] : 0u;
-    s_id[0][tid] = make_uint2(g, have ? a.offs[start + tid] : 0u);
-    s_rect[0][tid] = rect_of(have, g);
+    put(0, make_uint2(g, have ? a.offs[start + tid] : 0u), rect_of(have, g));
   }
   for (int t = tid; t < a.ntiles; t += NT) {
     s_pos[t] = a.table[(size_t)t * a.nblocks + b];
@@ -682,12 +762,24 @@ __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
     }
   }
   if (b == 0 && tid == 0) a.hdr->has_forward = 1u;
-  constexpr int TPG = NT / kRound;  // threads per Gaussian
+  // Visits of Gaussian i of the round: its bit in the masks of its tiles k,
+  // k + step, ...; its entries of these tiles.
+  const auto mark = [&](int i, const ushort4 rc, uint32_t c, uint32_t k, uint32_t step) {
+    const uint32_t bit = 1u << (i >> 2);
+    for (TileWalk t(rc, k, step, a.tiles_x); k < c; k += step, t.next()) atomicOr(&s_word[4 * t.tile + (i & 3)], bit);
+  };
+  const auto emit = [&](int i, const uint2 id, const ushort4 rc, uint32_t c, uint32_t k, uint32_t step) {
+    // Bits of the Gaussians before i in the four words.
+    const int word = i & 3, bit = i >> 2;
+    const uint32_t below = (1u << bit) - 1u, upto = (2u << bit) - 1u;
+    const uint32_t m0 = word > 0 ? upto : below, m1 = word > 1 ? upto : below, m2 = word > 2 ? upto : below;
+    for (TileWalk t(rc, k, step, a.tiles_x); k < c; k += step, t.next()) {
+      const uint4 m = s_mask[t.tile];
+      const uint32_t pos = s_pos[t.tile] + __popc(m.x & m0) + __popc(m.y & m1) + __popc(m.z & m2) + __popc(m.w & below);
+      if ((uint64_t)pos < cap) a.sorted[pos] = make_uint2(id.y + k, id.x);
+    }
+  };
   const int i = tid / TPG, sub = tid % TPG;
-  const int word = i & 3, bit = i >> 2;
-  // Bits of the Gaussians before i in the four words.
-  const uint32_t below = (1u << bit) - 1u, upto = (2u << bit) - 1u;
-  const uint32_t m0 = word > 0 ? upto : below, m1 = word > 1 ? upto : below, m2 = word > 2 ? upto : below;
   __syncthreads();
   int buf = 0;
   for (int r0 = 0; r0 < nloc; r0 += kRound, buf ^= 1) {
@@ -696,27 +788,30 @@ __global__ void __launch_bounds__(NT) bin_scatter_kernel(const ScatterArgs a) {
     const bool have = tid < kRound && rn < nloc;
     uint2 nid = make_uint2(0u, 0u);
     if (have) nid = make_uint2(a.order[start + rn], a.offs[start + rn]);
+    // A thread's own Gaussian, unless it is a wide one; then the wide ones.
     const ushort4 rc = s_rect[buf][i];
-    const uint32_t width = (uint32_t)(rc.z + 1) - rc.x, c = width * ((uint32_t)(rc.w + 1) - rc.y);
-    const float iw = 1.0f / (float)width;
-    for (uint32_t k = sub; k < c; k += TPG) atomicOr(&s_word[4 * rect_tile(rc, iw, k, a.tiles_x) + word], 1u << bit);
+    const uint32_t c = rect_tiles(rc) <= kNarrow * TPG ? rect_tiles(rc) : 0u;
+    const int items = s_wide[buf].items(warp, NT / 32);
+    mark(i, rc, c, sub, TPG);
+    for (int j = 0; j < items; ++j) {
+      bool huge;
+      const int w = s_wide[buf].item(j, warp, NT / 32, huge);
+      const ushort4 wrc = s_rect[buf][w];
+      mark(w, wrc, rect_tiles(wrc), huge ? tid : lane, huge ? NT : 32);
+    }
     __syncthreads();
     const ushort4 nrc = rect_of(have, nid.x);
-    if (sub < c) {
-      const uint2 id = s_id[buf][i];
-      for (uint32_t k = sub; k < c; k += TPG) {
-        const uint32_t tile = rect_tile(rc, iw, k, a.tiles_x);
-        const uint4 m = s_mask[tile];
-        const uint32_t pos = s_pos[tile] + __popc(m.x & m0) + __popc(m.y & m1) + __popc(m.z & m2) + __popc(m.w & below);
-        if ((uint64_t)pos < cap) a.sorted[pos] = make_uint2(id.y + k, id.x);
-      }
+    if (sub < c) emit(i, s_id[buf][i], rc, c, sub, TPG);
+    for (int j = 0; j < items; ++j) {
+      bool huge;
+      const int w = s_wide[buf].item(j, warp, NT / 32, huge);
+      const ushort4 wrc = s_rect[buf][w];
+      emit(w, s_id[buf][w], wrc, rect_tiles(wrc), huge ? tid : lane, huge ? NT : 32);
     }
     if (r0 + kRound >= nloc) break;
-    if (tid < kRound) {
-      s_id[buf ^ 1][tid] = nid;
-      s_rect[buf ^ 1][tid] = nrc;
-    }
+    if (tid < kRound) put(buf ^ 1, nid, nrc);
     __syncthreads();
+    if (tid == 0) s_wide[buf].clear();  // of the round after the next
     for (int t = tid; t < a.ntiles; t += NT) {
       const uint4 m = s_mask[t];
       s_pos[t] += __popc(m.x) + __popc(m.y) + __popc(m.z) + __popc(m.w);
