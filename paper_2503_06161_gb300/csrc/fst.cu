@@ -756,6 +756,13 @@ __device__ __forceinline__ void tc_zero(float (&a)[NT][4], float (&b)[NT][4]) {
     for (int i = 0; i < 4; ++i) a[nt][i] = b[nt][i] = 0.0f;
 }
 
+// max(x, 0) that keeps a NaN.
+__device__ __forceinline__ float relu_nan(float x) {
+  float y;
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // Columns 8 nt + 2 t, + 1 of four tiles (rows fr, fr + 8) as steps k0 and
 // k0 + 1 of the next layer's first operand: relu(z + bias), three terms.
 template <int KS>
@@ -765,9 +772,66 @@ __device__ __forceinline__ void tc_relu(const float (&z)[4][4], const float* __r
   for (int nt = 0; nt < 4; ++nt) {
     const float b0 = __ldg(bias + 8 * nt + 2 * ft), b1 = __ldg(bias + 8 * nt + 2 * ft + 1);
     const int k = k0 + (nt >> 1), i = 2 * (nt & 1);
-    split3(fmaxf(z[nt][0] + b0, 0.0f), fmaxf(z[nt][1] + b1, 0.0f), out[0][k][i], out[1][k][i], out[2][k][i]);
-    split3(fmaxf(z[nt][2] + b0, 0.0f), fmaxf(z[nt][3] + b1, 0.0f), out[0][k][i + 1], out[1][k][i + 1], out[2][k][i + 1]);
+    split3(relu_nan(z[nt][0] + b0), relu_nan(z[nt][1] + b1), out[0][k][i], out[1][k][i], out[2][k][i]);
+    split3(relu_nan(z[nt][2] + b0), relu_nan(z[nt][3] + b1), out[0][k][i + 1], out[1][k][i + 1], out[2][k][i + 1]);
   }
+}
+
+// The outputs `todo` (bit b: branch b; bit 4 + s: feature columns of stage s, zt
+// columns each) of Gaussian p with FP32 products, by one warp, in the order of
+// fst_fwd_kernel's sums.  For the Gaussians whose values leave the range of
+// the three BF16 terms: an infinity, or anything that rounds to one in BF16,
+// splits into terms that give NaN, which relu_nan carries to every output
+// behind it; FP32 products keep infinities and clamp NaNs at the ReLUs.
+// (What a diverged plane or weight does must not depend on whether reverse state
+// is kept; the outputs that it does not reach cost 4 us of 540 at 200k.)
+static_assert((2 * kFW + 2 * kFHalf) * 4 <= 12 * 512, "works in the warp's part of shared memory");
+__device__ __noinline__ void fst_row_fp32(const TcArgs& a, float* buf, int p, uint32_t todo, int D, int zt) {
+  const FstGeom& g = a.g;
+  const int lane = threadIdx.x & 31;
+  float *x = buf, *y = buf + kFW, *e = buf + 2 * kFW, *u = e + kFHalf;
+  // acc + sum_k w[o][k] in[k], k ascending.
+  auto dot = [&](int layer, int o, int k0, const float* in, int K, float acc) {
+    const float* w = a.mlp + g.pw[layer] + (int64_t)o * g.nin[layer] + k0;
+    for (int k = 0; k < K; ++k) acc = fmaf(in[k], __ldg(w + k), acc);
+    return acc;
+  };
+  auto relu_layer = [&](int layer, const float* in, float* out) {
+    for (int o = lane; o < g.nout[layer]; o += 32)
+      out[o] = fmaxf(dot(layer, o, 0, in, g.nin[layer], 0.0f) + a.mlp[g.pb[layer] + o], 0.0f);
+    __syncwarp();
+  };
+  __syncwarp();
+  relu_layer(0, a.f + (size_t)p * g.levels * kFC, x);
+  for (int j = 1; j < kFDepth; ++j) {
+    relu_layer(j, x, y);
+    float* t = x;
+    x = y;
+    y = t;
+  }
+  const float* srcs[4] = {a.means, a.quats, a.log_scales, a.logits};
+  float* dsts[4] = {a.means_t, a.quats_t, a.log_scales_t, a.logits_t};
+  float v[2] = {0.0f, 0.0f};
+  for (int b = 0; b < 4; ++b) {
+    const int l1 = branch_e1(b), dg = branch_out(b);
+    relu_layer(l1, x, e);
+    relu_layer(l1 + 1, e, u);
+    if (((todo >> b) & 1u) && lane < dg) {
+      const size_t at = (size_t)p * dg + lane;
+      dsts[b][at] = srcs[b][at] + dot(l1 + 2, lane, 0, u, kFHalf, a.mlp[g.pb[l1 + 2] + lane]);
+    }
+    for (int h = 0; h < 2; ++h) v[h] = dot(kLZ1, lane + 32 * h, b * kFHalf, u, kFHalf, v[h]);
+    __syncwarp();
+  }
+  for (int h = 0; h < 2; ++h) y[lane + 32 * h] = fmaxf(v[h] + a.mlp[g.pb[kLZ1] + lane + 32 * h], 0.0f);
+  __syncwarp();
+  for (int o = lane; o < D; o += 32) {
+    if (!((todo >> (4 + o / zt)) & 1u)) continue;
+    const size_t at = (size_t)p * D + o;
+    const float z = dot(kLZ2, o, 0, y, kFW, 0.0f);
+    store_feat(a.feat_t, a.feat_bf16, at, load_feat(a.feat, a.feat_bf16, at) + z + a.mlp[g.pb[kLZ2] + o]);
+  }
+  __syncwarp();
 }
 
 template <int D>
@@ -865,6 +929,16 @@ __global__ void __launch_bounds__(kTcThreads, 2) fst_fwd_tc_kernel(const __grid_
     for (int i = 0; i < 4; ++i) v[nt][i] = 0.0f;
   const float* srcs[4] = {a.means, a.quats, a.log_scales, a.logits};
   float* dsts[4] = {a.means_t, a.quats_t, a.log_scales_t, a.logits_t};
+  // Outputs of rows fr and fr + 8 that are left to fst_row_fp32 (its bits).
+  uint32_t todo[2] = {0u, 0u};
+  auto finite = [&](const float (&x)[2], int r, uint32_t bit) -> bool {
+    const uint32_t bad = __ballot_sync(0xFFFFFFFFu, valid[r] && !(isfinite(x[0]) && isfinite(x[1])));
+    if ((bad >> (4 * fr)) & 15u) {
+      todo[r] |= bit;
+      return false;
+    }
+    return true;
+  };
 #pragma unroll 1
   for (int b = 0; b < 4; ++b) {
     const int l1 = branch_e1(b);
@@ -903,11 +977,20 @@ __global__ void __launch_bounds__(kTcThreads, 2) fst_fwd_tc_kernel(const __grid_
       const int dg = branch_out(b);
       const float* bias = a.mlp + g.pb[l1 + 2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int o = 2 * ft + (i & 1), r = i >> 1;
-        if (o < dg && valid[r]) {
-          const size_t at = (size_t)p[r] * dg + o;
-          dsts[b][at] = srcs[b][at] + ((oh[0][i] + os[0][i]) + __ldg(bias + o));
+      for (int r = 0; r < 2; ++r) {
+        float off[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int o = 2 * ft + i;
+          off[i] = o < dg ? (oh[0][2 * r + i] + os[0][2 * r + i]) + __ldg(bias + o) : 0.0f;
+        }
+        if (finite(off, r, 1u << b)) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int o = 2 * ft + i;
+            const size_t at = (size_t)p[r] * dg + o;
+            if (o < dg && valid[r]) dsts[b][at] = srcs[b][at] + off[i];
+          }
         }
       }
     }
@@ -943,15 +1026,35 @@ __global__ void __launch_bounds__(kTcThreads, 2) fst_fwd_tc_kernel(const __grid_
     for (int ks = 0; ks < 4; ++ks) tc_step<ZT>(x[0][ks], x[1][ks], x[2][ks], w + ks * ZT * 768, lane, dh, ds);
     const float* bias = a.mlp + g.pb[kLZ2] + n0;
 #pragma unroll
-    for (int nt = 0; nt < ZT; ++nt)
+    for (int r = 0; r < 2; ++r) {
+      // (A sum of the row's values is finite only if each of them is.)
+      float any[2] = {0.0f, 0.0f};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int c = 8 * nt + 2 * ft + (i & 1), r = i >> 1;
-        if (valid[r]) {
-          const size_t at = (size_t)p[r] * D + n0 + c;
-          store_feat(a.feat_t, a.feat_bf16, at, load_feat(a.feat, a.feat_bf16, at) + (dh[nt][i] + ds[nt][i]) + __ldg(bias + c));
+      for (int nt = 0; nt < ZT; ++nt)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          dh[nt][2 * r + i] += ds[nt][2 * r + i];
+          any[i] += dh[nt][2 * r + i];
         }
-      }
+      if (!finite(any, r, 16u << (n0 / (8 * ZT)))) continue;
+#pragma unroll
+      for (int nt = 0; nt < ZT; ++nt)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int c = 8 * nt + 2 * ft + i;
+          if (valid[r]) {
+            const size_t at = (size_t)p[r] * D + n0 + c;
+            store_feat(a.feat_t, a.feat_bf16, at, load_feat(a.feat, a.feat_bf16, at) + dh[nt][2 * r + i] + __ldg(bias + c));
+          }
+        }
+    }
+  }
+  if (__any_sync(0xFFFFFFFFu, (todo[0] | todo[1]) != 0u)) {
+#pragma unroll 1
+    for (int r = 0; r < 16; ++r) {
+      const uint32_t w = __shfl_sync(0xFFFFFFFFu, r < 8 ? todo[0] : todo[1], 4 * (r & 7));
+      if (w) fst_row_fp32(a, reinterpret_cast<float*>(s_h), (int)blockIdx.x * kTcRows + warp * 16 + r, w, D, 8 * ZT);
+    }
   }
 }
 
