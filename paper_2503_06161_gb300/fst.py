@@ -26,7 +26,7 @@ class FSTDeform:
     def __init__(self, planes: torch.Tensor, mlp: torch.Tensor, levels: int, rs: int, rt: int, D: int, bbox_min,
                  bbox_max, P: int, with_backward: bool = True, device="cuda", exact_planes: bool = False):
         """exact_planes: plane gradients as exact fixed-point sums (bitwise
-        reproducible, about twice the reverse's time) instead of float
+        reproducible, about three times the reverse's time) instead of float
         atomics."""
         self.levels, self.rs, self.rt, self.D, self.P = int(levels), int(rs), int(rt), int(D), int(P)
         self.exact_planes = bool(exact_planes)
