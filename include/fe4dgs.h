@@ -361,7 +361,7 @@ typedef struct {
   int exact_planes;      /* reverse: 0 = plane gradients summed with float atomics (fast; the
                             last bits depend on the order of the additions); 1 = summed exactly
                             in fixed point, bitwise reproducible (workspace with_backward = 2;
-                            about twice the reverse's time) */
+                            about three times the reverse's time) */
 } fe_fst;
 
 /* Float counts of the plane and MLP arrays (0 for invalid arguments). */
@@ -398,7 +398,8 @@ fe_status fe_fst_forward(const fe_fst *fst, int P, const float *means, const flo
  * means and t).  Inputs: the gradients of the loss with respect to the
  * deformed arrays (device float32, layouts as above; d_feat_t [P,D]) --
  * e.g. the fe_grads of a render of the deformed Gaussians; d_feat_t 16-byte
- * aligned.  Because the
+ * aligned; fst->planes may be a copy that is not (4-byte accesses then, as
+ * for a d_planes that is not).  Because the
  * offsets are added, these are also the gradients of the offsets and of
  * the canonical quats, log_scales, opacity logits and features.  Outputs
  * (device float32, overwritten):

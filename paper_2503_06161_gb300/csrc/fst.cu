@@ -1624,8 +1624,8 @@ __device__ __forceinline__ void red_add4(float4* p, float x, float y, float z, f
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
-// How plane gradients are added: 16-byte atomics, 4-byte atomics (a gradient
-// array that is not 16-byte aligned), or exactly (fixed_add).  With the
+// How plane gradients are added: 16-byte atomics, 4-byte atomics (planes or a
+// gradient array that are not 16-byte aligned), or exactly (fixed_add).  With the
 // element-wise atomics lane q has channels q, q + 8, ..., so that each
 // instruction covers whole 32- or 64-byte pieces of a corner; with four
 // neighbouring channels to a lane they take four times the sectors (50k
@@ -2058,7 +2058,7 @@ extern "C" fe_status fe_fst_backward(const fe_fst* fst, int P, const float* mean
     return cudaMemsetAsync(d_mlp, 0, (size_t)g.mlp_packed * 4, st) == cudaSuccess ? FE_OK : FE_ERR_CUDA;
   }
   if (!fst->planes || !means || !d_means_t || !d_quats_t || !d_log_scales_t || !d_opacity_logits_t || !d_feat_t ||
-      !d_means || !al16p(d_feat_t) || !al16p(fst->planes))
+      !d_means || !al16p(d_feat_t))
     return FE_ERR_INVALID_ARG;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   unsigned long long* acc_hi = exact ? reinterpret_cast<unsigned long long*>(ws + w.acc) : nullptr;
@@ -2116,7 +2116,7 @@ extern "C" fe_status fe_fst_backward(const fe_fst* fst, int P, const float* mean
     } else {
       const size_t lb = line_bytes(g);
       if (cudaMemsetAsync(h.lines, 0, lb, st) != cudaSuccess) return FE_ERR_CUDA;
-      if (al16p(d_planes)) fst_hex_bwd_kernel<PlaneAdd::kVector><<<hb, kHexThreads, 0, st>>>(h);
+      if (al16p(d_planes) && al16p(fst->planes)) fst_hex_bwd_kernel<PlaneAdd::kVector><<<hb, kHexThreads, 0, st>>>(h);
       else fst_hex_bwd_kernel<PlaneAdd::kScalar><<<hb, kHexThreads, 0, st>>>(h);
       const int64_t nl = (int64_t)(lb / 16 / kLineCopies);
       fst_lines_out_kernel<<<(int)((nl + 255) / 256), 256, 0, st>>>(g, h.lines, t, d_planes, nl);
