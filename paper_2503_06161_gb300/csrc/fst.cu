@@ -1794,10 +1794,17 @@ struct TvArgs {
   int bstart[kFMaxL * 6 + 1];       // first block of each plane (blocks in proportion to plane size)
 };
 
+template <bool kQuads>
+__device__ __forceinline__ float4 load4(const float* p) {
+  return kQuads ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
+}
+
 // Each plane gets a share of the blocks in proportion to its size; each
 // thread takes four channels of a node (the planes are channels-last, so a
-// float4 per neighbour).  One loss partial per block, summed in a fixed
-// order afterwards.
+// float4 per neighbour; kQuads: both arrays are 16-byte aligned, else four
+// 4-byte accesses of the same sums).  One loss partial per block, summed in a
+// fixed order afterwards.
+template <bool kQuads>
 __global__ void __launch_bounds__(256) fst_tv_kernel(const TvArgs a) {
   __shared__ float s_w[8];
   const FstGeom& g = a.g;
@@ -1805,8 +1812,9 @@ __global__ void __launch_bounds__(256) fst_tv_kernel(const TvArgs a) {
   while (k + 1 < g.levels * 6 && (int)blockIdx.x >= a.bstart[k + 1]) ++k;
   const int b0 = a.bstart[k], nb = a.bstart[k + 1] - b0;
   const int ra = g.pra[k], rb = g.prb[k];
-  const float4* pl = reinterpret_cast<const float4*>(a.planes + g.poff[k]);
-  float4* dp = reinterpret_cast<float4*>(a.d_planes + g.poff[k]);
+  const float* planes = a.planes + g.poff[k];
+  float* d_planes = a.d_planes + g.poff[k];
+  const auto pl = [&](int e) { return load4<kQuads>(planes + 4 * (int64_t)e); };
   const int q4 = kFC / 4;
   const int total = ra * rb * q4;
   const float ia = 1.0f / (float)((int64_t)(ra - 1) * rb * kFC), ib = 1.0f / (float)((int64_t)ra * (rb - 1) * kFC);
@@ -1814,7 +1822,7 @@ __global__ void __launch_bounds__(256) fst_tv_kernel(const TvArgs a) {
   for (int e = ((int)blockIdx.x - b0) * blockDim.x + threadIdx.x; e < total; e += nb * blockDim.x) {
     const int node = e / q4;
     const int i = node / rb, j = node - i * rb;
-    const float4 v = pl[e];
+    const float4 v = pl(e);
     float4 gr = make_float4(0.f, 0.f, 0.f, 0.f);
     auto term = [&](const float4 n, float w, bool forward) {
       // forward: n is the next node (difference n - v, counted in the loss)
@@ -1824,13 +1832,18 @@ __global__ void __launch_bounds__(256) fst_tv_kernel(const TvArgs a) {
       const float s = forward ? -2.0f * w : 2.0f * w;
       gr.x += s * d.x; gr.y += s * d.y; gr.z += s * d.z; gr.w += s * d.w;
     };
-    if (i + 1 < ra) term(pl[e + rb * q4], ia, true);
-    if (i > 0) term(pl[e - rb * q4], ia, false);
-    if (j + 1 < rb) term(pl[e + q4], ib, true);
-    if (j > 0) term(pl[e - q4], ib, false);
-    float4 o = dp[e];
+    if (i + 1 < ra) term(pl(e + rb * q4), ia, true);
+    if (i > 0) term(pl(e - rb * q4), ia, false);
+    if (j + 1 < rb) term(pl(e + q4), ib, true);
+    if (j > 0) term(pl(e - q4), ib, false);
+    float* dp = d_planes + 4 * (int64_t)e;
+    float4 o = load4<kQuads>(dp);
     o.x += a.weight * gr.x; o.y += a.weight * gr.y; o.z += a.weight * gr.z; o.w += a.weight * gr.w;
-    dp[e] = o;
+    if (kQuads) {
+      *reinterpret_cast<float4*>(dp) = o;
+    } else {
+      dp[0] = o.x; dp[1] = o.y; dp[2] = o.z; dp[3] = o.w;
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, o);
@@ -2156,7 +2169,8 @@ extern "C" fe_status fe_fst_tv(const fe_fst* fst, float weight, float* loss, flo
     a.bstart[k + 1] = a.bstart[k] + 1 + (int)(budget * n / total);
   }
   const int nblk = a.bstart[np];
-  fst_tv_kernel<<<nblk, 256, 0, st>>>(a);
+  if (al16p(fst->planes) && al16p(d_planes)) fst_tv_kernel<true><<<nblk, 256, 0, st>>>(a);
+  else fst_tv_kernel<false><<<nblk, 256, 0, st>>>(a);
   fst_tv_finish<<<1, 256, 0, st>>>(scratch, nblk, weight, loss);
   return cudaGetLastError() == cudaSuccess ? FE_OK : FE_ERR_CUDA;
 }

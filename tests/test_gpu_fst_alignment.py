@@ -62,3 +62,25 @@ def test_reverse_takes_unaligned_planes(P, levels, D, skew_p, skew_d, exact):
         assert np.array_equal(got[1], want[1])
     else:
         assert rel_err(got[1], want[1]) < 1e-4
+
+
+@pytest.mark.parametrize("skew_p,skew_d", [(0, 1), (3, 0), (2, 2)])
+def test_total_variation_takes_unaligned_arrays(skew_p, skew_d):
+    # The reverse's gradient array may be unaligned, and the TV term is added
+    # to that same array.  Same sums in the same order: same bits.
+    levels, rs, rt, D = 2, 6, 5, 16
+    _, fst, _ = _case(1, levels, rs, rt, D, False)
+    base = torch.randn(fst.planes.numel(), generator=torch.Generator(device="cuda").manual_seed(8), device="cuda")
+
+    def tv(planes, d_planes):
+        loss, scratch = torch.zeros(1, device="cuda"), torch.empty(1024, device="cuda")
+        _lib.fe_fst_tv(_lib.make_fst(levels, rs, rt, D, planes, fst.mlp, LO, HI), 0.7, loss, d_planes, scratch)
+        torch.cuda.synchronize()
+        return loss.item(), d_planes.clone()
+
+    want = tv(fst.planes, base.clone())
+    store, d_planes = _view(base, skew_d)
+    got = tv(_view(fst.planes, skew_p)[1], d_planes)
+    assert got[0] == want[0]
+    assert torch.equal(got[1], want[1])
+    assert torch.isnan(store[:skew_d]).all() and torch.isnan(store[skew_d + d_planes.numel():]).all()
