@@ -23,16 +23,25 @@ namespace fe {
 namespace {
 
 // Gaussians per staged batch of the forward (two batches are in flight) and
-// blocks per SM.  Most tiles end within the first 200 entries of their list,
-// so at D = 32 batches of 64 land sooner and load less past the end (200k
-// Gaussians, 640 x 512: 167 us, 176 with 128, 182 with 32); at D = 16 two
-// blocks with room for registers and batches of 128 are the faster (30k,
-// 333 x 251: 57 us; three blocks 68, batches of 64 66), at D = 32 two and
-// three blocks are even.
+// blocks per SM, by the channels and the tiles of the launch.  Most tiles end
+// within the first 200 entries of their list, so batches of 64 land sooner and
+// load less past the end, but stop the block twice as often: with several
+// waves of tiles D = 32 takes 64 (frames of 200k Gaussians at 640 x 512: 279 us,
+// 282 with 128, 289 with 32; 100k at 1280 x 1024: 661, 671, 687), with all tiles
+// resident at once 128 (1,500 at 96 x 72: 57 us, 61 with 64; 30k at 160 x 128:
+// 169 and 176).  D = 16 takes two blocks per SM, whose registers suffice, while
+// the tiles fit about one such wave, else three (frames at two and three
+// blocks: 30k at 320 x 240, 300 tiles, 98 and 111 us; at 333 x 251, 336 tiles,
+// 102 and 114; at 352 x 288, 396 tiles, 111 and 111; at 384 x 288 117 and 109;
+// at 640 x 512 171 and 160; 100k at 352 x 288 141 and 125).
+constexpr int kSMs = 152;
 template <int D>
-constexpr int fwd_batch() { return D == 16 ? 128 : (D <= 64 ? 64 : 32); }
+constexpr int fwd_batch() { return D <= 16 ? 128 : (D <= 64 ? 64 : 32); }
 template <int D>
-constexpr int fwd_blocks() { return D == 32 ? 3 : (D <= 64 ? 2 : 1); }
+int fwd_batch_for(int tiles) { return D == 32 && tiles <= 3 * kSMs ? 128 : fwd_batch<D>(); }
+template <int D>
+constexpr int fwd_blocks() { return D <= 32 ? 3 : (D <= 64 ? 2 : 1); }
+constexpr int kTwoBlockTiles = 2 * kSMs + kSMs / 4;
 
 // Bytes of one staged batch: B render records (48 bytes each), then B
 // feature rows in their stored format (fp32 or bf16).
@@ -357,8 +366,8 @@ __device__ __forceinline__ void stage_init(uint64_t* s_bar) {
 }
 
 // One block per tile.
-template <int D, int B, bool kCount>
-__global__ void __launch_bounds__(kThreads, fwd_blocks<D>()) composite_fwd_kernel(const CompositeArgs a) {
+template <int D, int B, bool kCount, int NB>
+__global__ void __launch_bounds__(kThreads, NB) composite_fwd_kernel(const CompositeArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar[2];
   __shared__ int s_abort[2];
@@ -381,8 +390,8 @@ __device__ __forceinline__ int batch_view(const BatchCompositeArgs& ba, int item
 // Persistent form over a batch of views: each block takes (view, tile)
 // items from a device counter until the batch is exhausted (no block waits
 // for another: items are independent).
-template <int D, int B>
-__global__ void __launch_bounds__(kThreads, fwd_blocks<D>())
+template <int D, int B, int NB>
+__global__ void __launch_bounds__(kThreads, NB)
     composite_fwd_batch_kernel(const __grid_constant__ BatchCompositeArgs ba) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar[2];
@@ -951,10 +960,10 @@ __global__ void __launch_bounds__(kThreads, D <= 32 ? 2 : 1)
   }
 }
 
-template <int D, int B, bool kCount>
+template <int D, int B, bool kCount, int NB = fwd_blocks<D>()>
 cudaError_t launch_fwd_t(const CompositeArgs& a, cudaStream_t st) {
   const size_t smem = fwd_smem_bytes(B, D, a.feat_bf16);
-  auto k = composite_fwd_kernel<D, B, kCount>;
+  auto k = composite_fwd_kernel<D, B, kCount, NB>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   return launch_pdl(k, a.ntiles, kThreads, smem, st, a);
 }
@@ -963,12 +972,16 @@ cudaError_t launch_fwd_t(const CompositeArgs& a, cudaStream_t st) {
 // form runs with the default batch only.
 template <int D>
 cudaError_t launch_fwd_d(const CompositeArgs& a, int B, cudaStream_t st) {
-  if (B == 0) B = fwd_batch<D>();
+  if (a.counts && B == 0) B = fwd_batch<D>();
+  if (B == 0) B = fwd_batch_for<D>(a.ntiles);
   if (a.counts) return B == fwd_batch<D>() ? launch_fwd_t<D, fwd_batch<D>(), true>(a, st) : cudaErrorInvalidValue;
   switch (B) {
     case 32: return launch_fwd_t<D, 32, false>(a, st);
     case 64: return launch_fwd_t<D, 64, false>(a, st);
     case 128:
+      if constexpr (D == 16) {
+        if (a.ntiles <= kTwoBlockTiles) return launch_fwd_t<D, 128, false, 2>(a, st);
+      }
       if constexpr (D <= 64) return launch_fwd_t<D, 128, false>(a, st);
       break;
   }
@@ -998,10 +1011,10 @@ cudaError_t persistent_grid(Kern k, size_t smem, int nitems, int& grid) {
   return cudaSuccess;
 }
 
-template <int D, int B>
+template <int D, int B, int NB = fwd_blocks<D>()>
 cudaError_t launch_fwd_batch_t(const BatchCompositeArgs& b, int bf16, cudaStream_t st) {
   const size_t smem = fwd_smem_bytes(B, D, bf16);
-  auto k = composite_fwd_batch_kernel<D, B>;
+  auto k = composite_fwd_batch_kernel<D, B, NB>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int grid = 1;
   if (e == cudaSuccess) e = persistent_grid(k, smem, b.nitems, grid);
@@ -1011,11 +1024,14 @@ cudaError_t launch_fwd_batch_t(const BatchCompositeArgs& b, int bf16, cudaStream
 
 template <int D>
 cudaError_t launch_fwd_batch_d(const BatchCompositeArgs& b, int bf16, int B, cudaStream_t st) {
-  if (B == 0) B = fwd_batch<D>();
+  if (B == 0) B = fwd_batch_for<D>(b.nitems);
   switch (B) {
     case 32: return launch_fwd_batch_t<D, 32>(b, bf16, st);
     case 64: return launch_fwd_batch_t<D, 64>(b, bf16, st);
     case 128:
+      if constexpr (D == 16) {
+        if (b.nitems <= kTwoBlockTiles) return launch_fwd_batch_t<D, 128, 2>(b, bf16, st);
+      }
       if constexpr (D <= 64) return launch_fwd_batch_t<D, 128>(b, bf16, st);
       break;
   }
