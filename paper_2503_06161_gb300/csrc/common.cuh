@@ -88,12 +88,16 @@ constexpr int kPChunk = kThreads * kPItems;
 // Depth-ordered Gaussians per block of the tile count / scatter kernels: 512
 // where that gives every SM a block (longer runs of a tile's list per block,
 // a smaller (tile, block) table), else fewer, down to one round of the
-// scatter (128), so that a small scene is not left to a few blocks; 1024 from
-// four blocks per SM up (1M Gaussians at 1280 x 1024: counts 122 -> 101 us,
-// table scan 85 -> 64, scatter 536 -> 522, training iteration 4667 -> 4613).
+// scatter (128), so that a small scene is not left to a few blocks (512
+// throughout: a frame of 30k Gaussians at 333 x 251 105 us for 101, of 3k at
+// 1280 x 1024 188 for 164).  1024 from four blocks per SM up and where the
+// table is what counts (frames with 1024 and 512, D = 16 BF16: 630k Gaussians at
+// 1280 x 1024 963 and 986 us, 1M 1251 and 1302, 1M at 1920 x 1080 1907 and
+// 1977; but 1M at 1024 x 800, 3200 tiles, 865 and 863, at 640 x 512 493 and
+// 482: the few blocks of the near Gaussians have the most entries).
 constexpr int kBinChunk = 1024;
-inline int bin_chunk(int64_t P) {
-  return P >= 152 * 4 * kBinChunk ? kBinChunk : P >= 152 * 512 ? 512 : (P >= 152 * 256 ? 256 : 128);
+inline int bin_chunk(int64_t P, int ntiles) {
+  return P >= 152 * 4 * kBinChunk && ntiles > 4096 ? kBinChunk : P >= 152 * 512 ? 512 : (P >= 152 * 256 ? 256 : 128);
 }
 
 // Ticket slots in the header.
@@ -134,7 +138,7 @@ inline Layout make_layout(int P, int D, int W, int H, int tw, int th, int64_t ca
   const size_t Pn = (size_t)(P > 0 ? P : 1);
   const size_t Kn = (size_t)(cap > 0 ? cap : 1);
   L.pblocks = ceil_div((int64_t)Pn, kPChunk);
-  L.bchunk = bin_chunk((int64_t)Pn);
+  L.bchunk = bin_chunk((int64_t)Pn, L.ntiles);
   L.bblocks = ceil_div((int64_t)Pn, L.bchunk);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };

@@ -20,7 +20,9 @@ import test_gpu_render  # noqa: E402
 @pytest.mark.parametrize("P,W,H,tile,share", [
     (300, 640, 512, (16, 16), 1.0), (2000, 640, 512, (16, 16), 0.05), (1, 640, 512, (16, 16), 1.0),
     (129, 333, 251, (8, 32), 0.5), (3000, 1600, 1200, (16, 16), 0.02), (257, 1600, 1200, (16, 16), 0.7),
-    (1500, 4096, 64, (16, 16), 0.05), (700, 64, 4096, (32, 8), 0.05), (40000, 1300, 1000, (16, 16), 0.003)])
+    (1500, 4096, 64, (16, 16), 0.05), (700, 64, 4096, (32, 8), 0.05), (40000, 1300, 1000, (16, 16), 0.003),
+    # Either side of the largest blocks' limits (Gaussians, tiles).
+    (622592, 1100, 1000, (16, 16), 0.0005), (622591, 1100, 1000, (16, 16), 0.0), (622592, 1024, 1024, (16, 16), 0.0)])
 def test_lists_bit_exact(P, W, H, tile, share, monkeypatch):
     rng = np.random.default_rng(P + W)
     uv = np.c_[rng.uniform(-20, W + 20, P), rng.uniform(-20, H + 20, P)].astype(np.float32)
