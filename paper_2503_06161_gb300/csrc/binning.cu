@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads) depth_hist_kernel(const uint32_t* ke
 // ---------------------------------------------------------------------------
 // One stable LSD radix pass (8-bit digit at `shift`) with decoupled look-back.
 // Block b (taken from an atomic ticket so predecessors are always running)
-// handles elements [b*4096, b*4096+4096); warp w its sub-chunk of 512.
+// handles elements [256 ITEMS b, 256 ITEMS (b + 1)); warp w 32 ITEMS of them.
 // ---------------------------------------------------------------------------
 template <int ITEMS>
 struct PassSmem {
@@ -104,7 +104,7 @@ struct PassSmem {
 template <bool kIdentVals, int ITEMS>
 __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* keys_in, const uint32_t* vals_in,
                                                             uint32_t* keys_out, uint32_t* vals_out,
-                                                            const uint32_t* n_dev, int64_t n_cap, int shift,
+                                                            int64_t n_elems, int shift,
                                                             const uint32_t* hist, uint32_t* status,
                                                             uint32_t* ticket, uint32_t* err) {
   constexpr int CHUNK = kThreads * ITEMS;
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint32_t* keys
   grid_dep_wait();
   grid_dep_launch();
   const uint32_t b = sm.ticket;
-  const uint64_t n = n_dev ? min((uint64_t)*n_dev, (uint64_t)n_cap) : (uint64_t)n_cap;
+  const uint64_t n = (uint64_t)n_elems;
   const uint64_t start = (uint64_t)b * CHUNK;
   if (start >= n) return;
   const uint32_t cnt = (uint32_t)min((uint64_t)CHUNK, n - start);
@@ -897,7 +897,7 @@ cudaError_t launch_binning(BinArgs& b, cudaStream_t st) {
       const int i = p & 1, o = i ^ 1;
       e = launch_pdl(p == 0 ? onesweep_kernel<true, kPItems> : onesweep_kernel<false, kPItems>, pblocks, kThreads,
                      ppass_smem, st, (const uint32_t*)b.dkey[i], p == 0 ? (const uint32_t*)nullptr : (const uint32_t*)b.dval[i],
-                     b.dkey[o], b.dval[o], (const uint32_t*)nullptr, (int64_t)P, 8 * p, (const uint32_t*)(b.hist + 256 * p),
+                     b.dkey[o], b.dval[o], (int64_t)P, 8 * p, (const uint32_t*)(b.hist + 256 * p),
                      status_depth + (size_t)p * pblocks * 256, hdr->ticket + kTicketDepth0 + p, &hdr->err);
       if (e != cudaSuccess) return e;
     }

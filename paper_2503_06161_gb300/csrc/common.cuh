@@ -78,11 +78,7 @@ struct Header {           // first 256 bytes of every workspace
 };
 static_assert(sizeof(Header) == 256, "header is 256 bytes");
 
-// Radix / scan chunking: 256 threads x 16 items over the K list entries,
-// 256 threads x 4 items over the P Gaussians (so P-sized passes still fill
-// all SMs).
-constexpr int kSortItems = 16;
-constexpr int kSortChunk = kThreads * kSortItems;
+// Radix / scan chunking: 256 threads x 8 items.
 constexpr int kPItems = 8;
 constexpr int kPChunk = kThreads * kPItems;
 // Depth-ordered Gaussians per block of the tile count / scatter kernels: 512
@@ -149,7 +145,7 @@ inline Layout make_layout(int P, int D, int W, int H, int tw, int th, int64_t ca
   L.status_words = (size_t)L.pblocks * 256 * 4 + 2 * (size_t)L.bblocks + 2 * L.table_blocks;
   // What a forward clears lies together at the start (one memset).
   L.hdr = take(sizeof(Header));
-  L.hist = take((4 + 3) * 256 * 4);
+  L.hist = take(4 * 256 * 4);
   L.status = take(L.status_words * 4);
   L.ranges = take((size_t)L.ntiles * 8);
   L.cleared = off;

@@ -28,10 +28,10 @@
 // complete, so the next tile's feature terms load while the epilogue
 // finishes this tile.
 #include <cuda.h>
-#include <cuda_bf16.h>
 
 #include "common.cuh"
 #include "kernels.h"
+#include "mma.cuh"
 #include "tc.cuh"
 
 namespace fe {
@@ -86,26 +86,11 @@ __device__ __forceinline__ uint32_t chunk_off(int r, int c, int row_bytes) {
                          : (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4));
 }
 
-// Three-term BF16 split of a pair (low half = first value).
-__device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-  auto pack = [](float x, float y) -> uint32_t {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
-    return *reinterpret_cast<const uint32_t*>(&v);
-  };
-  hi = pack(a, b);
-  a -= __uint_as_float(hi << 16);
-  b -= __uint_as_float(hi & 0xFFFF0000u);
-  mid = pack(a, b);
-  a -= __uint_as_float(mid << 16);
-  b -= __uint_as_float(mid & 0xFFFF0000u);
-  lo = pack(a, b);
-}
-
 // Eight consecutive values as one 16-byte chunk of each term's row.
 __device__ __forceinline__ void store_split8(unsigned char* base, uint32_t term_bytes, uint32_t off, const float* x) {
   uint32_t h[4], m[4], l[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) split_pair(x[2 * i], x[2 * i + 1], h[i], m[i], l[i]);
+  for (int i = 0; i < 4; ++i) split3(x[2 * i], x[2 * i + 1], h[i], m[i], l[i]);
   *reinterpret_cast<uint4*>(base + off) = make_uint4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<uint4*>(base + term_bytes + off) = make_uint4(m[0], m[1], m[2], m[3]);
   *reinterpret_cast<uint4*>(base + 2 * term_bytes + off) = make_uint4(l[0], l[1], l[2], l[3]);

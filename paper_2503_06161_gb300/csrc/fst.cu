@@ -356,13 +356,12 @@ __device__ __forceinline__ const float* next_tile(const WTile* tiles, int ntiles
 
 struct FwdArgs {
   FstGeom g;
-  const float *planes, *wt;
+  const float* wt;
   WTile tiles[kMaxWTiles];
   int ntiles;
   const float *means, *quats, *log_scales, *logits;
   const void* feat;
   int feat_bf16;
-  float t;
   float *means_t, *quats_t, *log_scales_t, *logits_t;
   void* feat_t;
   float* act;
@@ -2006,7 +2005,6 @@ extern "C" fe_status fe_fst_forward(const fe_fst* fst, int P, const float* means
   fst_pack_kernel<<<(int)((g.mlp_packed + 255) / 256), 256, 0, st>>>(g, fst->mlp, wt, wn);
   FwdArgs a{};
   a.g = g;
-  a.planes = fst->planes;
   a.wt = wt;
   a.means = means;
   a.quats = quats;
@@ -2014,7 +2012,6 @@ extern "C" fe_status fe_fst_forward(const fe_fst* fst, int P, const float* means
   a.logits = opacity_logits;
   a.feat = feat;
   a.feat_bf16 = feat_bf16 ? 1 : 0;
-  a.t = t;
   a.means_t = means_t;
   a.quats_t = quats_t;
   a.log_scales_t = log_scales_t;

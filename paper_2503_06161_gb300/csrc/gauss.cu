@@ -10,10 +10,9 @@
 //              deformation query back to the canonical parameters (the MLP
 //              reverse, from the forward's unit masks, on the tensor cores:
 //              deform_mlp.cu).
-#include <cuda_bf16.h>
-
 #include "common.cuh"
 #include "kernels.h"
+#include "mma.cuh"
 
 namespace fe {
 
@@ -326,21 +325,13 @@ __global__ void __launch_bounds__(kThreads) hexplane_split_kernel(const GaussArg
     f[2] *= w00 * x[0].z + w10 * x[2].z + w01 * x[1].z + w11 * x[3].z;
     f[3] *= w00 * x[0].w + w10 * x[2].w + w01 * x[1].w + w11 * x[3].w;
   }
-  auto pack = [](float x, float y) -> uint32_t {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
-    return *reinterpret_cast<const uint32_t*>(&v);
-  };
+  uint32_t x01[3], x23[3];
+  split3(f[0], f[1], x01[0], x01[1], x01[2]);
+  split3(f[2], f[3], x23[0], x23[1], x23[2]);
   const size_t term = (size_t)a.P * (C / 4);
   uint2* out = reinterpret_cast<uint2*>(a.fsplit) + (size_t)g * (C / 4) + q;
 #pragma unroll
-  for (int t = 0; t < 3; ++t) {
-    const uint2 h = make_uint2(pack(f[0], f[1]), pack(f[2], f[3]));
-    out[t * term] = h;
-    f[0] -= __uint_as_float(h.x << 16);
-    f[1] -= __uint_as_float(h.x & 0xFFFF0000u);
-    f[2] -= __uint_as_float(h.y << 16);
-    f[3] -= __uint_as_float(h.y & 0xFFFF0000u);
-  }
+  for (int t = 0; t < 3; ++t) out[t * term] = make_uint2(x01[t], x23[t]);
 }
 
 // Deformation offsets of Gaussian g (zero for a static scene): the MLP's
