@@ -65,6 +65,31 @@ def hbm_peak():
         return HBM_FALLBACK_GBS, "fallback"
 
 
+# Kernel launches of the library's calls (tests compare them with a trace).
+def render_launches(P: int, D: int, deform: bool):
+    """(forward, reverse) of one view: projection, depth sort (one launch up
+    to 49,152 Gaussians, else histogram and four passes), counts, table scan,
+    scatter, compositing (128 channels a launch); compositing (64 channels a
+    launch), partial sums, projection; the deformation's sample and MLP and
+    their reverses."""
+    d = 2 if deform else 0
+    return ((1 if P <= 49152 else 5) + 4 + max(1, D // 128) + d, max(1, D // 64) + 2 + d)
+
+
+def dec_launches(D: int) -> int:
+    """Decoder launches of one fused loss call, without the fixed-order sum."""
+    return 2 if D == 128 else 1
+
+
+def batch_launches(P: int, D: int, deform: bool, views: int) -> int:
+    """A batch step: per view everything but the compositing, and two L1
+    losses of two kernels; the compositing of all views; beyond one view the
+    sums of the six gradients over the helper streams."""
+    fwd, bwd = render_launches(P, D, deform)
+    comp = max(1, D // 128) + max(1, D // 64)
+    return views * (fwd + bwd - comp + 4) + comp + (6 if views > 1 else 0)
+
+
 def parse():
     p = argparse.ArgumentParser()
     p.add_argument("--gpus", type=int, default=1)
@@ -587,14 +612,9 @@ def run_ours(args, world, rank, local):
                "d2h_bytes_per_step": int(d2h), "ms_per_step": round(e2e_ms, 4),
                "pipeline": "two buffer sets; uploads and read-backs on two copy streams overlap the compute"}
 
-    # forward: projection, depth sort (histogram and 4 passes, one launch for
-    # few Gaussians), count, table scan, scatter, composite; L1 x2 (2 kernels
-    # each); reverse: composite (a pass per 64 channels), feature sums,
-    # projection chain; the deformation adds its sample and MLP and their
-    # reverses.  (With a decoder, its kernel and fixed-order sum replace the two
-    # feature-L1 kernels.)  Training adds the depth L1 (2 kernels) and the Adam
-    # launch.
-    launches_per_step = ((6 if P <= 49152 else 10) + 4 + 2 + max(1, D // 64) + (4 if deform is not None else 0)
+    # Render forward and reverse, L1 rgb (2), feature L1 (2) or the decoder and
+    # its fixed-order sum, the depth L1 (2) and the Adam launch of training.
+    launches_per_step = (sum(render_launches(P, D, deform is not None)) + 2 + (2 if dec is None else 1 + dec_launches(D))
                          + (1 if opt is not None else 0) + (2 if tgt_depth is not None else 0))
     result = {
         "metric": METRIC, "value": round(world * 1000.0 / ms, 3), "unit": "it/s", "n_gpus": world,
@@ -961,11 +981,10 @@ def run_train_fst(args, world, rank, local, cfg):
         "e2e": {"value": round(world * 1000.0 / e2e_ms, 3), "unit": "it/s", "h2d_bytes_per_step": int(h2d),
                 "d2h_bytes_per_step": 16, "ms_per_step": round(e2e_ms, 4)},
         "device_errors": int(tr.rast.stats()["device_errors"]), "clocks": clk,
-        # per step: FST forward 3 (pack, sample, MLP); render forward 10; L1 rgb
-        # 2, decoder 2, depth L1 2; render reverse 3; FST reverse 5 (pack, MLP,
-        # HexPlane, lines, reduce); TV 2; Adam 2 (Gaussians + decoder, planes +
-        # MLP)
-        "gpu_launches": 31 * K,
+        # per step: FST forward 3 (pack, sample, MLP) and reverse 5 (pack, MLP,
+        # HexPlane, lines, reduce); render; L1 rgb 2, decoder and its sum, depth
+        # L1 2; TV 2; Adam 2 (Gaussians + decoder, planes + MLP)
+        "gpu_launches": (8 + sum(render_launches(P, D, False)) + 2 + 1 + dec_launches(D) + 2 + 2 + 2) * K,
     }
     if rank == 0:
         print(json.dumps(result))
@@ -1087,7 +1106,7 @@ def run_batch(args, world, rank, local, cfg):
         "roofline": {"kernel": "composite_bwd", "bound": "alu", "achieved": round(ach, 3), "peak": round(alu_peak, 2),
                      "unit": "TFLOP/s", "frac": round(ach / alu_peak, 4), "traffic": None,
                      "note": "the batched (persistent) compositing reverse over all views, eager pass"},
-        "device_errors": errs, "gpu_launches": n_views * 16 + 2 * n_views + 2, "clocks": clk, "e2e": None,
+        "device_errors": errs, "gpu_launches": batch_launches(P, D, deform is not None, n_views) * K_steps, "clocks": clk, "e2e": None,
     }
     if rank == 0:
         print(json.dumps(result))
