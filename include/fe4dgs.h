@@ -385,7 +385,10 @@ fe_status fe_fst_workspace_size(int P, int levels, int rs, int rt, int D, int wi
  * opacity_logits [P], feat [P,D] (bf16 if feat_bf16, else float32).
  * Outputs (device, caller-owned, overwritten): the deformed arrays in the
  * same layouts, feat_t in the same type as feat (bf16 outputs rounded to
- * nearest even).  Outputs must not alias inputs.  With with_backward the
+ * nearest even).  Outputs must not alias inputs.  The MLP's products are
+ * three-term BF16 ones on the tensor cores without with_backward and FP32 ones
+ * with it (the reverse repeats the ReLU decisions): equal within float32
+ * rounding, not in every bit.  With with_backward the
  * workspace (fe_fst_workspace_size with with_backward = 1) keeps the state
  * fe_fst_backward needs; it must not be touched in between.  Asynchronous
  * on `stream`. */

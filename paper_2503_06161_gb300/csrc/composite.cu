@@ -33,7 +33,9 @@ namespace {
 // the tiles fit about one such wave, else three (frames at two and three
 // blocks: 30k at 320 x 240, 300 tiles, 98 and 111 us; at 333 x 251, 336 tiles,
 // 102 and 114; at 352 x 288, 396 tiles, 111 and 111; at 384 x 288 117 and 109;
-// at 640 x 512 171 and 160; 100k at 352 x 288 141 and 125).
+// at 640 x 512 171 and 160; 100k at 352 x 288 141 and 125).  At three blocks
+// D = 32 spills 28 bytes (64-entry batches) or 56 (128); two blocks, without
+// spills, are 1% slower (200k at 640 x 512: 350 us for 347).
 constexpr int kSMs = 152;
 template <int D>
 constexpr int fwd_batch() { return D <= 16 ? 128 : (D <= 64 ? 64 : 32); }
@@ -443,7 +445,9 @@ __global__ void __launch_bounds__(kThreads, NB)
 // shared memory for every entry.  Measured, before and now: 200k Gaussians at
 // 640 x 512, D = 32: 365 -> 330 us; 90k, D = 128: 1520 -> 1345 us; 1M at
 // 1280 x 1024, D = 64 BF16: 2135 -> 1811 us; eight views of 100k, D = 32
-// BF16, in one launch: 1960 -> 1528 us.  (tcgen05 products over the whole
+// BF16, in one launch: 1960 -> 1528 us.  At D = 32 the second block per SM costs
+// 56 bytes of spills; one block takes 976 us for the 842 of a whole forward and
+// reverse (200k).  (tcgen05 products over the whole
 // tile were costed: they take every entry of a batch for every pixel where a
 // warp needs half of them, and their operands in three terms leave one block
 // per SM at D = 32 too.)

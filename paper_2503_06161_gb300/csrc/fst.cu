@@ -633,12 +633,13 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
 // order the products read them, staged 32 output columns at a time through
 // three shared-memory buffers (one barrier per stage).
 //
-// Bound by the tensor pipe (200k Gaussians, 4 levels: 75 M products of
-// 16 x 8 x 16, 236 us at the measured 607 TFLOP/s of mma.sync).  The products
-// with FP32 FMAs (fst_fwd_kernel), which training keeps -- the reverse's ReLU
-// masks are decisions that a different rounding would take differently -- are
-// bound by FMA issue at twice that.  Measured: 592 -> 395 us, and the same
-// error against 64 bits (2.5e-7 of the outputs).
+// The products alone need 236 us (200k Gaussians, 4 levels: 35 M products of
+// 16 x 8 x 16 at the measured 607 TFLOP/s of mma.sync); the kernel takes 400,
+// with the tensor pipe 58% busy: two blocks per SM cannot hide all of the
+// fragment loads and splits.  With FP32 FMAs (fst_fwd_kernel), which training keeps --
+// the reverse's ReLU masks are decisions that a different rounding would take
+// differently -- they are bound by FMA issue: 592 us, with the same error against
+// 64 bits (1e-7 of the outputs).
 // ---------------------------------------------------------------------------
 constexpr int kTcWarps = 8, kTcThreads = 32 * kTcWarps, kTcRows = 16 * kTcWarps;
 constexpr int kTcBuf = 4 * 4 * 768;   // bytes of the largest stage: K = 64, 32 columns
@@ -1276,10 +1277,13 @@ constexpr size_t kBwdSmem = 6 * (size_t)kTTerm + kBwdW + 1024;
 // relu(z).  The same term products and accumulators as the forward without
 // reverse state.
 //
-// Bound by the tensor pipe (200k Gaussians, 4 levels: 150 M products of
-// 16 x 8 x 16, 472 us at 607 TFLOP/s) and, under it, by the rounds' barriers
-// and fragment loads.  The FP32 form (8 x 8 register tiles of packed FMAs,
-// 249 registers, 8 warps per SM) took 1555 us.
+// The products alone need 472 us (200k Gaussians, 4 levels: 70 M products of
+// 16 x 8 x 16 at 607 TFLOP/s); the kernel takes 1094, the tensor pipe half
+// busy: the rounds' barriers and fragment loads are the rest.  The FP32 form
+// (8 x 8 register tiles of packed FMAs, 249 registers, 8 warps per SM) took
+// 1555 us.  Two blocks per SM leave 128 registers and 236 (D = 16) to 508
+// (D = 128) bytes of spills; one block without them is slower (module forward +
+// reverse + TV 2625 us for 2435).
 template <int D>
 __global__ void __launch_bounds__(kBwdThreads, 2) fst_bwd_kernel(const __grid_constant__ BwdArgs a) {
   extern __shared__ unsigned char s_raw[];

@@ -429,11 +429,13 @@ __global__ void __launch_bounds__(kThreads, 2) gauss_fwd_kernel(const GaussArgs 
 // Gaussian (1M Gaussians, D = 64: 256 us, now 218 from launch to end,
 // overlapping the kernel before it).
 // Ranks per warp: 8 for rows of at most 64 floats (D <= 52), else 4
-// (measured best at D = 32 and D = 128).
+// (measured best at D = 32 and D = 128).  Four blocks per SM up to D = 128;
+// D = 256 would spill 44 bytes there, and three are faster (50k Gaussians at
+// 640 x 512, forward + reverse: 3861 us for 3910).
 __host__ __device__ constexpr int ranks_per_warp(int D) { return (partial_stride(D) + 31) / 32 <= 2 ? 8 : 4; }
 
 template <int D>
-__global__ void __launch_bounds__(kThreads, 4) partial_reduce_kernel(const GaussBwdArgs b, int P) {
+__global__ void __launch_bounds__(kThreads, D <= 128 ? 4 : 3) partial_reduce_kernel(const GaussBwdArgs b, int P) {
   grid_dep_wait();
   grid_dep_launch();
   constexpr int NP = partial_stride(D);

@@ -4,6 +4,11 @@ branches and the semantic updater F_feat.  Every step runs in the library's
 kernels (fe_fst_forward / fe_fst_backward / fe_fst_tv); this module owns the
 device buffers and marshals the calls.
 
+A module built with_backward=False runs its MLP on the tensor cores (three
+BF16 terms per operand), one with reverse state in FP32 (whose ReLU decisions
+the reverse repeats): the same offsets within float32 rounding, not the same
+bits.
+
 It wraps the renderer: ``forward`` writes the deformed Gaussians G_t
 (Eq. 6) into a GaussianScene that a static render consumes, and
 ``backward`` turns that render's parameter gradients into the gradients of
