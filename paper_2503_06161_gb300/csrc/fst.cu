@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fst_fwd_kernel(const FwdArgs a
 // three shared-memory buffers (one barrier per stage).
 //
 // The products alone need 236 us (200k Gaussians, 4 levels: 35 M products of
-// 16 x 8 x 16 at the measured 607 TFLOP/s of mma.sync); the kernel takes 400,
+// 16 x 8 x 16 at the measured 607 TFLOP/s of mma.sync); the kernel takes 405,
 // with the tensor pipe 58% busy: two blocks per SM cannot hide all of the
 // fragment loads and splits.  With FP32 FMAs (fst_fwd_kernel), which training keeps --
 // the reverse's ReLU masks are decisions that a different rounding would take
